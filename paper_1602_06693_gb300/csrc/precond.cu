@@ -315,56 +315,145 @@ __device__ __forceinline__ void dot2_add(Acc2& a, float x, float y) {
     a.c += pi + sg;
 }
 
-// w_part[s][k][a] = sum_{i in split s} KXU[i][a] R[i][k]; K_XU and R enter as
-// FP32 pairs, products are split exactly and accumulated with Dot2.
-constexpr int PC = 4;  // columns per pass
+// K_UX R over a range of rows.  A CTA of 256 threads takes `aw` columns a of K_XU
+// (aw = 32, 64, 128 or 256: the smallest that covers m, so that a small m
+// leaves no thread idle) with 256 / aw groups of rows, rows g, g + 256/aw, ...
+// each; K_XU and R enter as FP32 pairs, products are split exactly and
+// accumulated with Dot2, the groups' sums are added in FP64 in a fixed order.
+// With few columns the pass is bound by HBM latency times the bytes in
+// flight (kRb loads of K_XU are issued before any is used), with many by
+// the ~13 FP32 issue slots of a Dot2 term; either way it needs CTAs on every
+// SM, so nys_rows_per_split makes the row ranges short (down to 32 rows) when
+// n m is small.  Ranges of 512 rows left 10 CTAs on a 152-SM GPU at n = 5000:
+// 0.50 ms per 17-column apply.
+constexpr int kRb = 8;  // rows (projection) or row chunks (back product) loaded per batch
 template <typename T>
-__global__ void __launch_bounds__(256)
-    nys_proj_kernel(const float2* __restrict__ KXU, int64_t n, int64_t m, const T* __restrict__ R,
-                    int64_t ldr, int ncols, int64_t rows_per_split, double* __restrict__ part,
-                    int c_total) {
-    __shared__ float2 sr[128][PC];  // r split into float hi + lo
-    const int64_t a = (int64_t)blockIdx.x * 256 + threadIdx.x;
-    const int64_t r0 = (int64_t)blockIdx.y * rows_per_split;
-    const int64_t r1 = min(n, r0 + rows_per_split);
-    Acc2 acc[PC];
+struct ProjR;  // R in shared memory: the FP32 value, or the FP64 one as a pair
+template <>
+struct ProjR<float> {
+    using S = float;
+    static __device__ __forceinline__ S cut(float v) { return v; }
+    static __device__ __forceinline__ void add(Acc2& a, float2 kv, S r) {
+        dot2_add(a, kv.x, r);
+        a.c = fmaf(kv.y, r, a.c);
+    }
+};
+template <>
+struct ProjR<double> {
+    using S = float2;
+    static __device__ __forceinline__ S cut(double v) {
+        const float hi = (float)v;
+        return make_float2(hi, (float)(v - (double)hi));
+    }
+    static __device__ __forceinline__ void add(Acc2& a, float2 kv, S r) {
+        dot2_add(a, kv.x, r.x);
+        a.c = fmaf(kv.x, r.y, fmaf(kv.y, r.x, a.c));
+    }
+};
+// shared memory of a projection CTA: the staged rows of R, then the groups' sums
+template <typename T, int NC>
+constexpr int proj_smem() {
+    const int a = 128 * NC * (int)sizeof(typename ProjR<T>::S), b = 256 * NC * 8;
+    return a > b ? a : b;
+}
+
+// out[k * m + a] = sum_{r0 <= i < r1} KXU[i][a] R[i][k], k < ncols <= NC, for the
+// aw columns a of block `ablk`
+template <typename T, int NC>
+__device__ __forceinline__ void nys_proj_body(const float2* __restrict__ KXU, int64_t m, int aw,
+                                              int64_t ablk, const T* __restrict__ R, int64_t ldr,
+                                              int ncols, int64_t r0, int64_t r1,
+                                              double* __restrict__ out, uint8_t* smem) {
+    using PR = ProjR<T>;
+    typename PR::S* sr = reinterpret_cast<typename PR::S*>(smem);  // [128][NC]
+    double* red = reinterpret_cast<double*>(smem);                 // [NC][256], after the rows
+    const int ax = threadIdx.x & (aw - 1), g = threadIdx.x / aw, ng = 256 / aw;
+    const int64_t a = ablk * aw + ax;
+    Acc2 acc[NC];
 #pragma unroll
-    for (int k = 0; k < PC; ++k) acc[k] = {0.f, 0.f};
+    for (int k = 0; k < NC; ++k) acc[k] = {0.f, 0.f};
     for (int64_t rs = r0; rs < r1; rs += 128) {
+        const int rn = (int)min((int64_t)128, r1 - rs);
         __syncthreads();
-        for (int e = threadIdx.x; e < 128 * PC; e += 256) {
-            const int k = e / 128, r = e % 128;
-            double v = (rs + r < r1 && k < ncols) ? (double)R[rs + r + (int64_t)k * ldr] : 0.0;
-            const float hi = (float)v;
-            sr[r][k] = make_float2(hi, (float)(v - (double)hi));
+        for (int k = threadIdx.x >> 7; k < NC; k += 2) {
+            const int r = threadIdx.x & 127;
+            if (r < rn) sr[r * NC + k] = PR::cut(k < ncols ? R[rs + r + (int64_t)k * ldr] : T(0));
         }
         __syncthreads();
-        const int rn = (int)min((int64_t)128, r1 - rs);
         if (a < m) {
             const float2* Kp = KXU + rs * m + a;
-#pragma unroll 4
-            for (int r = 0; r < rn; ++r) {
+            int r = g;
+            for (; r + (kRb - 1) * ng < rn; r += kRb * ng) {
+                float2 kv[kRb];
+#pragma unroll
+                for (int u = 0; u < kRb; ++u) kv[u] = __ldg(Kp + (int64_t)(r + u * ng) * m);
+#pragma unroll
+                for (int u = 0; u < kRb; ++u)
+#pragma unroll
+                    for (int k = 0; k < NC; ++k)
+                        if (k < ncols) PR::add(acc[k], kv[u], sr[(r + u * ng) * NC + k]);
+            }
+            for (; r < rn; r += ng) {
                 const float2 kv = __ldg(Kp + (int64_t)r * m);
 #pragma unroll
-                for (int k = 0; k < PC; ++k) {
-                    dot2_add(acc[k], kv.x, sr[r][k].x);
-                    acc[k].c = fmaf(kv.x, sr[r][k].y, fmaf(kv.y, sr[r][k].x, acc[k].c));
-                }
+                for (int k = 0; k < NC; ++k)
+                    if (k < ncols) PR::add(acc[k], kv, sr[r * NC + k]);
             }
         }
     }
-    if (a < m)
-        for (int k = 0; k < ncols; ++k)
-            part[((int64_t)blockIdx.y * c_total + k) * m + a] = (double)acc[k].s + (double)acc[k].c;
+    if (ng == 1) {
+        if (a < m)
+#pragma unroll
+            for (int k = 0; k < NC; ++k)
+                if (k < ncols) out[(int64_t)k * m + a] = (double)acc[k].s + (double)acc[k].c;
+        return;
+    }
+    __syncthreads();
+#pragma unroll
+    for (int k = 0; k < NC; ++k)
+        if (k < ncols) red[k * 256 + threadIdx.x] = (double)acc[k].s + (double)acc[k].c;
+    __syncthreads();
+    for (int k = g; k < ncols; k += ng) {
+        double s = 0.0;
+        for (int q = 0; q < ng; ++q) s += red[k * 256 + q * aw + ax];
+        if (a < m) out[(int64_t)k * m + a] = s;
+    }
 }
 
+// The smallest column group of a projection CTA that covers m.
+__host__ __device__ inline int proj_aw(int64_t m) { return m <= 32 ? 32 : m <= 64 ? 64 : m <= 128 ? 128 : 256; }
+
+// Rows per CTA of the projection: eight CTAs per SM over the whole call (`work` =
+// sum over problems of column blocks x rows), between 32 and 512 rows.
+int64_t nys_rows_per_split(int64_t work) {
+    const int64_t r = (work / (152 * 8) + 31) / 32 * 32;
+    return std::max<int64_t>(32, std::min<int64_t>(512, r));
+}
+
+// w_part[s][k][a] = sum_{i in split s} KXU[i][a] R[i][k] for one problem.
+template <typename T, int NC>
+__global__ void __launch_bounds__(256)
+    nys_proj_kernel(const float2* __restrict__ KXU, int64_t n, int64_t m, int aw,
+                    const T* __restrict__ R, int64_t ldr, int ncols, int64_t rows_per_split,
+                    double* __restrict__ part, int c_total) {
+    __shared__ __align__(16) uint8_t smem[proj_smem<T, NC>()];
+    const int64_t r0 = (int64_t)blockIdx.y * rows_per_split;
+    const int64_t r1 = min(n, r0 + rows_per_split);
+    nys_proj_body<T, NC>(KXU, m, aw, blockIdx.x, R, ldr, ncols, r0, r1,
+                         part + (int64_t)blockIdx.y * c_total * m, smem);
+}
+
+// out = sum of the split partials, a warp per entry: lanes stride over the splits,
+// then a fixed-order warp sum.
 __global__ void sum_splits_kernel(const double* __restrict__ part, int nsplit, int64_t len,
                                   double* __restrict__ out) {
-    const int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    const int lane = threadIdx.x & 31;
+    const int64_t e = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
     if (e >= len) return;
     double s = 0.0;
-    for (int sp = 0; sp < nsplit; ++sp) s += part[(int64_t)sp * len + e];
-    out[e] = s;
+    for (int sp = lane; sp < nsplit; sp += 32) s += part[(int64_t)sp * len + e];
+    s = warp_sum(s);
+    if (lane == 0) out[e] = s;
 }
 
 // y_k = L^{-1} w_k with U = L^{-T} row-major: y_i = sum_{j <= i} U[j][i] w_j.
@@ -410,7 +499,12 @@ __global__ void tri_upper_apply_kernel(const double* __restrict__ U, int64_t m,
 // components up to ~1e6 that cancel to O(1) in K_XU u; a compensated-FP32 sum
 // (2^-48) left ~3e-6 relative noise there and weakened the preconditioner,
 // FP64 (2^-53) matches the direct solve.
-template <typename T>
+// All columns of a group of NC share one read and one FP64 conversion of an
+// entry (two conversions and an add cost as much of the FP64 pipe, ~2
+// operations per clock and SM, as three products: done per column they were
+// three quarters of the work), and the NC sums are reduced over the lanes by a
+// butterfly that halves the columns a lane holds at each step.
+template <typename T, int NC>
 __global__ void __launch_bounds__(256)
     nys_back_kernel(const float2* __restrict__ KXU, int64_t n, int64_t m,
                     const double* __restrict__ u, int c, const T* __restrict__ R, int64_t ldr,
@@ -422,16 +516,37 @@ __global__ void __launch_bounds__(256)
     const int64_t warps = (int64_t)gridDim.x * (blockDim.x >> 5);
     for (int64_t i = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5; i < n; i += warps) {
         const float2* Ki = KXU + i * m;
-        for (int k = 0; k < c; ++k) {
-            const double* uk = su + (int64_t)k * m;
-            double acc = 0.0;
+        for (int k0 = 0; k0 < c; k0 += NC) {
+            const int nc = min(NC, c - k0);
+            const double* uk = su + (int64_t)k0 * m;
+            double acc[NC];
+#pragma unroll
+            for (int k = 0; k < NC; ++k) acc[k] = 0.0;
+#pragma unroll 4
             for (int64_t a = lane; a < m; a += 32) {
                 const float2 kv = __ldg(Ki + a);
-                acc = fma((double)kv.x + (double)kv.y, uk[a], acc);
+                const double kd = (double)kv.x + (double)kv.y;
+#pragma unroll
+                for (int k = 0; k < NC; ++k)
+                    if (k < nc) acc[k] = fma(kd, uk[(int64_t)k * m + a], acc[k]);
             }
-            const double sm = warp_sum(acc);
-            if (lane == 0)
-                Z[i + (int64_t)k * ldz] = (T)(((double)R[i + (int64_t)k * ldr] - sm) * inv_noise);
+#pragma unroll
+            for (int w = NC, o = 16; w > 1; w >>= 1, o >>= 1) {
+                const bool up_half = (lane & o) != 0;
+#pragma unroll
+                for (int q = 0; q < w / 2; ++q) {
+                    const double give = up_half ? acc[q] : acc[q + w / 2];
+                    const double keep = up_half ? acc[q + w / 2] : acc[q];
+                    acc[q] = keep + __shfl_xor_sync(0xffffffffu, give, o);
+                }
+            }
+#pragma unroll
+            for (int o = 16 / NC; o > 0; o >>= 1)
+                acc[0] += __shfl_xor_sync(0xffffffffu, acc[0], o);
+            const int k = lane / (32 / NC);
+            if ((lane & (32 / NC - 1)) == 0 && k < nc)
+                Z[i + (int64_t)(k0 + k) * ldz] =
+                    (T)(((double)R[i + (int64_t)(k0 + k) * ldr] - acc[0]) * inv_noise);
         }
     }
 }
@@ -936,27 +1051,50 @@ void block_jacobi_setup(PrecondState& P, const double* xs64, int64_t n, int dp, 
     P.ready = true;
 }
 
+// Columns per pass of a block of c, in ceil(c / 16) passes of nearly equal width.
+static int pass_cols(int c) { return (c + (c + 15) / 16 - 1) / ((c + 15) / 16); }
+
+// w (returned, column-major, ld m) = K_UX R in FP64: the split partials of the
+// projection, added in a fixed order.
+template <typename T>
+static double* nystrom_project(const PrecondState& P, const T* R, int64_t ldr, int c,
+                               cudaStream_t st) {
+    const int64_t n = P.n, m = P.m;
+    const int aw = proj_aw(m);
+    const int64_t ablk = (m + aw - 1) / aw;
+    const int64_t rps = nys_rows_per_split(ablk * n);
+    const int nsplit = (int)((n + rps - 1) / rps);
+    double* part = const_cast<PrecondState&>(P).wpart.need((size_t)nsplit * c * m);
+    double* w = const_cast<PrecondState&>(P).w.need((size_t)c * m);
+    const int step = pass_cols(c);
+    for (int k0 = 0; k0 < c; k0 += step) {
+        const int nc = std::min(step, c - k0);
+        const dim3 g((unsigned)ablk, (unsigned)nsplit);
+        auto go = [&](auto kern) {
+            kern<<<g, 256, 0, st>>>(P.KXU.p, n, m, aw, R + (int64_t)k0 * ldr, ldr, nc, rps,
+                                    part + (int64_t)k0 * m, c);
+        };
+        if (nc <= 1)
+            go(nys_proj_kernel<T, 1>);
+        else if (nc <= 4)
+            go(nys_proj_kernel<T, 4>);
+        else if (nc <= 9)
+            go(nys_proj_kernel<T, 9>);
+        else
+            go(nys_proj_kernel<T, 16>);
+        KPCG_LAUNCHED("nys_proj_kernel");
+    }
+    sum_splits_kernel<<<(unsigned)((c * m + 7) / 8), 256, 0, st>>>(part, nsplit, c * m, w);
+    KPCG_LAUNCHED("sum_splits_kernel");
+    return w;
+}
+
 template <typename T>
 static void nystrom_apply(const PrecondState& P, const T* R, int64_t ldr, int c, T* Z,
                           int64_t ldz, cudaStream_t st) {
     const int64_t n = P.n, m = P.m;
-    const int64_t ablk = (m + 255) / 256;
-    int nsplit = (int)std::max<int64_t>(1, std::min<int64_t>((152 * 4 + ablk - 1) / ablk,
-                                                             (n + 127) / 128));
-    const int64_t rps = (n + nsplit - 1) / nsplit;
-    nsplit = (int)((n + rps - 1) / rps);
-    double* part = const_cast<PrecondState&>(P).wpart.need((size_t)nsplit * c * m);
-    double* w = const_cast<PrecondState&>(P).w.need((size_t)c * m);
+    double* w = nystrom_project<T>(P, R, ldr, c, st);
     double* y = const_cast<PrecondState&>(P).y.need((size_t)c * m);
-    for (int k0 = 0; k0 < c; k0 += PC) {
-        const int nc = std::min(PC, c - k0);
-        dim3 g((unsigned)((m + 255) / 256), (unsigned)nsplit);
-        nys_proj_kernel<T><<<g, 256, 0, st>>>(P.KXU.p, n, m, R + (int64_t)k0 * ldr, ldr, nc, rps,
-                                              part + (int64_t)k0 * m, c);
-        KPCG_LAUNCHED("nys_proj_kernel");
-    }
-    sum_splits_kernel<<<(unsigned)((c * m + 255) / 256), 256, 0, st>>>(part, nsplit, c * m, w);
-    KPCG_LAUNCHED("sum_splits_kernel");
     tri_lower_apply_kernel<<<dim3((unsigned)((m + 31) / 32), c), 1024, 0, st>>>(P.U.p, m, w, y);
     KPCG_LAUNCHED("tri_lower_apply_kernel");
     tri_upper_apply_kernel<<<dim3((unsigned)((m * 32 + 255) / 256), c), 256, 0, st>>>(P.U.p, m, y,
@@ -964,34 +1102,28 @@ static void nystrom_apply(const PrecondState& P, const T* R, int64_t ldr, int c,
     KPCG_LAUNCHED("tri_upper_apply_kernel");
     const size_t smem = sizeof(double) * (size_t)m * c;
     if (smem > 200 * 1024) fail(KPCG_ERR_ARG, "Nystrom apply: m * c too large");
-    if (smem > 48 * 1024) raise_smem_limit((const void*)nys_back_kernel<T>, smem);
-    int blocks = (int)std::min<int64_t>((n + 7) / 8, 152 * 16);
-    nys_back_kernel<T><<<blocks, 256, smem, st>>>(P.KXU.p, n, m, w, c, R, ldr, Z, ldz,
-                                                  1.0 / P.apply_noise);
+    const int blocks = (int)std::min<int64_t>((n + 7) / 8, 152 * 16);
+    auto go = [&](auto kern) {
+        if (smem > 48 * 1024) raise_smem_limit((const void*)kern, smem);
+        kern<<<blocks, 256, smem, st>>>(P.KXU.p, n, m, w, c, R, ldr, Z, ldz, 1.0 / P.apply_noise);
+    };
+    if (c == 1)
+        go(nys_back_kernel<T, 1>);
+    else if (c <= 4)
+        go(nys_back_kernel<T, 4>);
+    else if (c <= 8)
+        go(nys_back_kernel<T, 8>);
+    else
+        go(nys_back_kernel<T, 16>);
     KPCG_LAUNCHED("nys_back_kernel");
 }
 
 // u = M^{-1} K_UX r for c columns (FP64 in and out, column-major, ld m for u).
 void nystrom_project_solve(const PrecondState& P, const double* R, int64_t ldr, int c, double* u,
                            cudaStream_t st) {
-    const int64_t n = P.n, m = P.m;
-    const int64_t ablk = (m + 255) / 256;
-    int nsplit = (int)std::max<int64_t>(1, std::min<int64_t>((152 * 4 + ablk - 1) / ablk,
-                                                             (n + 127) / 128));
-    const int64_t rps = (n + nsplit - 1) / nsplit;
-    nsplit = (int)((n + rps - 1) / rps);
-    double* part = const_cast<PrecondState&>(P).wpart.need((size_t)nsplit * c * m);
-    double* w = const_cast<PrecondState&>(P).w.need((size_t)c * m);
+    const int64_t m = P.m;
+    double* w = nystrom_project<double>(P, R, ldr, c, st);
     double* y = const_cast<PrecondState&>(P).y.need((size_t)c * m);
-    for (int k0 = 0; k0 < c; k0 += PC) {
-        const int nc = std::min(PC, c - k0);
-        dim3 g((unsigned)((m + 255) / 256), (unsigned)nsplit);
-        nys_proj_kernel<double><<<g, 256, 0, st>>>(P.KXU.p, n, m, R + (int64_t)k0 * ldr, ldr, nc,
-                                                   rps, part + (int64_t)k0 * m, c);
-        KPCG_LAUNCHED("nys_proj_kernel");
-    }
-    sum_splits_kernel<<<(unsigned)((c * m + 255) / 256), 256, 0, st>>>(part, nsplit, c * m, w);
-    KPCG_LAUNCHED("sum_splits_kernel");
     tri_lower_apply_kernel<<<dim3((unsigned)((m + 31) / 32), c), 1024, 0, st>>>(P.U.p, m, w, y);
     KPCG_LAUNCHED("tri_lower_apply_kernel");
     tri_upper_apply_kernel<<<dim3((unsigned)((m * 32 + 255) / 256), c), 256, 0, st>>>(P.U.p, m, y,
@@ -1158,8 +1290,6 @@ void precond_apply_f32(const PrecondState& P, const float* R, int64_t ldr, int c
 // return at once.
 namespace {
 
-constexpr int kSplitRows = 512;
-constexpr int kRb = 8;  // rows (projection) or row chunks (back product) loaded per batch
 
 __device__ __forceinline__ bool nb_live(const int* __restrict__ active, int p, int c) {
     if (!active) return true;
@@ -1174,65 +1304,17 @@ __global__ void __launch_bounds__(256)
     nys_batch_proj_kernel(const NysBatchProb* __restrict__ probs, int c, const float* __restrict__ R,
                           int64_t ldr, int k0, int ncols, const int* __restrict__ active,
                           double* __restrict__ part) {
-    __shared__ float sr[128][NC];
+    __shared__ __align__(16) uint8_t smem[proj_smem<float, NC>()];
     const int p = blockIdx.z;
     const NysBatchProb pb = probs[p];
-    if (pb.m == 0 || (int)blockIdx.y >= pb.nsplit || (int64_t)blockIdx.x * 256 >= pb.m ||
+    const int aw = proj_aw(pb.m);
+    if (pb.m == 0 || (int)blockIdx.y >= pb.nsplit || (int64_t)blockIdx.x * aw >= pb.m ||
         !nb_live(active, p, c))
         return;
-    const int64_t m = pb.m;
-    const int64_t a = (int64_t)blockIdx.x * 256 + threadIdx.x;
     const int64_t r0 = (int64_t)blockIdx.y * pb.rows_per_split;
     const int64_t r1 = min(pb.n, r0 + pb.rows_per_split);
-    const float* Rp = R + ((int64_t)p * c + k0) * ldr;
-    Acc2 acc[NC];
-#pragma unroll
-    for (int k = 0; k < NC; ++k) acc[k] = {0.f, 0.f};
-    for (int64_t rs = r0; rs < r1; rs += 128) {
-        __syncthreads();
-        for (int e = threadIdx.x; e < 128 * NC; e += 256) {
-            const int k = e / 128, r = e % 128;
-            sr[r][k] = (rs + r < r1 && k < ncols) ? Rp[rs + r + (int64_t)k * ldr] : 0.f;
-        }
-        __syncthreads();
-        const int rn = (int)min((int64_t)128, r1 - rs);
-        if (a < m) {
-            const float2* Kp = pb.KXU + rs * m + a;
-            // batches of kRb rows: their loads are issued before any is used, so
-            // each thread keeps kRb * 8 bytes of K_XU in flight (the pass is
-            // bound by HBM latency times the bytes in flight, not by the Dot2)
-            int r = 0;
-            for (; r + kRb <= rn; r += kRb) {
-                float2 kv[kRb];
-#pragma unroll
-                for (int u = 0; u < kRb; ++u) kv[u] = __ldg(Kp + (int64_t)(r + u) * m);
-#pragma unroll
-                for (int u = 0; u < kRb; ++u)
-#pragma unroll
-                    for (int k = 0; k < NC; ++k)
-                        if (k < ncols) {
-                            dot2_add(acc[k], kv[u].x, sr[r + u][k]);
-                            acc[k].c = fmaf(kv[u].y, sr[r + u][k], acc[k].c);
-                        }
-            }
-            for (; r < rn; ++r) {
-                const float2 kv = __ldg(Kp + (int64_t)r * m);
-#pragma unroll
-                for (int k = 0; k < NC; ++k)
-                    if (k < ncols) {
-                        dot2_add(acc[k], kv.x, sr[r][k]);
-                        acc[k].c = fmaf(kv.y, sr[r][k], acc[k].c);
-                    }
-            }
-        }
-    }
-    if (a < m) {
-#pragma unroll
-        for (int k = 0; k < NC; ++k)
-            if (k < ncols)
-                part[pb.pbase + ((int64_t)blockIdx.y * c + k0 + k) * m + a] =
-                    (double)acc[k].s + (double)acc[k].c;
-    }
+    nys_proj_body<float, NC>(pb.KXU, pb.m, aw, blockIdx.x, R + ((int64_t)p * c + k0) * ldr, ldr, ncols,
+                             r0, r1, part + pb.pbase + ((int64_t)blockIdx.y * c + k0) * pb.m, smem);
 }
 
 // w = sum of the split partials: a warp per entry (lanes stride over the
@@ -1312,6 +1394,16 @@ __global__ void nys_batch_upper_kernel(const NysBatchProb* __restrict__ probs, i
     }
 }
 
+// a + (the partner's b across lane bit o), high parts by TwoSum
+__device__ __forceinline__ Acc2 acc2_xor(Acc2 a, Acc2 b, int o) {
+    const float os = __shfl_xor_sync(0xffffffffu, b.s, o);
+    const float oc = __shfl_xor_sync(0xffffffffu, b.c, o);
+    const float t = a.s + os;
+    const float z = t - a.s;
+    const float e = (a.s - (t - z)) + (os - z);
+    return {t, a.c + oc + e};
+}
+
 // z = (r - K_XU u) / sigma^2 (warp per row, all columns k0 .. k0+ncols-1 of
 // the problem in one sweep over the row of K_XU), zero past n_p; m = 0 means
 // no preconditioner (z = r).  Problems with no active column are left as they
@@ -1353,9 +1445,10 @@ __global__ void __launch_bounds__(256)
             continue;
         }
         const float2* Ki = pb.KXU + i * pb.m;
-        Acc2 acc[NC];
+        constexpr int NCP = NC <= 1 ? 1 : NC <= 4 ? 4 : NC <= 8 ? 8 : 16;  // a power of two
+        Acc2 acc[NCP];
 #pragma unroll
-        for (int k = 0; k < NC; ++k) acc[k] = {0.f, 0.f};
+        for (int k = 0; k < NCP; ++k) acc[k] = {0.f, 0.f};
         // the row in batches of kRb chunks of 32 entries, all loads of a batch
         // issued before any is used (bytes in flight, as in the projection)
         for (int64_t a0 = lane; a0 < pb.m; a0 += 32 * kRb) {
@@ -1378,31 +1471,33 @@ __global__ void __launch_bounds__(256)
                     }
             }
         }
-        // warp sum of the pairs with TwoSum on every step (FP64 adds would
-        // hold the FP64 pipe, ~1/64 rate, longer than the whole sweep above)
+        // sum over the lanes with TwoSum on every step (FP64 adds would hold the
+        // FP64 pipe, ~1/64 rate, longer than the whole sweep above).  While a
+        // lane holds w > 1 columns it hands half of them to its partner across
+        // the next lane bit and adds the partner's copy of the other half:
+        // NC - 1 + log2(32 / NC) exchanges instead of 5 NC, after which lane l
+        // holds the sum of column l >> log2(32 / NCP).
 #pragma unroll
-        for (int k = 0; k < NC; ++k) {
-            if (k < ncols) {
-                float hs = acc[k].s, hc = acc[k].c;
+        for (int w = NCP, o = 16; w > 1; w >>= 1, o >>= 1) {
+            const bool up_half = (lane & o) != 0;
 #pragma unroll
-                for (int o = 16; o > 0; o >>= 1) {
-                    const float os = __shfl_xor_sync(0xffffffffu, hs, o);
-                    const float oc = __shfl_xor_sync(0xffffffffu, hc, o);
-                    const float t = hs + os;
-                    const float z = t - hs;
-                    const float e = (hs - (t - z)) + (os - z);
-                    hs = t;
-                    hc = hc + oc + e;
-                }
-                if (lane == 0) {
-                    // z = (r - (hs + hc)) / sigma^2: r - hs by TwoSum, then the tails
-                    const float r = Rp[i + (int64_t)k * ldr];
-                    const float d = r - hs;
-                    const float bv = d - r;
-                    const float de = (r - (d - bv)) + (-hs - bv);
-                    Zp[i + (int64_t)k * ldz] = (d + (de - hc)) * pb.inv_noise_f;
-                }
+            for (int q = 0; q < w / 2; ++q) {
+                Acc2 keep = up_half ? acc[q + w / 2] : acc[q];
+                const Acc2 give = up_half ? acc[q] : acc[q + w / 2];
+                acc[q] = acc2_xor(keep, give, o);
             }
+        }
+#pragma unroll
+        for (int o = 16 / NCP; o > 0; o >>= 1) acc[0] = acc2_xor(acc[0], acc[0], o);
+        const int k = lane / (32 / NCP);
+        if ((lane & (32 / NCP - 1)) == 0 && k < ncols) {
+            // z = (r - (hs + hc)) / sigma^2: r - hs by TwoSum, then the tails
+            const float hs = acc[0].s, hc = acc[0].c;
+            const float r = Rp[i + (int64_t)k * ldr];
+            const float d = r - hs;
+            const float bv = d - r;
+            const float de = (r - (d - bv)) + (-hs - bv);
+            Zp[i + (int64_t)k * ldz] = (d + (de - hc)) * pb.inv_noise_f;
         }
     }
 }
@@ -1419,19 +1514,25 @@ void nys_batch_plan(NysBatch& nb, const std::vector<const PrecondState*>& Ps, in
     nb.wtotal = 0;
     nb.ptotal = 0;
     nb.nsplit_max = 1;
+    auto uses = [](const PrecondState& P) {
+        return P.ready && (P.kind == KPCG_PREC_NYSTROM || P.kind == KPCG_PREC_SPECTRAL);
+    };
+    int64_t work = 0;
+    for (const PrecondState* P : Ps)
+        if (uses(*P)) work += (P->m + proj_aw(P->m) - 1) / proj_aw(P->m) * P->n;
+    const int64_t rps = nys_rows_per_split(work);
     for (int p = 0; p < nb.P; ++p) {
         const PrecondState& P = *Ps[(size_t)p];
         NysBatchProb& q = nb.hprobs[(size_t)p];
         q.n = P.n;
-        const bool on =
-            P.ready && (P.kind == KPCG_PREC_NYSTROM || P.kind == KPCG_PREC_SPECTRAL);
+        const bool on = uses(P);
         q.m = on ? P.m : 0;
         q.KXU = on ? P.KXU.p : nullptr;
         q.U = on ? P.U.p : nullptr;
         q.inv_noise = on ? 1.0 / P.apply_noise : 1.0;
         q.inv_noise_f = (float)q.inv_noise;
-        q.rows_per_split = kSplitRows;
-        q.nsplit = (int32_t)std::max<int64_t>(1, (P.n + kSplitRows - 1) / kSplitRows);
+        q.rows_per_split = (int32_t)rps;
+        q.nsplit = (int32_t)std::max<int64_t>(1, (P.n + rps - 1) / rps);
         q.wbase = nb.wtotal;
         q.pbase = nb.ptotal;
         nb.wtotal += (int64_t)c * q.m;
@@ -1471,12 +1572,16 @@ void nys_batch_apply(NysBatch& nb, const float* R, int64_t ldr, float* Z, int64_
                      int64_t nrows, const int* active, cudaStream_t st) {
     if (nb.P == 0) return;
     const int c = nb.c;
+    const int step = pass_cols(c);
     if (nb.mmax > 0) {
         const unsigned ablk = (unsigned)((nb.mmax + 255) / 256);
         const dim3 g(ablk, (unsigned)nb.nsplit_max, (unsigned)nb.P);
-        for (int k0 = 0; k0 < c; k0 += 16) {
-            const int nc = std::min(16, c - k0);
-            if (nc <= 4)
+        for (int k0 = 0; k0 < c; k0 += step) {
+            const int nc = std::min(step, c - k0);
+            if (nc <= 1)
+                nys_batch_proj_kernel<1><<<g, 256, 0, st>>>(nb.probs.p, c, R, ldr, k0, nc, active,
+                                                           nb.part.p);
+            else if (nc <= 4)
                 nys_batch_proj_kernel<4><<<g, 256, 0, st>>>(nb.probs.p, c, R, ldr, k0, nc, active,
                                                            nb.part.p);
             else if (nc <= 8)
@@ -1505,8 +1610,8 @@ void nys_batch_apply(NysBatch& nb, const float* R, int64_t ldr, float* Z, int64_
     // rows per problem: at least ~16 warps per SM over the whole batch
     const unsigned blocks =
         (unsigned)std::min<int64_t>((nrows + 7) / 8, std::max(256, 152 * 16 / std::max(1, nb.P)));
-    for (int k0 = 0; k0 < c; k0 += 16) {
-        const int nc = std::min(16, c - k0);
+    for (int k0 = 0; k0 < c; k0 += step) {
+        const int nc = std::min(step, c - k0);
         const dim3 g(blocks, (unsigned)nb.P);
         const size_t smem = sizeof(float2) * (size_t)nc * (size_t)nb.mmax;
         const bool stage = smem <= 200 * 1024;
@@ -1515,7 +1620,9 @@ void nys_batch_apply(NysBatch& nb, const float* R, int64_t ldr, float* Z, int64_
             kern<<<g, 256, stage ? smem : 0, st>>>(nb.probs.p, c, k0, nc, active, nb.u2.p, R, ldr,
                                                    Z, ldz, nrows);
         };
-        if (nc <= 4)
+        if (nc <= 1)
+            stage ? go(nys_batch_back_kernel<1, true>) : go(nys_batch_back_kernel<1, false>);
+        else if (nc <= 4)
             stage ? go(nys_batch_back_kernel<4, true>) : go(nys_batch_back_kernel<4, false>);
         else if (nc <= 8)
             stage ? go(nys_batch_back_kernel<8, true>) : go(nys_batch_back_kernel<8, false>);
