@@ -68,7 +68,8 @@ typedef enum {
 } kpcg_precond_kind;
 
 typedef enum {
-    KPCG_FP64 = 0,     /* FP64 entries, vectors and scalars throughout           */
+    KPCG_FP64 = 0,     /* FP64 vectors and scalars, products of FP64 accuracy
+                          (kpcg_matvec_f64, impl 0)                              */
     KPCG_FP32 = 1,     /* plain FP32 PCG: FP32 entries (direct differences),
                           FP32 vectors; no refinement                            */
     KPCG_FP32_IR = 2,  /* mixed: outer flexible CG (Notay) in FP64 whose
@@ -228,18 +229,24 @@ kpcg_status kpcg_precond_spectral(kpcg_t h, int64_t m, const double* omega);
 kpcg_status kpcg_precond_pitc(kpcg_t h, int64_t m, const int64_t* idx, int64_t b);
 
 /* O = (K + sigma^2 I) V for c columns (device float64, column-major), the
- * matrix-free product of Sec. 2.1.  impl 0: entries and sums in native FP64;
+ * matrix-free product of Sec. 2.1.  impl 0: FP64 accuracy, the product of KPCG_FP64
+ * and of the certified residuals: for d <= 16 and scaled inputs |x'| within ~8 in
+ * fixed point on the tensor cores (exact level sums of 10-bit slices of x',
+ * 56-bit entries and digits of V, sums without rounding; errors at or below
+ * those of FP64 sums), else entries and sums in native FP64;
  * impl 1: the double-float product of KPCG_DF64 and of the outer loop of the
  * mixed modes (FP32-pair arithmetic, about 44 bits per entry, sums carried as
- * FP32 pairs and added in FP64); for d <= 10 its squared distances come from
- * exact integer level sums of 8-bit slices of x' on the tensor cores, each
- * pair of points evaluated once for both triangles of K (n > 128), for
- * larger d from exact grid differences on the FP32 pipe;
+ * FP32 pairs and added in FP64), or the fixed-point product where that is the
+ * faster one (three and more columns, d > 10, few rows); in double-float for
+ * d <= 10 the squared distances come from exact integer level sums of 8-bit
+ * slices of x' on the tensor cores, each pair of points evaluated once for
+ * both triangles of K (n > 128), for larger d from exact grid differences on
+ * the FP32 pipe;
  * impl 2: the sliced tensor-core kernel of KPCG_TCX_IR with V as FP32 pairs
  * (entries to FP32 accuracy, compensated sums, FP64 out; d <= 10);
- * impl 3: impl 1 with the FP32-pipe distances at every d;
- * impl 4: impl 1 evaluating every entry of K (no use of its symmetry;
- * d <= 10). */
+ * impl 3: double-float with the FP32-pipe distances at every d;
+ * impl 4: double-float with tensor-core distances, evaluating every entry of K
+ * (no use of its symmetry; d <= 10). */
 kpcg_status kpcg_matvec_f64(kpcg_t h, const double* V, int64_t ldv, int32_t c, double* O,
                             int64_t ldo, int32_t impl);
 

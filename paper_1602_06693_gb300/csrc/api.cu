@@ -260,16 +260,11 @@ static void residual_f64(Ctx& h, const double* B, int64_t ldb, int c, const doub
                          double* R, std::vector<double>& rr, std::vector<double>& bb,
                          bool double_float = false) {
     cudaStream_t st = h.stream;
-    // symmetric tile pairs halve the FP64 exp work but take at most two
-    // columns per pass; from three columns on, one non-symmetric pass over up
-    // to 16 columns computes each entry's exp fewer times.  double_float: the
-    // double-float product instead (a residual that only steers the iteration)
+    // double_float: the double-float product instead (a residual that only
+    // steers the iteration)
     h.prof.time(Profiler::RESID, st, [&] {
         if (double_float)
             kv_df(h, X, ldx, c, B, ldb, R, h.ld, h.noise);
-        else if (c >= 3 && h.dp <= 16)
-            kv_f64(h.xs64.p, h.n, h.dp, h.c0_64(), h.noise, X, ldx, c, B, ldb, R, h.ld, h.kvws,
-                   st);
         else
             kv_f64_sym(h, X, ldx, c, B, ldb, R, h.ld, h.noise);
     });
@@ -664,9 +659,6 @@ kpcg_status solve_impl(Ctx& h, const double* B, int64_t ldb, int c, double tol,
                         h.prof.time(Profiler::KV_INNER, st, [&] {
                             if (dfk)
                                 kv_df(h, V, ldv, cc, nullptr, 0, O, ldo, h.noise);
-                            else if (cc >= 3 && h.dp <= 16)  // one pass over <= 16 columns
-                                kv_f64(h.xs64.p, h.n, h.dp, h.c0_64(), h.noise, V, ldv, cc,
-                                       nullptr, 0, O, ldo, h.kvws, h.stream);
                             else
                                 kv_f64_sym(h, V, ldv, cc, nullptr, 0, O, ldo, h.noise);
                         });
@@ -746,6 +738,7 @@ kpcg_status solve_impl(Ctx& h, const double* B, int64_t ldb, int c, double tol,
                            steps, rr, bb);
         rr_current = (status == KPCG_OK);  // converged exits certify on a recomputed residual
     }
+    if (kv_tc_error(h)) fail(KPCG_ERR_TIMEOUT, "a bounded wait in the tensor-core K.V expired");
     // FP64 residual of what is returned (the single-precision FP32 solver
     // checked its own operator only)
     double maxrel = 0.0;
@@ -1133,9 +1126,11 @@ kpcg_status kpcg_matvec_f64(kpcg_t h, const double* V, int64_t ldv, int32_t c, d
         if (c == 0) return KPCG_OK;
         kpcg::check_dev_ptr(V, "V");
         kpcg::check_dev_ptr(O, "O");
-        if (impl == 0)
+        if (impl == 0) {
             kpcg::kv_f64_sym(*h, V, ldv, c, nullptr, 0, O, ldo, h->noise);
-        else if (impl == 1) {
+            if (kpcg::kv_tc_error(*h))
+                fail(KPCG_ERR_TIMEOUT, "a bounded wait in the tensor-core K.V expired");
+        } else if (impl == 1) {
             kpcg::kv_df(*h, V, ldv, c, nullptr, 0, O, ldo, h->noise);
             if (kpcg::kv_tc_error(*h))
                 fail(KPCG_ERR_TIMEOUT, "a bounded wait in the tensor-core K.V expired");

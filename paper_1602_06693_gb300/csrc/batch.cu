@@ -375,8 +375,8 @@ kpcg_status kpcg_batch_solve(kpcg_batch_t b, const double* B, int64_t ld, int32_
                 // product's reach); steering only: double-float
                 M.prof.time(Profiler::RESID, M.stream, [&] {
                     if (certify)
-                        kv_f64(h.xs64.p, h.n, h.dp, h.c0_64(), h.noise, Xm + off * ldx, ldx, c,
-                               Bm + off * ldb, ldb, R + off * M.ld, M.ld, h.kvws, M.stream);
+                        kv_f64_sym(h, Xm + off * ldx, ldx, c, Bm + off * ldb, ldb, R + off * M.ld,
+                                   M.ld, h.noise);
                     else
                         kv_df(h, Xm + off * ldx, ldx, c, Bm + off * ldb, ldb, R + off * M.ld,
                               M.ld, h.noise);
@@ -424,6 +424,9 @@ kpcg_status kpcg_batch_solve(kpcg_batch_t b, const double* B, int64_t ld, int32_
             prev_worst = worst;
         }
         if (status != KPCG_OK) ops.residual(Bp, L, C, Xp, L, M.R64.p, rr, bn, true);
+        for (auto* h : b->sub)
+            if (kv_tc_error(*h))
+                fail(KPCG_ERR_TIMEOUT, "a bounded wait in the tensor-core K.V expired");
         // exactly ld rows per column of the caller's block (ld may be below L)
         masked_copy_kernel<double, double><<<g, 256, 0, st>>>(X, ld, Xp, L, b->nrow.p, c, ld);
         KPCG_LAUNCHED("masked_copy_kernel");

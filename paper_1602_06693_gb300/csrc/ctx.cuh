@@ -158,6 +158,13 @@ struct Ctx {
     DevBuf<uint16_t> tcdBs;
     DevBuf<int> tcds_work, tcds_rows;
     DevBuf<double> tcdsRow, tcdsCol;
+    // fixed-point FP64-class product (kv_fx.cu): scale S, slices, exp2 table, V bytes
+    int fx_version = -1, fx_op_version = -1;
+    double fx_S = 0.0;
+    DevBuf<uint8_t> fxA, fxB, fxV;
+    DevBuf<uint64_t> fx_tab;
+    DevBuf<unsigned long long> fx_max;
+    DevBuf<double> fxPart;
     // per-point-exact tensor-core operands (kv_tcx_apply), rebuilt when theta changes
     int tcx_version = -1, tcx_kch = 0, tcx_nmma = 0;
     float tcx_escale = 1.f;
@@ -188,8 +195,10 @@ void kv_tc_apply(Ctx& h, const float* V, int64_t ldv, int c, float* O, int64_t l
 // kernel (kv_df.cu); FP64 in and out.
 void kv_df(Ctx& h, const double* V, int64_t ldv, int c, const double* B, int64_t ldb, double* O,
            int64_t ldo, double noise);
-// Native-FP64 product on symmetric tile pairs (kv_df.cu); falls back to the
-// row-split kernel for small n or d > 16.  Same arguments as kv_df.
+// FP64 product (certified residuals, KPCG_FP64): in fixed point on the tensor cores
+// (kv_fx.cu) where that is FP64-accurate, else native FP64 on symmetric tile
+// pairs (kv_df.cu) or, for small n, d > 16 or three and more columns, the row-split
+// kernel.  Same arguments as kv_df.
 void kv_f64_sym(Ctx& h, const double* V, int64_t ldv, int c, const double* B, int64_t ldb,
                 double* O, int64_t ldo, double noise);
 // O = (K + noise I) V in FP32 with exact pairwise differences of the split
@@ -228,6 +237,12 @@ bool kv_tcv_supported(int d);
 void kv_tcd(Ctx& h, const double* V, int64_t ldv, int c, const double* B, int64_t ldb, double* O,
             int64_t ldo, double noise);
 bool kv_tcd_supported(const Ctx& h);
+// FP64-class K.V in fixed point on the tensor cores (kv_fx.cu; arguments of
+// kv_df), for handles where kv_fx_usable holds: d <= 16, scaled inputs within
+// smax, c columns' partial sums within 4 GiB.
+void kv_fx(Ctx& h, const double* V, int64_t ldv, int c, const double* B, int64_t ldb, double* O,
+           int64_t ldo, double noise);
+bool kv_fx_usable(Ctx& h, int c, double smax);
 // Double-float inputs of the handle (exp2 table, log2(s^2) pair), kv_df.cu.
 void df_prepare(Ctx& h);
 // Column count from which the inner products of the mixed solvers use

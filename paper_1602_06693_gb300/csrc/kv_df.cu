@@ -966,7 +966,17 @@ static void f64_sym_launch(int cb, const double* xs, int64_t n, int nt, double c
 void kv_f64_sym(Ctx& h, const double* V, int64_t ldv, int c, const double* B, int64_t ldb,
                 double* O, int64_t ldo, double noise) {
     if (h.n <= 0 || c <= 0) return;
-    if (!(h.dp <= 16 && h.n >= 4 * ST)) {
+    // the fixed-point tensor-core product wherever its operands keep FP64 accuracy
+    // (|y| <= 8: the dropped levels stay near 2^-53 of an entry): 12.1 ms against
+    // 119.6 ms at n = 65536, d = 8 and 0.07 against 0.18 ms at n = 200, one column
+    if (kv_fx_usable(h, c, 8.0)) {
+        kv_fx(h, V, ldv, c, B, ldb, O, ldo, noise);
+        return;
+    }
+    // otherwise on the FP64 pipe: symmetric tile pairs halve the exps but take at
+    // most two columns per pass; from three columns on, one pass over up to 16
+    // columns of the plain kernel computes each entry's exp fewer times
+    if (!(h.dp <= 16 && h.n >= 4 * ST) || (c >= 3 && h.dp <= 16)) {
         kv_f64(h.xs64.p, h.n, h.dp, h.c0_64(), noise, V, ldv, c, B, ldb, O, ldo, h.kvws, h.stream);
         return;
     }
@@ -1010,6 +1020,17 @@ void kv_f64_sym(Ctx& h, const double* V, int64_t ldv, int c, const double* B, in
 void kv_df(Ctx& h, const double* V, int64_t ldv, int c, const double* B, int64_t ldb, double* O,
            int64_t ldo, double noise) {
     if (h.n <= 0 || c <= 0) return;
+    // the fixed-point product (kv_fx.cu; one time for any number of columns) where it is
+    // the faster one: from three columns on (n = 65536, d = 8: 13.0 against
+    // 20.9 ms at three, 14.8 against 40.8 ms at nine; 12.2 against 11.2 ms at two),
+    // for d > 10, whose distances the kernels below take from the FP32 pipe (d = 14,
+    // one column, n = 16384: 0.92 against 1.63 ms), and for few row tiles
+    // (n = 2000, one column: 0.077 against 0.097 ms).  Up to |y| = 64 its dropped levels
+    // stay below the 2^-45 of a double-float entry.
+    if (h.df_tensor && (c >= 3 || h.d > 10 || h.n <= 2048) && kv_fx_usable(h, c, 64.0)) {
+        kv_fx(h, V, ldv, c, B, ldb, O, ldo, noise);
+        return;
+    }
     // the squared distances on the tensor cores where the sliced layout fits
     if (h.df_tensor && kv_tcd_supported(h)) {
         kv_tcd(h, V, ldv, c, B, ldb, O, ldo, noise);

@@ -454,6 +454,8 @@ kpcg_status kpcg_laplace(kpcg_t h, const double* y, double newton_tol, int32_t m
                 break;
             }
         }
+        if (kv_tc_error(c))
+            fail(KPCG_ERR_TIMEOUT, "a bounded wait in the tensor-core K.V expired");
         KPCG_CUDA(cudaMemcpyAsync(f_out, f, sizeof(double) * n, cudaMemcpyDeviceToDevice, st));
         if (a_out)
             KPCG_CUDA(cudaMemcpyAsync(a_out, a, sizeof(double) * n, cudaMemcpyDeviceToDevice, st));
@@ -581,6 +583,8 @@ kpcg_status kpcg_laplace_predict(kpcg_t h, const double* y, const double* f, con
                 KPCG_LAUNCHED("lap_prob_kernel");
             }
         }
+        if (kv_tc_error(c))
+            fail(KPCG_ERR_TIMEOUT, "a bounded wait in the tensor-core K.V expired");
         KPCG_CUDA(cudaStreamSynchronize(st));
         if (info) {
             info->newton_steps = 0;

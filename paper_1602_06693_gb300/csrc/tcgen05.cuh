@@ -88,6 +88,45 @@ __device__ __forceinline__ void mma_commit(uint64_t* b) {
             su32(b))
         : "memory");
 }
+// One thread of a converged warp: 1 in that thread, 0 in the others.  The issuing
+// warp of a kernel runs its loop with all 32 threads and predicates the MMAs on
+// this: the descriptors then live in uniform registers.  In a branch that
+// only lane 0 takes, an MMA with K = 16 issues every 94-107 cycles whatever N is;
+// predicated, every 64 (A in shared memory) or 44 (A in tensor memory) up to
+// N = 128 and N / 2 above (measured on back-to-back MMAs, M = 128).
+__device__ __forceinline__ uint32_t elect_one() {
+    uint32_t e;
+    asm volatile("{\n\t.reg .pred p;\n\telect.sync _|p, 0xffffffff;\n\tselp.u32 %0, 1, 0, p;\n\t}"
+                 : "=r"(e));
+    return e;
+}
+// kind::f16 MMA by the elected thread, A from shared memory / from tensor memory.
+__device__ __forceinline__ void mma_ss(uint32_t dt, uint64_t ad, uint64_t bd, uint32_t idesc,
+                                       uint32_t acc, uint32_t elected) {
+    asm volatile(
+        "{\n\t.reg .pred p, q;\n\tsetp.ne.b32 p, %4, 0;\n\tsetp.ne.b32 q, %5, 0;\n\t@q "
+        "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}" ::"r"(dt),
+        "l"(ad), "l"(bd), "r"(idesc), "r"(acc), "r"(elected));
+}
+__device__ __forceinline__ void mma_ts(uint32_t dt, uint32_t at, uint64_t bd, uint32_t idesc,
+                                       uint32_t acc, uint32_t elected) {
+    asm volatile(
+        "{\n\t.reg .pred p, q;\n\tsetp.ne.b32 p, %4, 0;\n\tsetp.ne.b32 q, %5, 0;\n\t@q "
+        "tcgen05.mma.cta_group::1.kind::f16 [%0], [%1], %2, %3, p;\n\t}" ::"r"(dt),
+        "r"(at), "l"(bd), "r"(idesc), "r"(acc), "r"(elected));
+}
+__device__ __forceinline__ void mma_commit(uint64_t* b, uint32_t elected) {
+    asm volatile(
+        "{\n\t.reg .pred q;\n\tsetp.ne.b32 q, %1, 0;\n\t@q "
+        "tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];\n\t}" ::"r"(
+            su32(b)),
+        "r"(elected)
+        : "memory");
+}
+// mbar_wait by all threads of a warp, with one outcome for all.
+__device__ __forceinline__ bool mbar_wait_warp(uint64_t* b, uint32_t parity, uint64_t deadline) {
+    return __all_sync(0xffffffffu, mbar_wait(b, parity, deadline));
+}
 __device__ __forceinline__ void fence_before() {
     asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
 }
