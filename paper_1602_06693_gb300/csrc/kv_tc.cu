@@ -379,38 +379,37 @@ __global__ void __launch_bounds__(NWARPS * 32, KCH == 1 ? 2 : 1)
             (void)mbar_wait(afull, 0, dl2);
         }
     } else if (warp == 1) {
-        if (lane == 0) {
-            // test hook: a wait on a barrier nothing arrives at runs out
-            if (stall && !mbar_wait(never, 0, deadline)) fail = 1;
-            if (!fail && !mbar_wait(afull, 0, deadline)) fail = 1;
-            fence_after();
-            const uint32_t a0 = su32(sA);
-            for (int t = 0; t < ntiles && !fail; ++t) {
-                const int s = t % NST, b = t & 1;
-                if (!mbar_wait(&full[s], (uint32_t)(t / NST) & 1u, deadline) ||
-                    !mbar_wait(&tempty[b], ((uint32_t)(t >> 1) & 1u) ^ 1u, deadline)) {
-                    fail = 1;
-                    break;
-                }
-                fence_after();
-                const uint32_t b0 = su32(sStage + (size_t)s * S::kStage);
-                const uint32_t dt = tmem + (uint32_t)(b * TN);
-#pragma unroll
-                for (int kc = 0; kc < KCH; ++kc)
-#pragma unroll
-                    for (int kk = 0; kk < KC / 16; ++kk) {
-                        // the exact operands stop at nmma chunks of K = 16
-                        if (EXACT && kc * (KC / 16) + kk >= nmma) continue;
-                        const uint32_t off = (uint32_t)kc * S::kSub + (uint32_t)kk * 32;
-                        mma_bf16(dt, sdesc(a0 + off), sdesc(b0 + off), (kc | kk) ? 1u : 0u);
-                    }
-                mma_commit(&tfull[b]);
-                mma_commit(&empty[s]);
+        const uint32_t el = elect_one();
+        // test hook: a wait on a barrier nothing arrives at runs out
+        if (stall && !mbar_wait_warp(never, 0, deadline)) fail = 1;
+        if (!fail && !mbar_wait_warp(afull, 0, deadline)) fail = 1;
+        fence_after();
+        const uint32_t a0 = su32(sA);
+        for (int t = 0; t < ntiles && !fail; ++t) {
+            const int s = t % NST, b = t & 1;
+            if (!mbar_wait_warp(&full[s], (uint32_t)(t / NST) & 1u, deadline) ||
+                !mbar_wait_warp(&tempty[b], ((uint32_t)(t >> 1) & 1u) ^ 1u, deadline)) {
+                fail = 1;
+                break;
             }
-            // drain: this commit arrives once every MMA issued above has finished
-            mma_commit(done);
-            if (!mbar_wait(done, 0, gtimer() + kWaitNs)) fail = 1;
+            fence_after();
+            const uint32_t b0 = su32(sStage + (size_t)s * S::kStage);
+            const uint32_t dt = tmem + (uint32_t)(b * TN);
+#pragma unroll
+            for (int kc = 0; kc < KCH; ++kc)
+#pragma unroll
+                for (int kk = 0; kk < KC / 16; ++kk) {
+                    // the exact operands stop at nmma chunks of K = 16
+                    if (EXACT && kc * (KC / 16) + kk >= nmma) continue;
+                    const uint32_t off = (uint32_t)kc * S::kSub + (uint32_t)kk * 32;
+                    mma_bf16(dt, sdesc(a0 + off), sdesc(b0 + off), (kc | kk) ? 1u : 0u, el);
+                }
+            mma_commit(&tfull[b], el);
+            mma_commit(&empty[s], el);
         }
+        // drain: this commit arrives once every MMA issued above has finished
+        mma_commit(done, el);
+        if (!mbar_wait_warp(done, 0, gtimer() + kWaitNs)) fail = 1;
     } else {
         for (int t = 0; t < ntiles; ++t) {
             const int s = t % NST, b = t & 1;
@@ -968,50 +967,49 @@ __global__ void __launch_bounds__(NWARPS * 32, 1)
             if (u > 0) (void)mbar_wait(afull, (u - 1) & 1u, dl2);
         }
     } else if (warp == 1) {
-        if (lane == 0) {
-            uint32_t t = 0, u = 0;
-            const uint32_t a0 = su32(sA);
-            for (int it = blockIdx.x; it < nitems && !fail; it += gridDim.x) {
-                const TcBatchItem w = items[it];
-                if (!prob_live(active, w.prob, cpp)) continue;
-                const int kch = probs[w.prob].kch;
-                const int nsub = w.two ? 2 : 1;
-                if (!mbar_wait(afull, u & 1u, deadline)) {
+        const uint32_t el = elect_one();
+        uint32_t t = 0, u = 0;
+        const uint32_t a0 = su32(sA);
+        for (int it = blockIdx.x; it < nitems && !fail; it += gridDim.x) {
+            const TcBatchItem w = items[it];
+            if (!prob_live(active, w.prob, cpp)) continue;
+            const int kch = probs[w.prob].kch;
+            const int nsub = w.two ? 2 : 1;
+            if (!mbar_wait_warp(afull, u & 1u, deadline)) {
+                fail = 1;
+                break;
+            }
+            ++u;
+            fence_after();
+            for (int j = 0; j < w.nt; ++j) {
+                const int s = (int)(t % NSTAGE), b = (int)(t & 1u);
+                if (!mbar_wait_warp(&full[s], (t / NSTAGE) & 1u, deadline) ||
+                    !mbar_wait_warp(&tempty[b], ((t >> 1) & 1u) ^ 1u, deadline)) {
                     fail = 1;
                     break;
                 }
-                ++u;
                 fence_after();
-                for (int j = 0; j < w.nt; ++j) {
-                    const int s = (int)(t % NSTAGE), b = (int)(t & 1u);
-                    if (!mbar_wait(&full[s], (t / NSTAGE) & 1u, deadline) ||
-                        !mbar_wait(&tempty[b], ((t >> 1) & 1u) ^ 1u, deadline)) {
-                        fail = 1;
-                        break;
-                    }
-                    fence_after();
-                    const uint32_t b0 = su32(sStage + (size_t)s * S::kStage);
-                    for (int sub = 0; sub < nsub; ++sub) {
-                        const uint32_t dt = tmem + (uint32_t)(b * 2 * TN + sub * TN);
-                        const uint32_t as = a0 + (uint32_t)sub * S::kA1;
-                        for (int kc = 0; kc < kch; ++kc)
+                const uint32_t b0 = su32(sStage + (size_t)s * S::kStage);
+                for (int sub = 0; sub < nsub; ++sub) {
+                    const uint32_t dt = tmem + (uint32_t)(b * 2 * TN + sub * TN);
+                    const uint32_t as = a0 + (uint32_t)sub * S::kA1;
+                    for (int kc = 0; kc < kch; ++kc)
 #pragma unroll
-                            for (int kk = 0; kk < KC / 16; ++kk) {
-                                const uint32_t off = (uint32_t)kc * S::kSub + (uint32_t)kk * 32;
-                                mma_bf16(dt, sdesc(as + off), sdesc(b0 + off),
-                                         (kc | kk) ? 1u : 0u);
-                            }
-                    }
-                    mma_commit(&tfull[b]);
-                    mma_commit(&empty[s]);
-                    ++t;
+                        for (int kk = 0; kk < KC / 16; ++kk) {
+                            const uint32_t off = (uint32_t)kc * S::kSub + (uint32_t)kk * 32;
+                            mma_bf16(dt, sdesc(as + off), sdesc(b0 + off),
+                                     (kc | kk) ? 1u : 0u, el);
+                        }
                 }
-                if (fail) break;
-                mma_commit(aempty);  // the A tile is free once these MMAs finished
+                mma_commit(&tfull[b], el);
+                mma_commit(&empty[s], el);
+                ++t;
             }
-            mma_commit(done);
-            if (!mbar_wait(done, 0, gtimer() + kWaitNs)) fail = 1;
+            if (fail) break;
+            mma_commit(aempty, el);  // the A tile is free once these MMAs finished
         }
+        mma_commit(done, el);
+        if (!mbar_wait_warp(done, 0, gtimer() + kWaitNs)) fail = 1;
     } else {
         uint32_t t = 0;
         for (int it = blockIdx.x; it < nitems && !fail; it += gridDim.x) {

@@ -203,8 +203,6 @@ struct TcdSmem {
 constexpr uint32_t kIdescD =
     (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(DTN >> 3) << 17) | ((uint32_t)(128 >> 4) << 24);
 
-__device__ __forceinline__ uint64_t sdesc_d(uint32_t saddr) { return sdesc(saddr); }
-
 __device__ __forceinline__ void two_sum(float a, float b, float& s, float& e) {
     s = a + b;
     const float bb = s - a;
@@ -303,37 +301,33 @@ __global__ void __launch_bounds__(DWARPS * 32, 1)
             (void)mbar_wait(afull, 0, dl2);
         }
     } else if (warp == 1) {
-        if (lane == 0) {
-            if (!mbar_wait(afull, 0, deadline)) fail = 1;
-            fence_after();
-            const uint32_t a0 = su32(sA);
-            for (int t = 0; t < ntiles && !fail; ++t) {
-                const int s = t % DNST, b = t & 1;
-                if (!mbar_wait(&full[s], (uint32_t)(t / DNST) & 1u, deadline) ||
-                    !mbar_wait(&tempty[b], ((uint32_t)(t >> 1) & 1u) ^ 1u, deadline)) {
-                    fail = 1;
-                    break;
-                }
-                fence_after();
-                const uint32_t b0 = su32(sStage + (size_t)s * S::kStage);
-                for (int g = 0; g < DNG; ++g) {
-                    const uint32_t dt = tmem + (uint32_t)(b * DNG * DTN + g * DTN);
-                    for (int c16 = L.off[g] >> 4; c16 < (L.off[g + 1] >> 4); ++c16) {
-                        const uint32_t aoff = (uint32_t)(c16 >> 2) * 128 * 128 + (uint32_t)(c16 & 3) * 32;
-                        const uint32_t boff = (uint32_t)(c16 >> 2) * DTN * 128 + (uint32_t)(c16 & 3) * 32;
-                        asm volatile(
-                            "{\n\t.reg .pred p;\n\tsetp.ne.b32 p, %4, 0;\n\t"
-                            "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}" ::"r"(dt),
-                            "l"(sdesc_d(a0 + aoff)), "l"(sdesc_d(b0 + boff)), "r"(kIdescD),
-                            "r"((uint32_t)(c16 != (L.off[g] >> 4))));
-                    }
-                }
-                mma_commit(&tfull[b]);
-                mma_commit(&empty[s]);
+        const uint32_t el = elect_one();
+        if (!mbar_wait_warp(afull, 0, deadline)) fail = 1;
+        fence_after();
+        const uint32_t a0 = su32(sA);
+        for (int t = 0; t < ntiles && !fail; ++t) {
+            const int s = t % DNST, b = t & 1;
+            if (!mbar_wait_warp(&full[s], (uint32_t)(t / DNST) & 1u, deadline) ||
+                !mbar_wait_warp(&tempty[b], ((uint32_t)(t >> 1) & 1u) ^ 1u, deadline)) {
+                fail = 1;
+                break;
             }
-            mma_commit(done);
-            if (!mbar_wait(done, 0, gtimer() + kWaitNs)) fail = 1;
+            fence_after();
+            const uint32_t b0 = su32(sStage + (size_t)s * S::kStage);
+            for (int g = 0; g < DNG; ++g) {
+                const uint32_t dt = tmem + (uint32_t)(b * DNG * DTN + g * DTN);
+                for (int c16 = L.off[g] >> 4; c16 < (L.off[g + 1] >> 4); ++c16) {
+                    const uint32_t aoff = (uint32_t)(c16 >> 2) * 128 * 128 + (uint32_t)(c16 & 3) * 32;
+                    const uint32_t boff = (uint32_t)(c16 >> 2) * DTN * 128 + (uint32_t)(c16 & 3) * 32;
+                    mma_ss(dt, sdesc(a0 + aoff), sdesc(b0 + boff), kIdescD,
+                           (uint32_t)(c16 != (L.off[g] >> 4)), el);
+                }
+            }
+            mma_commit(&tfull[b], el);
+            mma_commit(&empty[s], el);
         }
+        mma_commit(done, el);
+        if (!mbar_wait_warp(done, 0, gtimer() + kWaitNs)) fail = 1;
     } else {
         const uint32_t lane_base = tmem + ((uint32_t)(quarter * 32) << 16);
         for (int t = 0; t < ntiles; ++t) {
@@ -658,37 +652,33 @@ __global__ void __launch_bounds__(SWARPS * 32, 1)
             (void)mbar_wait(afull, 0, dl2);
         }
     } else if (warp == 1) {
-        if (lane == 0) {
-            if (!mbar_wait(afull, 0, deadline)) fail = 1;
-            fence_after();
-            const uint32_t a0 = su32(sA);
-            for (int t = 0; t < ntiles && !fail; ++t) {
-                const int s = t % SNST, b = t & 1;
-                if (!mbar_wait(&full[s], (uint32_t)(t / SNST) & 1u, deadline) ||
-                    !mbar_wait(&tempty[b], ((uint32_t)(t >> 1) & 1u) ^ 1u, deadline)) {
-                    fail = 1;
-                    break;
-                }
-                fence_after();
-                const uint32_t b0 = su32(sStage + (size_t)s * S::kStage);
-                for (int g = 0; g < DNG; ++g) {
-                    const uint32_t dt = tmem + (uint32_t)(b * DNG * STN + g * STN);
-                    for (int c16 = L.off[g] >> 4; c16 < (L.off[g + 1] >> 4); ++c16) {
-                        const uint32_t aoff = (uint32_t)(c16 >> 2) * 128 * 128 + (uint32_t)(c16 & 3) * 32;
-                        const uint32_t boff = (uint32_t)(c16 >> 2) * STN * 128 + (uint32_t)(c16 & 3) * 32;
-                        asm volatile(
-                            "{\n\t.reg .pred p;\n\tsetp.ne.b32 p, %4, 0;\n\t"
-                            "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}" ::"r"(dt),
-                            "l"(sdesc_d(a0 + aoff)), "l"(sdesc_d(b0 + boff)), "r"(kIdescS),
-                            "r"((uint32_t)(c16 != (L.off[g] >> 4))));
-                    }
-                }
-                mma_commit(&tfull[b]);
-                mma_commit(&empty[s]);
+        const uint32_t el = elect_one();
+        if (!mbar_wait_warp(afull, 0, deadline)) fail = 1;
+        fence_after();
+        const uint32_t a0 = su32(sA);
+        for (int t = 0; t < ntiles && !fail; ++t) {
+            const int s = t % SNST, b = t & 1;
+            if (!mbar_wait_warp(&full[s], (uint32_t)(t / SNST) & 1u, deadline) ||
+                !mbar_wait_warp(&tempty[b], ((uint32_t)(t >> 1) & 1u) ^ 1u, deadline)) {
+                fail = 1;
+                break;
             }
-            mma_commit(done);
-            if (!mbar_wait(done, 0, gtimer() + kWaitNs)) fail = 1;
+            fence_after();
+            const uint32_t b0 = su32(sStage + (size_t)s * S::kStage);
+            for (int g = 0; g < DNG; ++g) {
+                const uint32_t dt = tmem + (uint32_t)(b * DNG * STN + g * STN);
+                for (int c16 = L.off[g] >> 4; c16 < (L.off[g + 1] >> 4); ++c16) {
+                    const uint32_t aoff = (uint32_t)(c16 >> 2) * 128 * 128 + (uint32_t)(c16 & 3) * 32;
+                    const uint32_t boff = (uint32_t)(c16 >> 2) * STN * 128 + (uint32_t)(c16 & 3) * 32;
+                    mma_ss(dt, sdesc(a0 + aoff), sdesc(b0 + boff), kIdescS,
+                           (uint32_t)(c16 != (L.off[g] >> 4)), el);
+                }
+            }
+            mma_commit(&tfull[b], el);
+            mma_commit(&empty[s], el);
         }
+        mma_commit(done, el);
+        if (!mbar_wait_warp(done, 0, gtimer() + kWaitNs)) fail = 1;
     } else {
         const uint32_t lane_base = tmem + ((uint32_t)(quarter * 32) << 16);
         float2 vi[CB];  // this row's V, for the column sums

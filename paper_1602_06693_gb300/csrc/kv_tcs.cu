@@ -174,35 +174,34 @@ __global__ void __launch_bounds__(SWARPS_TCS * 32, 1)
             (void)mbar_wait(bfull, 0, dl2);
         }
     } else if (warp == 1) {
-        if (lane == 0) {
-            // test hook: a wait on a barrier nothing arrives at runs out
-            if (stall && !mbar_wait(never, 0, deadline)) fail = 1;
-            if (!fail && !mbar_wait(bfull, 0, deadline)) fail = 1;
-            fence_after();
-            const uint32_t b0 = su32(sB);
-            for (int t = 0; t < ntiles && !fail; ++t) {
-                const int s = t % STAGES_TCS, b = t & 1;
-                if (!mbar_wait(&full[s], (uint32_t)(t / STAGES_TCS) & 1u, deadline) ||
-                    !mbar_wait(&tempty[b], ((uint32_t)(t >> 1) & 1u) ^ 1u, deadline)) {
-                    fail = 1;
-                    break;
-                }
-                fence_after();
-                const uint32_t a0 = su32(sStage + (size_t)s * S::kStage);
-                const uint32_t dt = tmem + (uint32_t)(b * TN);
-#pragma unroll
-                for (int kc = 0; kc < KCH; ++kc)
-#pragma unroll
-                    for (int kk = 0; kk < KC / 16; ++kk) {
-                        const uint32_t off = (uint32_t)kc * S::kSub + (uint32_t)kk * 32;
-                        mma_bf16(dt, sdesc(a0 + off), sdesc(b0 + off), (kc | kk) ? 1u : 0u);
-                    }
-                mma_commit(&tfull[b]);
-                mma_commit(&empty[s]);
+        const uint32_t el = elect_one();
+        // test hook: a wait on a barrier nothing arrives at runs out
+        if (stall && !mbar_wait_warp(never, 0, deadline)) fail = 1;
+        if (!fail && !mbar_wait_warp(bfull, 0, deadline)) fail = 1;
+        fence_after();
+        const uint32_t b0 = su32(sB);
+        for (int t = 0; t < ntiles && !fail; ++t) {
+            const int s = t % STAGES_TCS, b = t & 1;
+            if (!mbar_wait_warp(&full[s], (uint32_t)(t / STAGES_TCS) & 1u, deadline) ||
+                !mbar_wait_warp(&tempty[b], ((uint32_t)(t >> 1) & 1u) ^ 1u, deadline)) {
+                fail = 1;
+                break;
             }
-            mma_commit(done);
-            if (!mbar_wait(done, 0, gtimer() + kWaitNs)) fail = 1;
+            fence_after();
+            const uint32_t a0 = su32(sStage + (size_t)s * S::kStage);
+            const uint32_t dt = tmem + (uint32_t)(b * TN);
+#pragma unroll
+            for (int kc = 0; kc < KCH; ++kc)
+#pragma unroll
+                for (int kk = 0; kk < KC / 16; ++kk) {
+                    const uint32_t off = (uint32_t)kc * S::kSub + (uint32_t)kk * 32;
+                    mma_bf16(dt, sdesc(a0 + off), sdesc(b0 + off), (kc | kk) ? 1u : 0u, el);
+                }
+            mma_commit(&tfull[b], el);
+            mma_commit(&empty[s], el);
         }
+        mma_commit(done, el);
+        if (!mbar_wait_warp(done, 0, gtimer() + kWaitNs)) fail = 1;
     } else {
         // this thread's 64 columns of the resident tile: V_J in registers,
         // column accumulators over the row tiles of the item

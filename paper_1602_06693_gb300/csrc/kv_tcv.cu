@@ -70,15 +70,6 @@ constexpr uint32_t idesc_f16() {
     return (1u << 4) | ((uint32_t)(NB >> 3) << 17) | ((uint32_t)(TM >> 4) << 24);
 }
 
-// D (TMEM) += A (TMEM) B (shared-memory descriptor).
-__device__ __forceinline__ void mma_f16_ta(uint32_t dt, uint32_t at, uint64_t bd, uint32_t idesc,
-                                           uint32_t acc) {
-    asm volatile(
-        "{\n\t.reg .pred p;\n\tsetp.ne.b32 p, %4, 0;\n\ttcgen05.mma.cta_group::1.kind::f16 [%0], "
-        "[%1], %2, %3, p;\n\t}" ::"r"(dt),
-        "r"(at), "l"(bd), "r"(idesc), "r"(acc));
-}
-
 __device__ __forceinline__ void tmem_st32(uint32_t taddr, const uint32_t* r) {
     asm volatile(
         "tcgen05.st.sync.aligned.32x32b.x32.b32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8, %9, %10, "
@@ -215,64 +206,63 @@ __global__ void __launch_bounds__(VWARPS * 32, 1)
             (void)mbar_wait(afull, 0, dl2);
         }
     } else if (warp == 1) {
-        if (lane == 0) {
-            if (stall && !mbar_wait(never, 0, deadline)) fail = 1;
-            if (!fail && !mbar_wait(afull, 0, deadline)) fail = 1;
+        const uint32_t el = elect_one();
+        if (stall && !mbar_wait_warp(never, 0, deadline)) fail = 1;
+        if (!fail && !mbar_wait_warp(afull, 0, deadline)) fail = 1;
+        fence_after();
+        const uint32_t a0 = su32(sA);
+        // the E'.V MMAs of tile u: A = E' hi (part 0) / lo (part 1) in
+        // S[u&1] (half h of the tile's columns at 64 h, hi in its first 32
+        // TMEM columns, lo in the next 32), B = the V tile of stage u % NST
+        auto mma2 = [&](int u) -> bool {
+            const int b = u & 1, s = u % NST;
+            if (!mbar_wait_warp(&efull[b], (uint32_t)(u >> 1) & 1u, deadline) ||
+                !mbar_wait_warp(&dempty[b], ((uint32_t)(u >> 1) & 1u) ^ 1u, deadline))
+                return false;
             fence_after();
-            const uint32_t a0 = su32(sA);
-            // the E'.V MMAs of tile u: A = E' hi (part 0) / lo (part 1) in
-            // S[u&1] (half h of the tile's columns at 64 h, hi in its first 32
-            // TMEM columns, lo in the next 32), B = the V tile of stage u % NST
-            auto mma2 = [&](int u) -> bool {
-                const int b = u & 1, s = u % NST;
-                if (!mbar_wait(&efull[b], (uint32_t)(u >> 1) & 1u, deadline) ||
-                    !mbar_wait(&dempty[b], ((uint32_t)(u >> 1) & 1u) ^ 1u, deadline))
-                    return false;
-                fence_after();
-                const uint32_t vb = su32(sStage + (size_t)s * S::kStage + S::kBst);
-                const uint32_t sb = tmem + (uint32_t)(b * TN);
-                const uint32_t db = tmem + 256u + (uint32_t)(b * 128);
+            const uint32_t vb = su32(sStage + (size_t)s * S::kStage + S::kBst);
+            const uint32_t sb = tmem + (uint32_t)(b * TN);
+            const uint32_t db = tmem + 256u + (uint32_t)(b * 128);
 #pragma unroll
-                for (int p = 0; p < 2; ++p)
+            for (int p = 0; p < 2; ++p)
 #pragma unroll
-                    for (int kk = 0; kk < TN / 16; ++kk) {
-                        const uint32_t at =
-                            sb + (uint32_t)((kk >> 2) * 64 + p * 32 + (kk & 3) * 8);
-                        const uint64_t bd =
-                            sdesc(vb + (uint32_t)((kk >> 2) * (NB * 128) + (kk & 3) * 32));
-                        // K-chunk kk into region kk / KPR of D, each region restarted
-                        mma_f16_ta(db + (uint32_t)((kk / KPR) * NB), at, bd, idesc_f16<NB>(),
-                                   (p | (kk % KPR)) ? 1u : 0u);
-                    }
-                mma_commit(&sfree[b]);
-                mma_commit(&dfull[b]);
-                mma_commit(&empty[s]);
-                return true;
-            };
-            for (int t = 0; t < ntiles && !fail; ++t) {
-                const int s = t % NST, b = t & 1;
-                if (!mbar_wait(&full[s], (uint32_t)(t / NST) & 1u, deadline) ||
-                    !mbar_wait(&sfree[b], ((uint32_t)(t >> 1) & 1u) ^ 1u, deadline)) {
-                    fail = 1;
-                    break;
+                for (int kk = 0; kk < TN / 16; ++kk) {
+                    const uint32_t at =
+                        sb + (uint32_t)((kk >> 2) * 64 + p * 32 + (kk & 3) * 8);
+                    const uint64_t bd =
+                        sdesc(vb + (uint32_t)((kk >> 2) * (NB * 128) + (kk & 3) * 32));
+                    // K-chunk kk into region kk / KPR of D, each region restarted
+                    mma_ts(db + (uint32_t)((kk / KPR) * NB), at, bd, idesc_f16<NB>(),
+                               (p | (kk % KPR)) ? 1u : 0u, el);
                 }
-                fence_after();
-                const uint32_t b0 = su32(sStage + (size_t)s * S::kStage);
-                const uint32_t dt = tmem + (uint32_t)(b * TN);
-#pragma unroll
-                for (int kc = 0; kc < KCH; ++kc)
-#pragma unroll
-                    for (int kk = 0; kk < KC / 16; ++kk) {
-                        const uint32_t off = (uint32_t)kc * S::kSub + (uint32_t)kk * 32;
-                        mma_bf16(dt, sdesc(a0 + off), sdesc(b0 + off), (kc | kk) ? 1u : 0u);
-                    }
-                mma_commit(&tfull[b]);
-                if (t >= 1 && !mma2(t - 1)) fail = 1;
+            mma_commit(&sfree[b], el);
+            mma_commit(&dfull[b], el);
+            mma_commit(&empty[s], el);
+            return true;
+        };
+        for (int t = 0; t < ntiles && !fail; ++t) {
+            const int s = t % NST, b = t & 1;
+            if (!mbar_wait_warp(&full[s], (uint32_t)(t / NST) & 1u, deadline) ||
+                !mbar_wait_warp(&sfree[b], ((uint32_t)(t >> 1) & 1u) ^ 1u, deadline)) {
+                fail = 1;
+                break;
             }
-            if (!fail && ntiles >= 1 && !mma2(ntiles - 1)) fail = 1;
-            mma_commit(done);
-            if (!mbar_wait(done, 0, gtimer() + kWaitNs)) fail = 1;
+            fence_after();
+            const uint32_t b0 = su32(sStage + (size_t)s * S::kStage);
+            const uint32_t dt = tmem + (uint32_t)(b * TN);
+#pragma unroll
+            for (int kc = 0; kc < KCH; ++kc)
+#pragma unroll
+                for (int kk = 0; kk < KC / 16; ++kk) {
+                    const uint32_t off = (uint32_t)kc * S::kSub + (uint32_t)kk * 32;
+                    mma_bf16(dt, sdesc(a0 + off), sdesc(b0 + off), (kc | kk) ? 1u : 0u, el);
+                }
+            mma_commit(&tfull[b], el);
+            if (t >= 1 && !mma2(t - 1)) fail = 1;
         }
+        if (!fail && ntiles >= 1 && !mma2(ntiles - 1)) fail = 1;
+        mma_commit(done, el);
+        if (!mbar_wait_warp(done, 0, gtimer() + kWaitNs)) fail = 1;
     } else {
         const uint32_t lane_base = tmem + ((uint32_t)(quarter * 32) << 16);
         // D of tile u into the row sums (columns 2k, 2k+1: E'.V'hi, E'.V'lo)
@@ -646,75 +636,74 @@ __global__ void __launch_bounds__(VWARPS * 32, 1)
             if (u > 0) (void)mbar_wait(afull, (u - 1) & 1u, dl2);
         }
     } else if (warp == 1) {
-        if (lane == 0) {
-            const uint32_t a0 = su32(sA);
-            auto mma2 = [&](uint32_t v) -> bool {
-                const int b = (int)(v & 1u), s = (int)(v % NST);
-                if (!mbar_wait(&efull[b], (v >> 1) & 1u, deadline) ||
-                    !mbar_wait(&dempty[b], ((v >> 1) & 1u) ^ 1u, deadline))
-                    return false;
-                fence_after();
-                const uint32_t vb = su32(sStage + (size_t)s * S::kStage + S::kBst);
-                const uint32_t sb = tmem + (uint32_t)(b * TN);
-                const uint32_t db = tmem + 256u + (uint32_t)(b * 128);
+        const uint32_t el = elect_one();
+        const uint32_t a0 = su32(sA);
+        auto mma2 = [&](uint32_t v) -> bool {
+            const int b = (int)(v & 1u), s = (int)(v % NST);
+            if (!mbar_wait_warp(&efull[b], (v >> 1) & 1u, deadline) ||
+                !mbar_wait_warp(&dempty[b], ((v >> 1) & 1u) ^ 1u, deadline))
+                return false;
+            fence_after();
+            const uint32_t vb = su32(sStage + (size_t)s * S::kStage + S::kBst);
+            const uint32_t sb = tmem + (uint32_t)(b * TN);
+            const uint32_t db = tmem + 256u + (uint32_t)(b * 128);
 #pragma unroll
-                for (int p = 0; p < 2; ++p)
+            for (int p = 0; p < 2; ++p)
 #pragma unroll
-                    for (int kk = 0; kk < TN / 16; ++kk) {
-                        const uint32_t at =
-                            sb + (uint32_t)((kk >> 2) * 64 + p * 32 + (kk & 3) * 8);
-                        const uint64_t bd =
-                            sdesc(vb + (uint32_t)((kk >> 2) * (NB * 128) + (kk & 3) * 32));
-                        // K-chunk kk into region kk / KPR of D, each region restarted
-                        mma_f16_ta(db + (uint32_t)((kk / KPR) * NB), at, bd, idesc_f16<NB>(),
-                                   (p | (kk % KPR)) ? 1u : 0u);
-                    }
-                mma_commit(&sfree[b]);
-                mma_commit(&dfull[b]);
-                mma_commit(&empty[s]);
-                return true;
-            };
-            uint32_t t = 0, u = 0;
-            for (int it = blockIdx.x; it < nitems && !fail; it += gridDim.x) {
-                const TcBatchItem w = items[it];
-                if (!live(w.prob)) continue;
-                const int kch = probs[w.prob].kch;
-                if (!mbar_wait(afull, u & 1u, deadline)) {
+                for (int kk = 0; kk < TN / 16; ++kk) {
+                    const uint32_t at =
+                        sb + (uint32_t)((kk >> 2) * 64 + p * 32 + (kk & 3) * 8);
+                    const uint64_t bd =
+                        sdesc(vb + (uint32_t)((kk >> 2) * (NB * 128) + (kk & 3) * 32));
+                    // K-chunk kk into region kk / KPR of D, each region restarted
+                    mma_ts(db + (uint32_t)((kk / KPR) * NB), at, bd, idesc_f16<NB>(),
+                               (p | (kk % KPR)) ? 1u : 0u, el);
+                }
+            mma_commit(&sfree[b], el);
+            mma_commit(&dfull[b], el);
+            mma_commit(&empty[s], el);
+            return true;
+        };
+        uint32_t t = 0, u = 0;
+        for (int it = blockIdx.x; it < nitems && !fail; it += gridDim.x) {
+            const TcBatchItem w = items[it];
+            if (!live(w.prob)) continue;
+            const int kch = probs[w.prob].kch;
+            if (!mbar_wait_warp(afull, u & 1u, deadline)) {
+                fail = 1;
+                break;
+            }
+            ++u;
+            fence_after();
+            for (int j = 0; j < w.nt; ++j) {
+                const int s = (int)(t % NST), b = (int)(t & 1u);
+                if (!mbar_wait_warp(&full[s], (t / NST) & 1u, deadline) ||
+                    !mbar_wait_warp(&sfree[b], ((t >> 1) & 1u) ^ 1u, deadline)) {
                     fail = 1;
                     break;
                 }
-                ++u;
                 fence_after();
-                for (int j = 0; j < w.nt; ++j) {
-                    const int s = (int)(t % NST), b = (int)(t & 1u);
-                    if (!mbar_wait(&full[s], (t / NST) & 1u, deadline) ||
-                        !mbar_wait(&sfree[b], ((t >> 1) & 1u) ^ 1u, deadline)) {
-                        fail = 1;
-                        break;
-                    }
-                    fence_after();
-                    const uint32_t b0 = su32(sStage + (size_t)s * S::kStage);
-                    const uint32_t dt = tmem + (uint32_t)(b * TN);
-                    for (int kc = 0; kc < kch; ++kc)
+                const uint32_t b0 = su32(sStage + (size_t)s * S::kStage);
+                const uint32_t dt = tmem + (uint32_t)(b * TN);
+                for (int kc = 0; kc < kch; ++kc)
 #pragma unroll
-                        for (int kk = 0; kk < KC / 16; ++kk) {
-                            const uint32_t off = (uint32_t)kc * S::kSub + (uint32_t)kk * 32;
-                            mma_bf16(dt, sdesc(a0 + off), sdesc(b0 + off), (kc | kk) ? 1u : 0u);
-                        }
-                    mma_commit(&tfull[b]);
-                    if (t >= 1 && !mma2(t - 1)) {
-                        fail = 1;
-                        break;
+                    for (int kk = 0; kk < KC / 16; ++kk) {
+                        const uint32_t off = (uint32_t)kc * S::kSub + (uint32_t)kk * 32;
+                        mma_bf16(dt, sdesc(a0 + off), sdesc(b0 + off), (kc | kk) ? 1u : 0u, el);
                     }
-                    ++t;
+                mma_commit(&tfull[b], el);
+                if (t >= 1 && !mma2(t - 1)) {
+                    fail = 1;
+                    break;
                 }
-                if (fail) break;
-                mma_commit(aempty);  // the A tile is free once these MMAs finished
+                ++t;
             }
-            if (!fail && t >= 1 && !mma2(t - 1)) fail = 1;
-            mma_commit(done);
-            if (!mbar_wait(done, 0, gtimer() + kWaitNs)) fail = 1;
+            if (fail) break;
+            mma_commit(aempty, el);  // the A tile is free once these MMAs finished
         }
+        if (!fail && t >= 1 && !mma2(t - 1)) fail = 1;
+        mma_commit(done, el);
+        if (!mbar_wait_warp(done, 0, gtimer() + kWaitNs)) fail = 1;
     } else {
         const uint32_t lane_base = tmem + ((uint32_t)(quarter * 32) << 16);
         float acc[KH];

@@ -76,18 +76,6 @@ __device__ __forceinline__ uint64_t sdesc(uint32_t saddr) {
 constexpr uint32_t kIdesc = (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(TN >> 3) << 17) |
                             ((uint32_t)(TM >> 4) << 24);
 
-__device__ __forceinline__ void mma_bf16(uint32_t dt, uint64_t ad, uint64_t bd, uint32_t acc) {
-    asm volatile(
-        "{\n\t.reg .pred p;\n\tsetp.ne.b32 p, %4, 0;\n\ttcgen05.mma.cta_group::1.kind::f16 [%0], "
-        "%1, %2, %3, p;\n\t}" ::"r"(dt),
-        "l"(ad), "l"(bd), "r"(kIdesc), "r"(acc));
-}
-__device__ __forceinline__ void mma_commit(uint64_t* b) {
-    asm volatile(
-        "tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(
-            su32(b))
-        : "memory");
-}
 // One thread of a converged warp: 1 in that thread, 0 in the others.  The issuing
 // warp of a kernel runs its loop with all 32 threads and predicates the MMAs on
 // this: the descriptors then live in uniform registers.  In a branch that
@@ -114,6 +102,10 @@ __device__ __forceinline__ void mma_ts(uint32_t dt, uint32_t at, uint64_t bd, ui
         "{\n\t.reg .pred p, q;\n\tsetp.ne.b32 p, %4, 0;\n\tsetp.ne.b32 q, %5, 0;\n\t@q "
         "tcgen05.mma.cta_group::1.kind::f16 [%0], [%1], %2, %3, p;\n\t}" ::"r"(dt),
         "r"(at), "l"(bd), "r"(idesc), "r"(acc), "r"(elected));
+}
+__device__ __forceinline__ void mma_bf16(uint32_t dt, uint64_t ad, uint64_t bd, uint32_t acc,
+                                         uint32_t elected) {
+    mma_ss(dt, ad, bd, kIdesc, acc, elected);
 }
 __device__ __forceinline__ void mma_commit(uint64_t* b, uint32_t elected) {
     asm volatile(
