@@ -55,6 +55,15 @@ __device__ __forceinline__ bool mbar_wait(uint64_t* b, uint32_t parity, uint64_t
         if ((it & 255u) == 0 && gtimer() > deadline) return false;
     }
 }
+// The same for a warp that runs ahead of the others (a producer): it sleeps between
+// attempts instead of polling in the issue slots of the warps that compute.
+__device__ __forceinline__ bool mbar_wait_idle(uint64_t* b, uint32_t parity, uint64_t deadline) {
+    for (uint32_t it = 1;; ++it) {
+        if (mbar_try(b, parity)) return true;
+        if ((it & 255u) == 0 && gtimer() > deadline) return false;
+        __nanosleep(100);
+    }
+}
 __device__ __forceinline__ void bulk_g2s(void* dst, const void* src, uint32_t bytes,
                                          uint64_t* bar) {
     asm volatile(
@@ -118,6 +127,18 @@ __device__ __forceinline__ void mma_commit(uint64_t* b, uint32_t elected) {
 // mbar_wait by all threads of a warp, with one outcome for all.
 __device__ __forceinline__ bool mbar_wait_warp(uint64_t* b, uint32_t parity, uint64_t deadline) {
     return __all_sync(0xffffffffu, mbar_wait(b, parity, deadline));
+}
+__device__ __forceinline__ float4 lds128(uint32_t saddr) {
+    float4 v;
+    asm volatile("ld.shared.v4.f32 {%0, %1, %2, %3}, [%4];"
+                 : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w)
+                 : "r"(saddr));
+    return v;
+}
+__device__ __forceinline__ float lds32(uint32_t saddr) {
+    float v;
+    asm volatile("ld.shared.f32 %0, [%1];" : "=f"(v) : "r"(saddr));
+    return v;
 }
 __device__ __forceinline__ void fence_before() {
     asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
