@@ -3,9 +3,9 @@
 // Nystrom.  P = K_XU K_UU^{-1} K_UX + sigma^2 I, inverted by the matrix
 // inversion lemma as P^{-1} = sigma^{-2} [I - K_XU M^{-1} K_UX] with
 // M = sigma^2 K_UU + K_UX K_XU (the printed inverse drops the sigma^2 on K_UU).
-// K_XU holds FP64 entries as exact FP32 pairs; M is formed from it with FP64
-// products and sums (see syrk_kxu_kernel for why nothing less will do).  M = L L^T is factored in FP64 and
-// L^{-1} formed explicitly (stored as U = L^{-T}, row-major), so an apply is
+// K_XU holds FP64 entries as exact FP32 pairs; M is formed from it in fixed point
+// (syrk_fx.cu, which says why nothing below FP64 accuracy will do).  M = L L^T is
+// factored in FP64 and L^{-1} formed explicitly (stored as U = L^{-T}, row-major), so an apply is
 // two skinny products with K_XU and two m x m triangular products.  K_UX r uses
 // compensated FP32 (Dot2) on the pairs, the rest is FP64: with sigma^2 small
 // the difference r - K_XU M^{-1} K_UX r cancels almost completely along the
@@ -219,75 +219,21 @@ __global__ void gather_rows_f64(const double* __restrict__ src, const int64_t* _
     dst[e] = src[idx[a] * dp + (e - a * dp)];
 }
 
-// part[s][a][b] = sum over rows of split s of KXU[i][a] KXU[i][b], lower tiles,
-// in FP64 (entries are exact FP32 pairs, hi + lo).  M = noise K_UU + K_UX K_XU
-// is nearly singular (kappa ~ 1e11 at noise 1e-4) and the preconditioner it
-// defines implicitly inverts K_UU, whose small eigenvalues are far below the
-// 2^-48 relative error of a compensated-FP32 sum divided by the noise: such
-// errors made the preconditioner indefinite and doubled the PCG iteration
-// count.  FP64 products and sums keep it at the accuracy of a direct FP64
-// construction.
-constexpr int ST = 64;  // output tile
-constexpr int SR = 16;  // rows per stage
-__global__ void __launch_bounds__(256)
-    syrk_kxu_kernel(const float2* __restrict__ KXU, int64_t n, int64_t m, int64_t rows_per_split,
-                    double* __restrict__ part) {
-    __shared__ double Aa[SR][ST];
-    __shared__ double Ab[SR][ST];
-    const int64_t ta = blockIdx.y, tb = blockIdx.x;
-    if (tb > ta) return;
-    const int64_t a0 = ta * ST, b0 = tb * ST;
-    const int64_t r0 = (int64_t)blockIdx.z * rows_per_split;
-    const int64_t r1 = min(n, r0 + rows_per_split);
-    const int tx = threadIdx.x & 15, ty = threadIdx.x >> 4;  // 4 x 4 outputs each
-    double acc[4][4];
-#pragma unroll
-    for (int u = 0; u < 4; ++u)
-#pragma unroll
-        for (int v = 0; v < 4; ++v) acc[u][v] = 0.0;
-    for (int64_t rs = r0; rs < r1; rs += SR) {
-        __syncthreads();
-        for (int e = threadIdx.x; e < SR * ST; e += 256) {
-            const int r = e / ST, c = e % ST;
-            const int64_t i = rs + r;
-            float2 ka = (i < r1 && a0 + c < m) ? KXU[i * m + a0 + c] : make_float2(0.f, 0.f);
-            float2 kb = (i < r1 && b0 + c < m) ? KXU[i * m + b0 + c] : make_float2(0.f, 0.f);
-            Aa[r][c] = (double)ka.x + (double)ka.y;
-            Ab[r][c] = (double)kb.x + (double)kb.y;
-        }
-        __syncthreads();
-#pragma unroll 2
-        for (int r = 0; r < SR; ++r) {
-            double va[4], vb[4];
-#pragma unroll
-            for (int u = 0; u < 4; ++u) va[u] = Aa[r][ty * 4 + u];
-#pragma unroll
-            for (int v = 0; v < 4; ++v) vb[v] = Ab[r][tx * 4 + v];
-#pragma unroll
-            for (int u = 0; u < 4; ++u)
-#pragma unroll
-                for (int v = 0; v < 4; ++v) acc[u][v] = fma(va[u], vb[v], acc[u][v]);
-        }
-    }
-    double* P = part + (int64_t)blockIdx.z * m * m;
-#pragma unroll
-    for (int u = 0; u < 4; ++u)
-#pragma unroll
-        for (int v = 0; v < 4; ++v) {
-            const int64_t a = a0 + ty * 4 + u, bb = b0 + tx * 4 + v;
-            if (a < m && bb < m && bb <= a) P[a * m + bb] = acc[u][v];
-        }
-}
-
-// M[a][b] += sum_s part[s][a][b] (lower), then mirror to the upper triangle.
+// M[a][b] += sum_s part[s][a][b] (lower), then mirror to the upper triangle.  TwoSum keeps
+// the additions' errors: up to 152 parts, each with FP64's rounding only.
 __global__ void syrk_reduce_kernel(const double* __restrict__ part, int nsplit, int64_t m,
                                    double* __restrict__ M) {
     const int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (e >= m * m) return;
     const int64_t a = e / m, b = e % m;
     if (b > a) return;
-    double s = M[e];
-    for (int sp = 0; sp < nsplit; ++sp) s += part[(int64_t)sp * m * m + e];
+    double s = M[e], r = 0.0;
+    for (int sp = 0; sp < nsplit; ++sp) {
+        const double v = part[(int64_t)sp * m * m + e], t = s + v, z = t - s;
+        r += (s - (t - z)) + (v - z);
+        s = t;
+    }
+    s += r;
     M[e] = s;
     M[b * m + a] = s;
 }
@@ -678,7 +624,7 @@ static double factor_with_rule(PrecondState& P, const double* A0, int64_t m, cud
     const double kPivotTol = 3e-12;
     double* M = P.M.need((size_t)m * m);
     double* U = P.U.need((size_t)m * m);
-    int* status = P.status.need(1);
+    int* status = P.status.need(2);
     int rc = 1;
     double jitter = 0.0;
     for (int k = -1; k <= 6 && rc; ++k) {
@@ -694,27 +640,22 @@ static double factor_with_rule(PrecondState& P, const double* A0, int64_t m, cud
     return jitter;
 }
 
-// M0 += K_UX K_XU (FP64 SYRK over the pairs of P.KXU, n x m), then M0 is
+// M0 += K_UX K_XU (fixed-point sum over the pairs of P.KXU, n x m), then M0 is
 // factored by the rule.
 static void nys_syrk_factor(PrecondState& P, int64_t n, int64_t m, cudaStream_t st,
                             const char* what) {
     double* M0 = P.M0.p;
-    const int64_t tiles = (m + ST - 1) / ST;
-    // row splits: one per 4096 rows (at most 64), and enough for about four
-    // CTAs per SM over the lower tiles when m is small, with >= 4 SR rows each
-    const int64_t lower = tiles * (tiles + 1) / 2;
-    int64_t ns = std::max<int64_t>(std::min<int64_t>(64, (n + 4095) / 4096),
-                                   (152 * 4 + lower - 1) / lower);
-    ns = std::min<int64_t>(ns, std::max<int64_t>(1, n / (4 * SR)));
-    int nsplit = (int)std::max<int64_t>(1, ns);
-    const int64_t rps = ((n + nsplit - 1) / nsplit + SR - 1) / SR * SR;
-    nsplit = (int)((n + rps - 1) / rps);
+    const int nsplit = syrk_fx_splits(n, m);
     double* part = P.scratch.need((size_t)nsplit * m * m);
-    dim3 gs((unsigned)tiles, (unsigned)tiles, (unsigned)nsplit);
-    syrk_kxu_kernel<<<gs, 256, 0, st>>>(P.KXU.p, n, m, rps, part);
-    KPCG_LAUNCHED("syrk_kxu_kernel");
+    int* late = P.status.need(2) + 1;
+    KPCG_CUDA(cudaMemsetAsync(late, 0, sizeof(int), st));
+    syrk_fx(P.KXU.p, n, m, P.digits, part, late, st);
     syrk_reduce_kernel<<<(unsigned)((m * m + 255) / 256), 256, 0, st>>>(part, nsplit, m, M0);
     KPCG_LAUNCHED("syrk_reduce_kernel");
+    int bad = 0;
+    KPCG_CUDA(cudaMemcpyAsync(&bad, late, sizeof(int), cudaMemcpyDeviceToHost, st));
+    KPCG_CUDA(cudaStreamSynchronize(st));
+    if (bad) fail(KPCG_ERR_TIMEOUT, "a bounded wait in the Nystrom set-up expired");
     P.jitter = factor_with_rule(P, M0, m, st, what);
 }
 

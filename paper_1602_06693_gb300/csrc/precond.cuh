@@ -22,6 +22,7 @@ struct PrecondState {
     DevBuf<double> M;        // Cholesky factor(s) L
     DevBuf<double> U;        // L^{-T}, row-major (per block for block-Jacobi)
     DevBuf<double> scratch;  // split partials of the set-up products
+    DevBuf<uint8_t> digits;  // row blocks of K_XU as digits (syrk_fx.cu)
     DevBuf<double> wpart, w, y;
     DevBuf<int> status;
     double apply_noise = 0.0;  // divisor of the Nystrom apply (1 for FITC's scaled form)
@@ -41,6 +42,7 @@ struct PrecondState {
         M.release();
         U.release();
         scratch.release();
+        digits.release();
         wpart.release();
         w.release();
         y.release();
@@ -98,6 +100,13 @@ void fitc_setup(PrecondState& P, const float* xs32, const double* xs64, int64_t 
 void pitc_setup(PrecondState& P, const float* xs32, const double* xs64, int64_t n, int dp,
                 double c0_64, double noise, const int64_t* idx_host, int64_t m, int64_t b,
                 cudaStream_t st);
+
+// part[s] (s < syrk_fx_splits(n, m), each m x m row-major) = parts of the lower triangle
+// of KXU^T KXU (KXU n x m FP32 pairs) in fixed point on the tensor cores (syrk_fx.cu).
+// err is set if a bounded wait expires.
+int syrk_fx_splits(int64_t n, int64_t m);
+void syrk_fx(const float2* KXU, int64_t n, int64_t m, DevBuf<uint8_t>& work, double* part,
+             int* err, cudaStream_t st);
 
 // ------------------------------------------- batched Nystrom apply
 // Problems laid out column by column (problem p owns columns p*c .. p*c+c-1
