@@ -205,14 +205,9 @@ static int pcg_core(Ctx& h, int c, const T* B, int64_t ldb, T* X, int64_t ldx, b
     const bool graphs = h.use_graph && !h.prof.on;
     auto body = [&](cudaStream_t s) {
         matvec(p, ld, c, q, ld);
-        dot_cols<T>(p, ld, q, ld, n, c, partial, nblk, s);
-        finalize(partial, nblk, c, FIN_ALPHA, S, tol, tol_mode, n, nullptr, s);
-        update_xr<T>(X, ldx, r, ld, p, ld, q, ld, n, c, S.alpha, partial, nblk, s);
-        finalize(partial, nblk, c, FIN_RR, S, tol, tol_mode, n, nullptr, s);
+        cg_step<T>(X, ldx, r, ld, p, ld, q, ld, n, c, S, partial, nblk, s);
         precond(r, ld, c, z, ld);
-        dot_cols<T>(r, ld, z, ld, n, c, partial, nblk, s);
-        finalize(partial, nblk, c, FIN_BETA, S, tol, tol_mode, n, nullptr, s);
-        update_p<T>(p, ld, z, ld, n, c, S.beta, S.active, s);
+        cg_direction<T>(p, ld, r, ld, z, ld, n, c, S, partial, nblk, s);
     };
     while (active > 0 && it < max_iter) {
         if (graphs && it >= every && it + every <= max_iter) {
@@ -230,10 +225,7 @@ static int pcg_core(Ctx& h, int c, const T* B, int64_t ldb, T* X, int64_t ldx, b
             continue;
         }
         matvec(p, ld, c, q, ld);
-        dot_cols<T>(p, ld, q, ld, n, c, partial, nblk, st);
-        finalize(partial, nblk, c, FIN_ALPHA, S, tol, tol_mode, n, nullptr, st);
-        update_xr<T>(X, ldx, r, ld, p, ld, q, ld, n, c, S.alpha, partial, nblk, st);
-        finalize(partial, nblk, c, FIN_RR, S, tol, tol_mode, n, nullptr, st);
+        cg_step<T>(X, ldx, r, ld, p, ld, q, ld, n, c, S, partial, nblk, st);
         ++it;
         if (it % every == 0 || it >= max_iter) {
             KPCG_CUDA(cudaMemcpyAsync(hf, S.flags, 2 * sizeof(int), cudaMemcpyDeviceToHost, st));
@@ -242,9 +234,7 @@ static int pcg_core(Ctx& h, int c, const T* B, int64_t ldb, T* X, int64_t ldx, b
             if (active == 0) break;
         }
         precond(r, ld, c, z, ld);
-        dot_cols<T>(r, ld, z, ld, n, c, partial, nblk, st);
-        finalize(partial, nblk, c, FIN_BETA, S, tol, tol_mode, n, nullptr, st);
-        update_p<T>(p, ld, z, ld, n, c, S.beta, S.active, st);
+        cg_direction<T>(p, ld, r, ld, z, ld, n, c, S, partial, nblk, st);
     }
     std::vector<int> its((size_t)c);
     KPCG_CUDA(cudaMemcpyAsync(its.data(), S.iters, sizeof(int) * c, cudaMemcpyDeviceToHost, st));

@@ -7,6 +7,12 @@
 // in a fixed order by one small kernel that also runs the scalar logic
 // (deterministic, no atomics).  Scalars never leave the device; the host
 // only polls the count of active columns.
+//
+// Up to kStepN rows one cluster of CTAs per column does a whole half of the iteration: step_kernel
+// (p.q, alpha, x and r, ||r||^2 and the stop test) and direction_kernel (r.z, beta, p),
+// two launches for the seven of the parts.  Vectors of this size live in L2 and the parts
+// are launches and latency.
+#include <cooperative_groups.h>
 #include <cuda_runtime.h>
 
 #include "kpcg_internal.cuh"
@@ -36,6 +42,16 @@ __device__ __forceinline__ double block_sum(double v, double* sh) {
     return t;
 }
 
+// (double)f for any f: integer operations, since the conversion instruction runs at one per
+// clock and SM.
+__device__ __forceinline__ double widen(float f) {
+    const unsigned u = __float_as_uint(f), e = u & 0x7f800000u;
+    if (e == 0x7f800000u || (e == 0u && (u << 1))) return (double)f;  // Inf, NaN, subnormal
+    const unsigned hi = (u & 0x80000000u) | (e ? ((u & 0x7fffffffu) >> 3) + 0x38000000u : 0u);
+    return __hiloint2double((int)hi, (int)(u << 29));
+}
+__device__ __forceinline__ double widen(double f) { return f; }
+
 template <typename T>
 __global__ void __launch_bounds__(DT)
     dot_kernel(const T* __restrict__ A, int64_t lda, const T* __restrict__ B, int64_t ldb,
@@ -46,7 +62,7 @@ __global__ void __launch_bounds__(DT)
     const T* b = B + (int64_t)k * ldb;
     double s = 0.0;
     for (int64_t i = (int64_t)blockIdx.x * DT + threadIdx.x; i < n; i += (int64_t)nblk * DT)
-        s = fma((double)a[i], (double)b[i], s);
+        s = fma(widen(a[i]), widen(b[i]), s);
     s = block_sum(s, sh);
     if (threadIdx.x == 0) partial[(int64_t)k * nblk + blockIdx.x] = s;
 }
@@ -74,7 +90,7 @@ __global__ void __launch_bounds__(DT)
             ri = fma(-a, qk[i], ri);
             rk[i] = ri;
         }
-        s = fma((double)ri, (double)ri, s);
+        s = fma(widen(ri), widen(ri), s);
     }
     s = block_sum(s, sh);
     if (threadIdx.x == 0) partial[(int64_t)k * nblk + blockIdx.x] = s;
@@ -161,6 +177,172 @@ __global__ void finalize_kernel(const double* __restrict__ partial, int nblk, in
     }
 }
 
+constexpr int QT = 256;  // threads per CTA of the cluster kernels
+constexpr int QCL = 8;   // CTAs per cluster at most (the portable size)
+
+// Sum over the cluster in a fixed order, the same in every thread.  An FP64 addition of a
+// warp takes 16 cycles whatever its lanes do, so one warp adds the CTA's values column by
+// column instead of every warp running a butterfly.  slot: one per call of a kernel; the
+// kernel ends with a cluster barrier, as the peers read it.
+__device__ __forceinline__ double cluster_sum(double v, double* sh, double* slot) {
+    namespace cg = cooperative_groups;
+    cg::cluster_group cl = cg::this_cluster();
+    sh[threadIdx.x] = v;
+    __syncthreads();
+    if (threadIdx.x < 32) {
+        double t = 0.0;
+#pragma unroll
+        for (int j = 0; j < QT / 32; ++j) t += sh[j * 32 + threadIdx.x];
+        t = warp_sum(t);
+        if (threadIdx.x == 0) *slot = t;
+    }
+    cl.sync();
+    const unsigned nr = cl.num_blocks();
+    if (threadIdx.x < 32) {
+        double t = 0.0;
+        for (unsigned b = 0; b < nr; ++b) t += *cl.map_shared_rank(slot, b);
+        if (threadIdx.x == 0) sh[0] = t;
+    }
+    __syncthreads();
+    const double t = sh[0];
+    __syncthreads();
+    return t;
+}
+
+// A thread's elements i, i + di, ... of the batch at i (zero past n): all loads of a batch
+// are in flight together.
+constexpr int QU = 8;
+template <typename T>
+__device__ __forceinline__ void load_batch(T (&v)[QU], const T* a, int64_t i, int64_t di, int64_t n) {
+#pragma unroll
+    for (int u = 0; u < QU; ++u) v[u] = (i + u * di < n) ? a[i + u * di] : T(0);
+}
+// An FP64 multiply-add takes a warp 16 cycles, so the places past n are left out.
+template <typename T>
+__device__ __forceinline__ double dot_batch(const T (&a)[QU], const T (&b)[QU], int64_t i,
+                                            int64_t di, int64_t n, double s) {
+    double t = 0.0;
+#pragma unroll
+    for (int u = 0; u < QU; u += 2) {
+        if (i + u * di < n) s = fma(widen(a[u]), widen(b[u]), s);
+        if (i + (u + 1) * di < n) t = fma(widen(a[u + 1]), widen(b[u + 1]), t);
+    }
+    return s + t;
+}
+
+// One column: alpha = rho / p.q (a breakdown stops it), x += alpha p, r -= alpha q, rr and
+// the stop test.  Grid (cluster size, c).  The first batch (all of it up to 16384 rows) stays
+// in registers.
+template <typename T>
+__global__ void __launch_bounds__(QT)
+    step_kernel(T* __restrict__ x, int64_t ldx, T* __restrict__ r, int64_t ldr,
+                const T* __restrict__ p, int64_t ldp, const T* __restrict__ q, int64_t ldq,
+                int64_t n, CgScalars s) {
+    __shared__ double sh[QT];
+    __shared__ double slot[2];
+    const int k = blockIdx.y;
+    if (!s.active[k]) return;  // x and r stay; all CTAs read it before the change below
+    const double rho = s.rho[k];
+    const int64_t i0 = (int64_t)blockIdx.x * QT + threadIdx.x, di = (int64_t)gridDim.x * QT;
+    T* xk = x + (int64_t)k * ldx;
+    T* rk = r + (int64_t)k * ldr;
+    const T* pk = p + (int64_t)k * ldp;
+    const T* qk = q + (int64_t)k * ldq;
+    T pv[QU], qv[QU], rv[QU], xv[QU];
+    load_batch(pv, pk, i0, di, n);
+    load_batch(qv, qk, i0, di, n);
+    load_batch(rv, rk, i0, di, n);
+    load_batch(xv, xk, i0, di, n);
+    double v = dot_batch(pv, qv, i0, di, n, 0.0);
+    for (int64_t i = i0 + QU * di; i < n; i += QU * di) {
+        T a[QU], b[QU];
+        load_batch(a, pk, i, di, n);
+        load_batch(b, qk, i, di, n);
+        v = dot_batch(a, b, i, di, n, v);
+    }
+    v = cluster_sum(v, sh, &slot[0]);
+    const bool ok = v > 0.0 && isfinite(v) && isfinite(rho);
+    const double al = ok ? rho / v : 0.0;
+    const T a = (T)al;
+    double w = 0.0;
+    for (int64_t i = i0;;) {
+        if (al != 0.0) {
+#pragma unroll
+            for (int u = 0; u < QU; ++u) {
+                if (i + u * di < n) {
+                    rv[u] = fma(-a, qv[u], rv[u]);
+                    xk[i + u * di] = fma(a, pv[u], xv[u]);
+                    rk[i + u * di] = rv[u];
+                }
+            }
+        }
+        w = dot_batch(rv, rv, i, di, n, w);
+        i += QU * di;
+        if (i >= n) break;
+        load_batch(pv, pk, i, di, n);
+        load_batch(qv, qk, i, di, n);
+        load_batch(rv, rk, i, di, n);
+        load_batch(xv, xk, i, di, n);
+    }
+    w = cluster_sum(w, sh, &slot[1]);
+    if (blockIdx.x == 0 && threadIdx.x == 0) {
+        s.alpha[k] = al;
+        s.rr[k] = w;
+        const int it = s.iters[k];
+        s.iters[k] = ok ? it + 1 : -1 - it;  // breakdown marker
+        if (!ok) atomicAdd(&s.flags[1], 1);
+        if (!ok || w <= s.thr2[k]) {
+            s.active[k] = 0;
+            atomicSub(&s.flags[0], 1);
+        }
+    }
+    cooperative_groups::this_cluster().sync();
+}
+
+// One column: beta = r.z / rho, rho = r.z, p = z + beta p.
+template <typename T>
+__global__ void __launch_bounds__(QT)
+    direction_kernel(T* __restrict__ p, int64_t ldp, const T* __restrict__ r, int64_t ldr,
+                     const T* __restrict__ z, int64_t ldz, int64_t n, CgScalars s) {
+    __shared__ double sh[QT];
+    __shared__ double slot;
+    const int k = blockIdx.y;
+    if (!s.active[k]) return;
+    const double rho = s.rho[k];
+    const int64_t i0 = (int64_t)blockIdx.x * QT + threadIdx.x, di = (int64_t)gridDim.x * QT;
+    T* pk = p + (int64_t)k * ldp;
+    const T* rk = r + (int64_t)k * ldr;
+    const T* zk = z + (int64_t)k * ldz;
+    T zv[QU], pv[QU], rv[QU];
+    load_batch(rv, rk, i0, di, n);
+    load_batch(zv, zk, i0, di, n);
+    load_batch(pv, pk, i0, di, n);
+    double v = dot_batch(rv, zv, i0, di, n, 0.0);
+    for (int64_t i = i0 + QU * di; i < n; i += QU * di) {
+        T a[QU], b[QU];
+        load_batch(a, rk, i, di, n);
+        load_batch(b, zk, i, di, n);
+        v = dot_batch(a, b, i, di, n, v);
+    }
+    v = cluster_sum(v, sh, &slot);
+    const double be = v / rho;
+    const T b = (T)be;
+    for (int64_t i = i0;;) {
+#pragma unroll
+        for (int u = 0; u < QU; ++u)
+            if (i + u * di < n) pk[i + u * di] = fma(b, pv[u], zv[u]);
+        i += QU * di;
+        if (i >= n) break;
+        load_batch(zv, zk, i, di, n);
+        load_batch(pv, pk, i, di, n);
+    }
+    if (blockIdx.x == 0 && threadIdx.x == 0) {  // after the sum's barrier: rho has been read
+        s.beta[k] = be;
+        s.rho[k] = v;
+    }
+    cooperative_groups::this_cluster().sync();
+}
+
 template <typename T>
 __global__ void copy_cols_kernel(T* __restrict__ dst, int64_t ldd, const T* __restrict__ src,
                                  int64_t lds, int64_t n) {
@@ -229,19 +411,58 @@ void finalize(const double* partial, int nblk, int c, int mode, CgScalars s, dou
     KPCG_LAUNCHED("finalize_kernel");
 }
 
-template <typename T>
-void update_xr(T* x, int64_t ldx, T* r, int64_t ldr, const T* p, int64_t ldp, const T* q,
-               int64_t ldq, int64_t n, int c, const double* alpha, double* partial, int nblk,
-               cudaStream_t st) {
-    update_xr_kernel<T><<<dim3(nblk, c), DT, 0, st>>>(x, ldx, r, ldr, p, ldp, q, ldq, n, alpha,
-                                                      partial, nblk);
-    KPCG_LAUNCHED("update_xr_kernel");
+// Rows up to which one cluster per column beats the seven launches of the parts.  One step
+// and one direction in a graph, parts -> clusters: n = 1000 18.9 -> 10.9 us (17 columns
+// 17.9 -> 10.9), n = 4096 FP64, 17 columns 18.7 -> 15.3, n = 15000 22.0 -> 14.5 (17 columns
+// 23.2 -> 21.6), n = 32768 24.6 -> 22.3 but 17 columns 31.8 -> 33.0, n = 65536 27.7 -> 35.9:
+// eight SMs' FP64 units against all.
+constexpr int64_t kStepN = 24576;
+
+template <typename... A, typename... B>
+static void launch_clusters(void (*k)(A...), int64_t n, int c, cudaStream_t st, B... args) {
+    int cl = 1;
+    while (cl < QCL && (int64_t)cl * QT < n) cl *= 2;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((unsigned)cl, (unsigned)c);
+    cfg.blockDim = dim3(QT);
+    cfg.stream = st;
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeClusterDimension;
+    at[0].val.clusterDim.x = (unsigned)cl;
+    at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
+    cfg.attrs = at;
+    cfg.numAttrs = 1;
+    KPCG_CUDA(cudaLaunchKernelEx(&cfg, k, args...));
 }
 
 template <typename T>
-void update_p(T* p, int64_t ldp, const T* z, int64_t ldz, int64_t n, int c, const double* beta,
-              const int* active, cudaStream_t st) {
-    update_p_kernel<T><<<dim3(grid_x(n), c), 256, 0, st>>>(p, ldp, z, ldz, n, beta, active);
+void cg_step(T* x, int64_t ldx, T* r, int64_t ldr, const T* p, int64_t ldp, const T* q,
+             int64_t ldq, int64_t n, int c, CgScalars s, double* partial, int nblk,
+             cudaStream_t st) {
+    if (n <= kStepN) {
+        launch_clusters(step_kernel<T>, n, c, st, x, ldx, r, ldr, p, ldp, q, ldq, n, s);
+        KPCG_LAUNCHED("step_kernel");
+        return;
+    }
+    dot_cols<T>(p, ldp, q, ldq, n, c, partial, nblk, st);
+    finalize(partial, nblk, c, FIN_ALPHA, s, 0.0, 0, n, nullptr, st);
+    update_xr_kernel<T><<<dim3(nblk, c), DT, 0, st>>>(x, ldx, r, ldr, p, ldp, q, ldq, n, s.alpha,
+                                                      partial, nblk);
+    KPCG_LAUNCHED("update_xr_kernel");
+    finalize(partial, nblk, c, FIN_RR, s, 0.0, 0, n, nullptr, st);
+}
+
+template <typename T>
+void cg_direction(T* p, int64_t ldp, const T* r, int64_t ldr, const T* z, int64_t ldz, int64_t n,
+                  int c, CgScalars s, double* partial, int nblk, cudaStream_t st) {
+    if (n <= kStepN) {
+        launch_clusters(direction_kernel<T>, n, c, st, p, ldp, r, ldr, z, ldz, n, s);
+        KPCG_LAUNCHED("direction_kernel");
+        return;
+    }
+    dot_cols<T>(r, ldr, z, ldz, n, c, partial, nblk, st);
+    finalize(partial, nblk, c, FIN_BETA, s, 0.0, 0, n, nullptr, st);
+    update_p_kernel<T><<<dim3(grid_x(n), c), 256, 0, st>>>(p, ldp, z, ldz, n, s.beta, s.active);
     KPCG_LAUNCHED("update_p_kernel");
 }
 
@@ -284,16 +505,14 @@ template void dot_cols<float>(const float*, int64_t, const float*, int64_t, int6
                               int, cudaStream_t);
 template void dot_cols<double>(const double*, int64_t, const double*, int64_t, int64_t, int,
                                double*, int, cudaStream_t);
-template void update_xr<float>(float*, int64_t, float*, int64_t, const float*, int64_t,
-                               const float*, int64_t, int64_t, int, const double*, double*, int,
-                               cudaStream_t);
-template void update_xr<double>(double*, int64_t, double*, int64_t, const double*, int64_t,
-                                const double*, int64_t, int64_t, int, const double*, double*, int,
-                                cudaStream_t);
-template void update_p<float>(float*, int64_t, const float*, int64_t, int64_t, int,
-                              const double*, const int*, cudaStream_t);
-template void update_p<double>(double*, int64_t, const double*, int64_t, int64_t, int,
-                               const double*, const int*, cudaStream_t);
+template void cg_step<float>(float*, int64_t, float*, int64_t, const float*, int64_t, const float*, int64_t,
+                             int64_t, int, CgScalars, double*, int, cudaStream_t);
+template void cg_direction<float>(float*, int64_t, const float*, int64_t, const float*, int64_t, int64_t, int,
+                                  CgScalars, double*, int, cudaStream_t);
+template void cg_step<double>(double*, int64_t, double*, int64_t, const double*, int64_t, const double*, int64_t,
+                             int64_t, int, CgScalars, double*, int, cudaStream_t);
+template void cg_direction<double>(double*, int64_t, const double*, int64_t, const double*, int64_t, int64_t, int,
+                                  CgScalars, double*, int, cudaStream_t);
 template void copy_cols<float>(float*, int64_t, const float*, int64_t, int64_t, int, cudaStream_t);
 template void copy_cols<double>(double*, int64_t, const double*, int64_t, int64_t, int,
                                 cudaStream_t);

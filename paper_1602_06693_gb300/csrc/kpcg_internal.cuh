@@ -136,13 +136,15 @@ void dot_cols(const T* A, int64_t lda, const T* B, int64_t ldb, int64_t n, int c
 // Reduce partial dots and run the per-column scalar logic of Algorithm 1.
 void finalize(const double* partial, int nblk, int c, int mode, CgScalars s, double tol,
               int tol_mode, int64_t n, int* host_flags, cudaStream_t st);
+// alpha, x, r, ||r||^2 and the stop test (FIN_ALPHA, FIN_RR) after q = A p, and beta, rho, p
+// (FIN_BETA) after z = P^-1 r.
 template <typename T>
-void update_xr(T* x, int64_t ldx, T* r, int64_t ldr, const T* p, int64_t ldp, const T* q,
-               int64_t ldq, int64_t n, int c, const double* alpha, double* partial, int nblk,
-               cudaStream_t st);
+void cg_step(T* x, int64_t ldx, T* r, int64_t ldr, const T* p, int64_t ldp, const T* q,
+             int64_t ldq, int64_t n, int c, CgScalars s, double* partial, int nblk,
+             cudaStream_t st);
 template <typename T>
-void update_p(T* p, int64_t ldp, const T* z, int64_t ldz, int64_t n, int c, const double* beta,
-              const int* active, cudaStream_t st);
+void cg_direction(T* p, int64_t ldp, const T* r, int64_t ldr, const T* z, int64_t ldz, int64_t n,
+                  int c, CgScalars s, double* partial, int nblk, cudaStream_t st);
 template <typename T>
 void copy_cols(T* dst, int64_t ldd, const T* src, int64_t lds, int64_t n, int c, cudaStream_t st);
 template <typename TD, typename TS>
