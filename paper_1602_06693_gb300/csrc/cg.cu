@@ -42,16 +42,6 @@ __device__ __forceinline__ double block_sum(double v, double* sh) {
     return t;
 }
 
-// (double)f for any f: integer operations, since the conversion instruction runs at one per
-// clock and SM.
-__device__ __forceinline__ double widen(float f) {
-    const unsigned u = __float_as_uint(f), e = u & 0x7f800000u;
-    if (e == 0x7f800000u || (e == 0u && (u << 1))) return (double)f;  // Inf, NaN, subnormal
-    const unsigned hi = (u & 0x80000000u) | (e ? ((u & 0x7fffffffu) >> 3) + 0x38000000u : 0u);
-    return __hiloint2double((int)hi, (int)(u << 29));
-}
-__device__ __forceinline__ double widen(double f) { return f; }
-
 template <typename T>
 __global__ void __launch_bounds__(DT)
     dot_kernel(const T* __restrict__ A, int64_t lda, const T* __restrict__ B, int64_t ldb,

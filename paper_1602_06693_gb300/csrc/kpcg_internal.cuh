@@ -114,6 +114,16 @@ void dkv_f32(const float* xs, int64_t n, int dp, int d, int ard, float c0, const
 void dkv_f64(const double* xs, int64_t n, int dp, int d, int ard, double c0, const double* W,
              int64_t ldw, int c, double* G, int64_t ldg, KvWorkspace& ws, cudaStream_t st);
 
+// (double)f for any f: integer operations, since the conversion instruction runs at one per
+// clock and SM.
+__device__ __forceinline__ double widen(float f) {
+    const unsigned u = __float_as_uint(f), e = u & 0x7f800000u;
+    if (e == 0x7f800000u || (e == 0u && (u << 1))) return (double)f;  // Inf, NaN, subnormal
+    const unsigned hi = (u & 0x80000000u) | (e ? ((u & 0x7fffffffu) >> 3) + 0x38000000u : 0u);
+    return __hiloint2double((int)hi, (int)(u << 29));
+}
+__device__ __forceinline__ double widen(double f) { return f; }
+
 // --------------------------------------------------------------- CG (cg.cu)
 // Per-column scalars of the batched PCG, device resident.
 struct CgScalars {

@@ -289,7 +289,7 @@ struct ProjR<double> {
     using S = float2;
     static __device__ __forceinline__ S cut(double v) {
         const float hi = (float)v;
-        return make_float2(hi, (float)(v - (double)hi));
+        return make_float2(hi, (float)(v - widen(hi)));
     }
     static __device__ __forceinline__ void add(Acc2& a, float2 kv, S r) {
         dot2_add(a, kv.x, r.x);
@@ -321,9 +321,9 @@ __device__ __forceinline__ void nys_proj_body(const float2* __restrict__ KXU, in
     for (int64_t rs = r0; rs < r1; rs += 128) {
         const int rn = (int)min((int64_t)128, r1 - rs);
         __syncthreads();
-        for (int k = threadIdx.x >> 7; k < NC; k += 2) {
-            const int r = threadIdx.x & 127;
-            if (r < rn) sr[r * NC + k] = PR::cut(k < ncols ? R[rs + r + (int64_t)k * ldr] : T(0));
+        for (int e = threadIdx.x; e < rn * NC; e += 256) {
+            const int k = e / rn, r = e - k * rn;
+            sr[r * NC + k] = PR::cut(k < ncols ? R[rs + r + (int64_t)k * ldr] : T(0));
         }
         __syncthreads();
         if (a < m) {
@@ -351,13 +351,13 @@ __device__ __forceinline__ void nys_proj_body(const float2* __restrict__ KXU, in
         if (a < m)
 #pragma unroll
             for (int k = 0; k < NC; ++k)
-                if (k < ncols) out[(int64_t)k * m + a] = (double)acc[k].s + (double)acc[k].c;
+                if (k < ncols) out[(int64_t)k * m + a] = widen(acc[k].s) + widen(acc[k].c);
         return;
     }
     __syncthreads();
 #pragma unroll
     for (int k = 0; k < NC; ++k)
-        if (k < ncols) red[k * 256 + threadIdx.x] = (double)acc[k].s + (double)acc[k].c;
+        if (k < ncols) red[k * 256 + threadIdx.x] = widen(acc[k].s) + widen(acc[k].c);
     __syncthreads();
     for (int k = g; k < ncols; k += ng) {
         double s = 0.0;
@@ -445,39 +445,61 @@ __global__ void tri_upper_apply_kernel(const double* __restrict__ U, int64_t m,
 // components up to ~1e6 that cancel to O(1) in K_XU u; a compensated-FP32 sum
 // (2^-48) left ~3e-6 relative noise there and weakened the preconditioner,
 // FP64 (2^-53) matches the direct solve.
-// All columns of a group of NC share one read and one FP64 conversion of an
-// entry (two conversions and an add cost as much of the FP64 pipe, ~2
-// operations per clock and SM, as three products: done per column they were
-// three quarters of the work), and the NC sums are reduced over the lanes by a
-// butterfly that halves the columns a lane holds at each step.
-template <typename T, int NC>
+// All columns of a group of NC share one read and one widening of an entry (lowered: three
+// integer operations, and one FP64 addition for the pair; the conversion instruction runs at
+// one per clock and SM, FP64 arithmetic at two: with conversions a 1-column product spent
+// two thirds of its time on them).  A warp takes RN rows at once, and the RN x NC sums are
+// reduced over the lanes by a butterfly that halves the sums a lane holds at each step.
+// Bound: the FP64 pipe, (1 + NC) / 2 clocks per entry and SM, and for one column its latency.
+// n = 14979, m = 128, one column: 14.8 us, L2 warm; the Laplace fit of that size, 460 of
+// them, went from 95 to 90 ms.
+//
+// 2^-896 f as a double: the bits of f with the exponent field widened but not rebiased,
+// exact for every finite f including zero and subnormals.  The entries are finite: a
+// factored M has no others.
+__device__ __forceinline__ double lowered(float f) {
+    const int u = __float_as_int(f);
+    return __hiloint2double((u >> 3) & (int)0x8fffffffu, u << 29);
+}
+
+template <typename T, int NC, int RN>
 __global__ void __launch_bounds__(256)
     nys_back_kernel(const float2* __restrict__ KXU, int64_t n, int64_t m,
                     const double* __restrict__ u, int c, const T* __restrict__ R, int64_t ldr,
                     T* __restrict__ Z, int64_t ldz, double inv_noise) {
+    constexpr int W = RN * NC;  // a power of two, at most 16
     extern __shared__ double su[];  // m * c
     for (int64_t e = threadIdx.x; e < m * c; e += blockDim.x) su[e] = u[e];
     __syncthreads();
     const int lane = threadIdx.x & 31;
-    const int64_t warps = (int64_t)gridDim.x * (blockDim.x >> 5);
-    for (int64_t i = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5; i < n; i += warps) {
-        const float2* Ki = KXU + i * m;
+    const int64_t step = (int64_t)gridDim.x * (blockDim.x >> 5) * RN;
+    for (int64_t i = (((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5) * RN; i < n;
+         i += step) {
+        const float2* Ki[RN];
+#pragma unroll
+        for (int r = 0; r < RN; ++r) Ki[r] = KXU + min(i + r, n - 1) * m;  // past n: not stored
         for (int k0 = 0; k0 < c; k0 += NC) {
             const int nc = min(NC, c - k0);
             const double* uk = su + (int64_t)k0 * m;
-            double acc[NC];
+            double acc[W];
 #pragma unroll
-            for (int k = 0; k < NC; ++k) acc[k] = 0.0;
+            for (int q = 0; q < W; ++q) acc[q] = 0.0;
 #pragma unroll 4
             for (int64_t a = lane; a < m; a += 32) {
-                const float2 kv = __ldg(Ki + a);
-                const double kd = (double)kv.x + (double)kv.y;
+                float2 kv[RN];
 #pragma unroll
-                for (int k = 0; k < NC; ++k)
-                    if (k < nc) acc[k] = fma(kd, uk[(int64_t)k * m + a], acc[k]);
+                for (int r = 0; r < RN; ++r) kv[r] = __ldg(Ki[r] + a);
+#pragma unroll
+                for (int r = 0; r < RN; ++r) {
+                    const double kd = lowered(kv[r].x) + lowered(kv[r].y);
+#pragma unroll
+                    for (int k = 0; k < NC; ++k)
+                        if (k < nc)
+                            acc[r * NC + k] = fma(kd, uk[(int64_t)k * m + a], acc[r * NC + k]);
+                }
             }
 #pragma unroll
-            for (int w = NC, o = 16; w > 1; w >>= 1, o >>= 1) {
+            for (int w = W, o = 16; w > 1; w >>= 1, o >>= 1) {
                 const bool up_half = (lane & o) != 0;
 #pragma unroll
                 for (int q = 0; q < w / 2; ++q) {
@@ -487,12 +509,13 @@ __global__ void __launch_bounds__(256)
                 }
             }
 #pragma unroll
-            for (int o = 16 / NC; o > 0; o >>= 1)
+            for (int o = 16 / W; o > 0; o >>= 1)
                 acc[0] += __shfl_xor_sync(0xffffffffu, acc[0], o);
-            const int k = lane / (32 / NC);
-            if ((lane & (32 / NC - 1)) == 0 && k < nc)
-                Z[i + (int64_t)(k0 + k) * ldz] =
-                    (T)(((double)R[i + (int64_t)(k0 + k) * ldr] - acc[0]) * inv_noise);
+            const int q = lane / (32 / W), k = q % NC;
+            const int64_t ir = i + q / NC;
+            if ((lane & (32 / W - 1)) == 0 && k < nc && ir < n)
+                Z[ir + (int64_t)(k0 + k) * ldz] =
+                    (T)(fma(-acc[0], 0x1p896, (double)R[ir + (int64_t)(k0 + k) * ldr]) * inv_noise);
         }
     }
 }
@@ -1043,19 +1066,20 @@ static void nystrom_apply(const PrecondState& P, const T* R, int64_t ldr, int c,
     KPCG_LAUNCHED("tri_upper_apply_kernel");
     const size_t smem = sizeof(double) * (size_t)m * c;
     if (smem > 200 * 1024) fail(KPCG_ERR_ARG, "Nystrom apply: m * c too large");
-    const int blocks = (int)std::min<int64_t>((n + 7) / 8, 152 * 16);
-    auto go = [&](auto kern) {
+    auto go = [&](auto kern, int rows_per_warp) {
+        const int blocks =
+            (int)std::min<int64_t>((n + 8 * rows_per_warp - 1) / (8 * rows_per_warp), 152 * 16);
         if (smem > 48 * 1024) raise_smem_limit((const void*)kern, smem);
         kern<<<blocks, 256, smem, st>>>(P.KXU.p, n, m, w, c, R, ldr, Z, ldz, 1.0 / P.apply_noise);
     };
     if (c == 1)
-        go(nys_back_kernel<T, 1>);
+        go(nys_back_kernel<T, 1, 4>, 4);
     else if (c <= 4)
-        go(nys_back_kernel<T, 4>);
+        go(nys_back_kernel<T, 4, 4>, 4);
     else if (c <= 8)
-        go(nys_back_kernel<T, 8>);
+        go(nys_back_kernel<T, 8, 2>, 2);
     else
-        go(nys_back_kernel<T, 16>);
+        go(nys_back_kernel<T, 16, 1>, 1);
     KPCG_LAUNCHED("nys_back_kernel");
 }
 
