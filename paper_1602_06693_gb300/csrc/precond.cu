@@ -58,91 +58,123 @@ __device__ __forceinline__ int64_t bsize(int64_t q, int64_t b, int64_t n_total) 
     return (n_total - r0 < b) ? (n_total - r0) : b;
 }
 
+// The 32 x 32 kernels below are chains of FP64 operations, and an FP64 instruction of a warp
+// holds the FP64 unit of its SM quarter for 64 cycles, however few lanes it is for.  So a
+// CTA has four warps, one per quarter; a row of 32 values is spread over four lanes,
+// value u with lane u % 4, so that an update of a row's rest is at most eight instructions
+// for eight rows; and quotients are x (1/d) with one correction instead of a division each.
+// m = 1024, per panel of 32: diagonal block 45 -> 31 us, panel solve 41 -> 17 us; L^{-T} by
+// panels 1.2 ms, by a warp per column 3.0 ms.
+
+// x / d given inv = 1 / d
+__device__ __forceinline__ double div_by(double x, double d, double inv) {
+    const double q = x * inv;
+    return fma(fma(-q, d, x), inv, q);
+}
+
 // Factor the nb x nb diagonal block at (j0, j0) of matrix q in place; a pivot
 // not above thr fails the factorization.
-__global__ void potrf_diag_kernel(double* A, int64_t stride, int64_t b, int64_t n_total,
-                                  int64_t j0, int* status, double thr) {
+__global__ void __launch_bounds__(128)
+    potrf_diag_kernel(double* A, int64_t stride, int64_t b, int64_t n_total, int64_t j0,
+                      int* status, double thr) {
     __shared__ double S[NB][NB + 1];
-    __shared__ int bad;
     const int64_t q = blockIdx.x;
     const int64_t bq = bsize(q, b, n_total);
     if (j0 >= bq || status[q]) return;
     const int nb = (int)min((int64_t)NB, bq - j0);
-    double* M = A + q * stride;
-    const int64_t ld = bq;
-    for (int e = threadIdx.x; e < nb * nb; e += blockDim.x) {
-        const int r = e / nb, c = e % nb;
-        S[r][c] = M[(j0 + r) * ld + j0 + c];
+    double* M = A + q * stride + j0 * bq + j0;
+    for (int e = threadIdx.x; e < NB * NB; e += 128) {
+        const int r = e / NB, c = e % NB;  // the identity past nb
+        S[r][c] = (r < nb && c < nb) ? M[r * bq + c] : (r == c ? 1.0 : 0.0);
     }
-    if (threadIdx.x == 0) bad = 0;
     __syncthreads();
-    for (int j = 0; j < nb; ++j) {
-        if (threadIdx.x == 0) {
-            const double piv = S[j][j];
-            if (!(piv > thr) || !isfinite(piv)) {
-                bad = 1;
-            } else {
-                S[j][j] = sqrt(piv);
-            }
-        }
-        __syncthreads();
-        if (bad) {
+    const int row = threadIdx.x >> 2, part = threadIdx.x & 3;
+    double x[NB / 4];
+#pragma unroll
+    for (int v = 0; v < NB / 4; ++v) x[v] = S[row][4 * v + part];
+#pragma unroll
+    for (int j = 0; j < NB; ++j) {
+        // column j of rows >= j is final in S
+        const double piv = S[j][j];
+        if (j < nb && (!(piv > thr) || !isfinite(piv))) {
             if (threadIdx.x == 0) status[q] = (int)(j0 + j + 1);
             return;
         }
-        const double ljj = S[j][j];
-        for (int i = j + 1 + threadIdx.x; i < nb; i += blockDim.x) S[i][j] /= ljj;
+        const double inv = rsqrt(piv);
+        double d = piv * inv;
+        d = fma(fma(-d, d, piv), 0.5 * inv, d);  // sqrt(piv)
+        const double l = row > j ? div_by(S[row][j], d, inv) : d;
         __syncthreads();
-        for (int e = threadIdx.x; e < nb * nb; e += blockDim.x) {
-            const int i = e / nb, k = e % nb;
-            if (i > j && k > j && k <= i) S[i][k] -= S[i][j] * S[k][j];
+        if (part == 0 && row >= j) S[row][j] = l;
+        __syncthreads();
+#pragma unroll
+        for (int v = 0; v < NB / 4; ++v) {
+            const int k = 4 * v + part;
+            if (4 * v + 3 > j) {
+                if (k > j) x[v] -= l * S[k][j];  // used where row >= k
+                if (k == j + 1) S[row][k] = x[v];
+            }
         }
         __syncthreads();
     }
-    for (int e = threadIdx.x; e < nb * nb; e += blockDim.x) {
+    for (int e = threadIdx.x; e < nb * nb; e += 128) {
         const int r = e / nb, c = e % nb;
-        M[(j0 + r) * ld + j0 + c] = (c <= r) ? S[r][c] : 0.0;
+        M[r * bq + c] = (c <= r) ? S[r][c] : 0.0;
     }
 }
 
-// Panel solve: rows i >= j0+nb of columns j0..j0+nb-1 become L21 = A21 L11^{-T}.
-__global__ void trsm_panel_kernel(double* A, int64_t stride, int64_t b, int64_t n_total,
-                                  int64_t j0, const int* status) {
+// X <- X L11^{-T} for rows of 32 values at column j0: the panel below the diagonal block
+// (rows j0 + nb .. of A, U = null), or the rows 0 .. j0 + nb - 1 of U on their way to L^{-T}.
+// A CTA takes 32 rows; a solved value is taken out of all later ones at once, so that the
+// multiply-adds do not wait for one another.
+__global__ void __launch_bounds__(128)
+    trsm_panel_kernel(double* A, double* U, int64_t stride, int64_t b, int64_t n_total,
+                      int64_t j0, const int* status) {
     __shared__ double L[NB][NB + 1];
-    const int64_t q = blockIdx.y;
+    __shared__ double X[NB][NB + 1];
+    __shared__ double inv[NB];
+    const int64_t q = blockIdx.x;  // there may be more matrices than a grid has rows
     const int64_t bq = bsize(q, b, n_total);
     if (j0 >= bq || status[q]) return;
     const int nb = (int)min((int64_t)NB, bq - j0);
-    double* M = A + q * stride;
-    const int64_t ld = bq;
-    for (int e = threadIdx.x; e < nb * nb; e += blockDim.x) {
-        const int r = e / nb, c = e % nb;
-        L[r][c] = M[(j0 + r) * ld + j0 + c];
+    const double* M = A + q * stride + j0 * bq + j0;
+    const int64_t i0 = (U ? 0 : j0 + nb) + (int64_t)blockIdx.y * 32, i1 = U ? j0 + nb : bq;
+    if (i0 >= i1) return;
+    double* G = (U ? U : A) + q * stride + i0 * bq + j0;
+    const int nr = (int)min((int64_t)32, i1 - i0);
+    for (int e = threadIdx.x; e < NB * NB; e += 128) {
+        const int r = e / NB, c = e % NB;
+        L[r][c] = (r < nb && c < nb) ? M[r * bq + c] : (r == c ? 1.0 : 0.0);
+        X[r][c] = (r < nr && c < nb) ? G[r * bq + c] : 0.0;
     }
     __syncthreads();
-    const int64_t i = j0 + nb + (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= bq) return;
-    double x[NB];
+    if (threadIdx.x < NB) inv[threadIdx.x] = 1.0 / L[threadIdx.x][threadIdx.x];
+    __syncthreads();
+    const int row = threadIdx.x >> 2, part = threadIdx.x & 3;
+    double x[NB / 4];
 #pragma unroll
-    for (int t = 0; t < NB; ++t) x[t] = (t < nb) ? M[i * ld + j0 + t] : 0.0;
+    for (int v = 0; v < NB / 4; ++v) x[v] = X[row][4 * v + part];
 #pragma unroll
     for (int t = 0; t < NB; ++t) {
-        if (t < nb) {
-            double s = x[t];
+        const double xt = div_by(__shfl_sync(0xffffffffu, x[t / 4], t % 4, 4), L[t][t], inv[t]);
+        if (part == t % 4) x[t / 4] = xt;
 #pragma unroll
-            for (int u = 0; u < NB; ++u)
-                if (u < t) s -= x[u] * L[t][u];
-            x[t] = s / L[t][t];
-        }
+        for (int v = 0; v < NB / 4; ++v)
+            if (4 * v + 3 > t && 4 * v + part > t) x[v] -= xt * L[4 * v + part][t];
     }
 #pragma unroll
-    for (int t = 0; t < NB; ++t)
-        if (t < nb) M[i * ld + j0 + t] = x[t];
+    for (int v = 0; v < NB / 4; ++v) X[row][4 * v + part] = x[v];
+    __syncthreads();
+    for (int e = threadIdx.x; e < NB * NB; e += 128) {
+        const int r = e / NB, c = e % NB;
+        if (r < nr && c < nb) G[r * bq + c] = X[r][c];
+    }
 }
 
-// Trailing update A22 -= L21 L21^T on the lower triangle; 32x32 output tiles.
-__global__ void syrk_update_kernel(double* A, int64_t stride, int64_t b, int64_t n_total,
-                                   int64_t j0, const int* status) {
+// Trailing update A22 -= L21 L21^T on the lower triangle, or (U given) U2 -= U1 L21^T for the
+// rows 0 .. j0 + nb - 1 of U; 32x32 output tiles.
+__global__ void panel_update_kernel(double* A, double* U, int64_t stride, int64_t b,
+                                    int64_t n_total, int64_t j0, const int* status) {
     __shared__ double Li[32][NB + 1];
     __shared__ double Lk[32][NB + 1];
     const int64_t q = blockIdx.z;
@@ -151,14 +183,15 @@ __global__ void syrk_update_kernel(double* A, int64_t stride, int64_t b, int64_t
     const int nb = (int)min((int64_t)NB, bq - j0);
     const int64_t t0 = j0 + nb;
     const int64_t ti = blockIdx.y, tk = blockIdx.x;
-    if (tk > ti) return;
-    const int64_t i0 = t0 + ti * 32, k0 = t0 + tk * 32;
-    if (i0 >= bq) return;
+    if (!U && tk > ti) return;
+    const int64_t i0 = (U ? 0 : t0) + ti * 32, k0 = t0 + tk * 32, i1 = U ? t0 : bq;
+    if (i0 >= i1 || k0 >= bq) return;
     double* M = A + q * stride;
+    double* X = (U ? U : A) + q * stride;
     const int64_t ld = bq;
     for (int e = threadIdx.x; e < 32 * NB; e += blockDim.x) {
         const int r = e / NB, c = e % NB;
-        Li[r][c] = (i0 + r < bq && c < nb) ? M[(i0 + r) * ld + j0 + c] : 0.0;
+        Li[r][c] = (i0 + r < i1 && c < nb) ? X[(i0 + r) * ld + j0 + c] : 0.0;
         Lk[r][c] = (k0 + r < bq && c < nb) ? M[(k0 + r) * ld + j0 + c] : 0.0;
     }
     __syncthreads();
@@ -169,38 +202,21 @@ __global__ void syrk_update_kernel(double* A, int64_t stride, int64_t b, int64_t
         for (int c2 = 0; c2 < 2; ++c2) {
             const int r = ty * 2 + a, cc = tx * 2 + c2;
             const int64_t i = i0 + r, k = k0 + cc;
-            if (i < bq && k < bq && k <= i) {
+            if (i < i1 && k < bq && (U || k <= i)) {
                 double s = 0.0;
 #pragma unroll
                 for (int u = 0; u < NB; ++u) s = fma(Li[r][u], Lk[cc][u], s);
-                M[i * ld + k] -= s;
+                X[i * ld + k] -= s;
             }
         }
 }
 
-// U = L^{-T}: warp w solves L x = e_j for column j, writing x into row j of U.
-__global__ void trinv_kernel(const double* Lb, double* Ub, int64_t stride, int64_t b,
-                             int64_t n_total, int64_t nmat) {
-    const int64_t gw = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-    const int lane = threadIdx.x & 31;
-    // Flat column index over the batch: matrix q holds columns [q*b, q*b+bq).
-    const int64_t q = gw / b, j = gw % b;
+__global__ void identity_kernel(double* U, int64_t b, int64_t n_total, int64_t nmat) {
+    const int64_t g = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    const int64_t q = g / (b * b), e = g - q * b * b;
     if (q >= nmat) return;
     const int64_t bq = bsize(q, b, n_total);
-    if (j >= bq) return;
-    const double* L = Lb + q * stride;
-    double* U = Ub + q * stride + j * bq;  // row j of U
-    for (int64_t i = lane; i < j; i += 32) U[i] = 0.0;
-    if (lane == 0) U[j] = 1.0 / L[j * bq + j];
-    __syncwarp();
-    for (int64_t i = j + 1; i < bq; ++i) {
-        const double* Li = L + i * bq;
-        double s = 0.0;
-        for (int64_t k = j + lane; k < i; k += 32) s = fma(Li[k], U[k], s);
-        s = warp_sum(s);
-        if (lane == 0) U[i] = -s / Li[i];
-        __syncwarp();
-    }
+    if (e < bq * bq) U[g] = e % (bq + 1) == 0 ? 1.0 : 0.0;
 }
 
 // ---------------------------------------------------------------- Nystrom
@@ -580,18 +596,18 @@ static int factor_and_invert(double* A, double* U, int64_t b, int64_t n_total, i
                              int* status_dev, cudaStream_t st, double thr = 0.0) {
     KPCG_CUDA(cudaMemsetAsync(status_dev, 0, sizeof(int) * nmat, st));
     for (int64_t j0 = 0; j0 < b; j0 += NB) {
-        potrf_diag_kernel<<<(unsigned)nmat, 256, 0, st>>>(A, b * b, b, n_total, j0, status_dev,
+        potrf_diag_kernel<<<(unsigned)nmat, 128, 0, st>>>(A, b * b, b, n_total, j0, status_dev,
                                                           thr);
         KPCG_LAUNCHED("potrf_diag_kernel");
         const int64_t rows = b - j0 - NB;
         if (rows > 0) {
-            dim3 g1((unsigned)((rows + 127) / 128), (unsigned)nmat);
-            trsm_panel_kernel<<<g1, 128, 0, st>>>(A, b * b, b, n_total, j0, status_dev);
+            dim3 g1((unsigned)nmat, (unsigned)((rows + 31) / 32));
+            trsm_panel_kernel<<<g1, 128, 0, st>>>(A, nullptr, b * b, b, n_total, j0, status_dev);
             KPCG_LAUNCHED("trsm_panel_kernel");
             const unsigned nt = (unsigned)((rows + 31) / 32);
             dim3 g2(nt, nt, (unsigned)nmat);
-            syrk_update_kernel<<<g2, 256, 0, st>>>(A, b * b, b, n_total, j0, status_dev);
-            KPCG_LAUNCHED("syrk_update_kernel");
+            panel_update_kernel<<<g2, 256, 0, st>>>(A, nullptr, b * b, b, n_total, j0, status_dev);
+            KPCG_LAUNCHED("panel_update_kernel");
         }
     }
     std::vector<int> hs((size_t)nmat);
@@ -600,10 +616,21 @@ static int factor_and_invert(double* A, double* U, int64_t b, int64_t n_total, i
     KPCG_CUDA(cudaStreamSynchronize(st));
     for (int64_t q = 0; q < nmat; ++q)
         if (hs[(size_t)q]) return hs[(size_t)q] + (int)(q * b);
-    const int64_t warps = nmat * b;
-    trinv_kernel<<<(unsigned)((warps * 32 + 255) / 256), 256, 0, st>>>(A, U, b * b, b, n_total,
-                                                                      nmat);
-    KPCG_LAUNCHED("trinv_kernel");
+    // U = L^{-T}: the identity's rows go through the same panels
+    identity_kernel<<<(unsigned)((nmat * b * b + 255) / 256), 256, 0, st>>>(U, b, n_total, nmat);
+    KPCG_LAUNCHED("identity_kernel");
+    for (int64_t j0 = 0; j0 < b; j0 += NB) {
+        const unsigned nr = (unsigned)(std::min(j0 + NB, b) + 31) / 32;
+        trsm_panel_kernel<<<dim3((unsigned)nmat, nr), 128, 0, st>>>(A, U, b * b, b, n_total, j0,
+                                                                   status_dev);
+        KPCG_LAUNCHED("trsm_panel_kernel");
+        const int64_t rows = b - j0 - NB;
+        if (rows > 0) {
+            panel_update_kernel<<<dim3((unsigned)((rows + 31) / 32), nr, (unsigned)nmat), 256, 0,
+                                  st>>>(A, U, b * b, b, n_total, j0, status_dev);
+            KPCG_LAUNCHED("panel_update_kernel");
+        }
+    }
     return 0;
 }
 
