@@ -5,7 +5,7 @@ Workload (one "step"): the ARD-RBF system (K + sigma^2 I) alpha = y with
 n = 65536, d = 8, X ~ U[0,1]^8, l_r ~ LogUniform(0.3, 3), s = 1, sigma^2 = 1e-4
 (seeded, synthetic), Nystrom preconditioner with m = 1024 random inducing
 points built inside the step, solved to ||y - K_y alpha|| <= 1e-8 ||y||
-(recomputed in native FP64) by the mixed-precision solver: flexible CG in FP64
+(recomputed with FP64 accuracy) by the mixed-precision solver: flexible CG in FP64
 (double-float direction products, FP64 certified residuals) around an inner
 FP32 PCG with the tensor-core K.V (--precision selects another mode).  Inputs
 are resident in HBM when the timed region starts; L2 is flushed between steps.
@@ -44,7 +44,7 @@ METRIC = "PCG time-to-rel-res 1e-8 at n=65k vs plain FP32; K.V TFLOP/s vs roofli
 WORKLOAD = ("ARD-RBF n=65536 d=8 X~U[0,1]^8 l~LogU(0.3,3) s=1 noise=1e-4, y=sum sin(x)+N(0,0.01); "
             "Nystrom m=1024 built in-step; tol 1e-8 rel; 1 RHS")
 # The headline solver: flexible CG in FP64 (double-float outer directions,
-# native-FP64 certified residuals) around an inner FP32 PCG whose K.V runs on
+# FP64-accurate certified residuals) around an inner FP32 PCG whose K.V runs on
 # the tensor cores, on the operator shifted by inner_shift * sigma^2.  The
 # shift and inner tolerance were picked by the sweep that
 # `--workload precision` runs.
@@ -136,11 +136,12 @@ def df_issue_efficiency(n, d, c, ms, rates):
 
 
 def df_kernel_name(d):
-    """The double-float product's kernel at dimension d (the tensor-core
+    """The one-column double-float product's kernel at dimension d (the tensor-core
     distances of kv_tcds_kernel, one evaluation per pair of points, up to
-    d = 10; the FP32-pipe kernel above)."""
+    d = 10; above it, and for three or more columns, the FP64-class
+    fixed-point kernel up to d = 16)."""
     return ("kv_tcds_kernel (double-float, tensor-core distances, symmetric)" if d <= 10 else
-            "kv_df_sym_kernel (double-float)")
+            FX_NAME if d <= 16 else "kv_df_sym_kernel (double-float)")
 
 
 def df_issue_eff(n, d, c, ms, rates, symmetric=True):
@@ -701,8 +702,9 @@ def run_laplace(args):
     rates = probed_rates(kpcg)
     roof = alu_roofline(df_kernel_name(p.d) + ", 1 column", p.n, p.d, 1, kv_ms, rates)
     roof.update({"traffic": None, "peak_source": PEAK_SOURCE,
-                 "timing": f"{reps} back-to-back products, CUDA events on the launching stream",
-                 "issue_efficiency": df_issue_eff(p.n, p.d, 1, kv_ms, rates)})
+                 "timing": f"{reps} back-to-back products, CUDA events on the launching stream"})
+    if p.d <= 10:
+        roof["issue_efficiency"] = df_issue_eff(p.n, p.d, 1, kv_ms, rates)
     # the inner product of the mixed B-solves: tensor-core K.V of one column
     roof_inner = None
     if prec == kpcg.KPCG_TC_IR:
@@ -966,10 +968,13 @@ DTYPES = {"tc_ir": "bf16x3 exponent, f32 inner, f64 outer (double-float directio
           "fp32_ir": "f32 inner, f64 outer", "xf_ir": "f32 inner (exact differences), f64 outer",
           "tcx_ir": "sliced bf16 exponent, f32 inner, f64 outer",
           "df64": "double-float iterations, fp64 certified residual", "fp64": "f64"}
+# the FP64-class product for d <= 16 (its distances and contraction run on the tensor cores,
+# so it is held against the tensor/MUFU bound, not the FP64 pipe)
+FX_NAME = "kv_fx_kernel (FP64 class, fixed point on the tensor cores)"
 KV_NAMES = {"tc_ir": "kv_tcs_kernel (tcgen05 exponent, symmetric tile pairs)",
             "tcx_ir": "kv_tcx_kernel (tcgen05 sliced exponent, compensated contraction)",
             "fp32_ir": "kv_simt_kernel<float>", "xf_ir": "kv_xf_sym_kernel (exact differences)",
-            "df64": df_kernel_name(D), "fp64": "kv_f64_sym_kernel (FP64)"}
+            "df64": df_kernel_name(D), "fp64": FX_NAME}
 # DRAM bytes per launch from ncu captures at n = 16384, by kernel
 # name, as a function of n: each kernel reads only its inputs from DRAM (the
 # n x n work stays on chip), so the traffic grows like n.  A kernel changed
@@ -1061,8 +1066,7 @@ def run_solve(args):
     cats = {}
     if pinfo.kv_inner_calls:
         ms = pinfo.kv_inner_ms / pinfo.kv_inner_calls
-        cats["kv_inner"] = alu_roofline(KV_NAMES[mode], p.n, D, 1, ms, rates,
-                                        fp64=(mode == "fp64"))
+        cats["kv_inner"] = alu_roofline(KV_NAMES[mode], p.n, D, 1, ms, rates)
         cats["kv_inner"].update(calls=pinfo.kv_inner_calls, total_ms=pinfo.kv_inner_ms)
         if mode == "df64":
             cats["kv_inner"]["issue_efficiency"] = df_issue_eff(p.n, D, 1, ms, rates)
@@ -1074,8 +1078,7 @@ def run_solve(args):
                                 issue_efficiency=df_issue_eff(p.n, D, 1, ms, rates))
     if pinfo.resid_calls:
         ms = pinfo.resid_ms / pinfo.resid_calls
-        cats["resid"] = alu_roofline("kv_f64_sym_kernel (native FP64 certified residual)",
-                                     p.n, D, 1, ms, rates, fp64=True)
+        cats["resid"] = alu_roofline(FX_NAME + " (certified residual)", p.n, D, 1, ms, rates)
         cats["resid"].update(calls=pinfo.resid_calls, total_ms=pinfo.resid_ms)
     if pinfo.precond_calls:
         ms = pinfo.precond_ms / pinfo.precond_calls
@@ -1207,7 +1210,7 @@ def comparisons(kpcg, X, y, p, idx, stream, mode, extra_opts, args):
     return out
 
 
-KV_IMPLS = {"f64": ("f64", 0, "kv_f64_sym_kernel (native FP64)"),
+KV_IMPLS = {"f64": ("f64", 0, FX_NAME),
             "df": ("f64", 1, "kv_tcds_kernel (double-float, tensor-core distances, symmetric)"),
             "df1": ("f64", 4, "kv_tcd_kernel (double-float, tensor-core distances, every entry)"),
             "dfs": ("f64", 3, "kv_df_sym_kernel (double-float)"),
@@ -1248,10 +1251,12 @@ def run_kv(args):
     ms /= args.steps
     rates = probed_rates(kpcg)
     rates["bf16_tflops"] = float(measured_peaks().get("bf16_tflops", 1934.6))
-    roof = alu_roofline(kname, p.n, p.d, c, ms, rates, fp64=(args.kv_impl == "f64"))
+    if args.kv_impl == "df" and (c > 2 or p.n <= 2048):
+        kname = FX_NAME  # the double-float entry takes it there
+    roof = alu_roofline(kname, p.n, p.d, c, ms, rates)
     roof.update({"peak_source": PEAK_SOURCE, "traffic": known_traffic(kname, p.n),
                  "timing": f"{args.steps} back-to-back products, CUDA events on the stream"})
-    if args.kv_impl in ("df", "df1"):
+    if args.kv_impl in ("df", "df1") and kname != FX_NAME:
         roof["issue_efficiency"] = df_issue_eff(p.n, p.d, c, ms, rates,
                                                 symmetric=(args.kv_impl == "df"))
     elif args.kv_impl == "dfs":
@@ -1274,7 +1279,7 @@ PRECISION_SWEEP = (("fp32_ir", 0.25, 0.1), ("fp32_ir", 1.0, 0.1), ("fp32_ir", 4.
 def run_precision(args):
     """The record behind the choice of solver for the headline system: for
     each reduced-precision product, the norm of its error operator
-    ||K_op - K||_2 (power iteration against the native-FP64 product) and its
+    ||K_op - K||_2 (power iteration against the FP64-class product) and its
     error on a smooth (constant) and a rough (Rademacher) unit vector, at
     n = 4096, 16384 and --n; then the flexible-CG solve of the n = --n system
     for each (mode, inner shift, inner tolerance) of the sweep, with the worst

@@ -82,7 +82,7 @@ typedef enum {
     KPCG_DF64 = 4,     /* FP64 vectors and scalars; iterations use the
                           double-float K.V (FP32-pair arithmetic on the FP32
                           pipe, about 44 bits); stop and restart decisions use
-                          the native FP64 residual                               */
+                          the FP64-accurate residual (kpcg_matvec_f64, impl 0)   */
     KPCG_FP32X_IR = 5, /* as KPCG_FP32_IR, the inner K.V in FP32 on exact
                           pairwise differences: the scaled inputs stay split
                           into FP32 pairs (no per-point rounding), each entry
@@ -123,7 +123,9 @@ typedef struct {
                              wait expires and the call returns KPCG_ERR_TIMEOUT;
                              default 0                                          */
     int64_t wait_limit_ns; /* limit of each wait inside the tensor-core kernels
-                             (ns); 0 = the default, 2 s; a wait that expires
+                             (ns); 0 = the default, 2 s, which the FP64-class
+                             product and the preconditioner set-up always
+                             use; a wait that expires
                              records an error, lets the kernel's own bulk copies
                              land, frees its tensor memory and returns          */
     int32_t inner_f64;    /* KPCG_TCX_IR: 1 runs the inner PCG on FP64 vectors
@@ -441,7 +443,7 @@ kpcg_status kpcg_mlp_get_params(kpcg_mlp_t m, float* params);
 void kpcg_mlp_destroy(kpcg_mlp_t m);
 const char* kpcg_mlp_last_error(kpcg_mlp_t m);
 
-/* The native-FP64 product O = (K + sigma^2 I) V of kpcg_matvec_f64 (impl 0)
+/* The product O = (K + sigma^2 I) V of kpcg_matvec_f64 (impl 0) in native FP64,
  * for callers that cannot allocate device memory: for example a host program
  * whose GPU memory is entirely reserved by another allocator (a framework's
  * pool that has claimed the device), or a latency-critical caller that must
@@ -491,7 +493,7 @@ kpcg_status kpcg_probe_rates(void* stream, double* out);
  * with its own inputs, hyperparameters and Nystrom preconditioner (Sec. 3.1);
  * every one of its c right-hand sides runs its own CG (Algorithm 1) and stops
  * on its own.  The solve is the mixed-precision one (KPCG_TC_IR): an FP64
- * flexible-CG outer loop (double-float direction products, native-FP64 residuals) around an
+ * flexible-CG outer loop (double-float direction products, FP64-accurate residuals) around an
  * inner FP32 PCG whose products with K are ONE persistent tensor-core launch
  * over the tiles of all problems, and whose preconditioner applies are one
  * batched launch sequence.

@@ -561,7 +561,7 @@ static MixedOps single_ops(Ctx& h) {
         }
     };
     // directions of the outer loop: double-float (their product error scales
-    // with the correction); true residuals stay native FP64 (residual_f64)
+    // with the correction); true residuals keep FP64 accuracy (residual_f64)
     o.outer_mv = [hp](const double* V, int64_t ldv, int cc, double* O, int64_t ldo) {
         kv_df(*hp, V, ldv, cc, nullptr, 0, O, ldo, hp->noise);
     };

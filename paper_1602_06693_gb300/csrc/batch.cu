@@ -6,7 +6,7 @@
 // with K is one persistent tensor-core launch over the flat tile list of all
 // problems and every preconditioner apply is one batched launch sequence.
 // The outer loop's direction products use the double-float kernel per
-// problem and every true residual the native-FP64 one (its error scales with
+// problem and every true residual the FP64-accurate one (its error scales with
 // the full solution, the directions' with the small correction).  Columns,
 // hence problems, stop independently.
 #include <cuda_runtime.h>
@@ -370,7 +370,7 @@ kpcg_status kpcg_batch_solve(kpcg_batch_t b, const double* B, int64_t ld, int32_
             for (size_t p = 0; p < bb->sub.size(); ++p) {
                 Ctx& h = *bb->sub[p];
                 const int64_t off = (int64_t)p * c;
-                // certify: native FP64 (b - K x cancels terms up to ~|x|/|b| ~
+                // certify: FP64 accuracy (b - K x cancels terms up to ~|x|/|b| ~
                 // 1/sigma^2 larger than the result, beyond the double-float
                 // product's reach); steering only: double-float
                 M.prof.time(Profiler::RESID, M.stream, [&] {

@@ -53,10 +53,10 @@
 // next unit and the byte MMAs of the last one run behind a unit's evaluation.
 // All bytes of K accumulate into the same columns [level l][column of V], byte a
 // against V's bytes moved down by a levels (operand rows that start a x cpad rows
-// earlier, in zeros): MMAs whose accumulators overlap without being the same
-// took ~260 cycles each, ones that share them a sixth of that.  (Units
-// of 16 columns, two sets of warps on alternate units: 42 distance MMAs per 32 columns
-// instead of 21, at ~70 cycles each, whatever N is below 64.)
+// earlier, in zeros), so that one accumulator takes all of them: the order of MMAs whose
+// accumulators overlap without being the same is not defined.  (Units of 16 columns with
+// two sets of warps on alternate units took a third longer: twice the distance MMAs, and an
+// MMA takes the same time whatever N is below 64.)
 // TMEM: 6 x 32 columns of levels, 7 x 16 of bytes, 8 x cpad (<= 192) of sums.
 // Every mbarrier wait is bounded.
 #include <cuda_fp16.h>

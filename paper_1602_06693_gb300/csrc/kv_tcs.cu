@@ -434,8 +434,8 @@ void tcs_plan(Ctx& h, int64_t n_t) {
 
 }  // namespace
 
-// Usable while its row partials (n_t (n_t + 1) / 2 tile pairs x 2 halves x 128
-// FP32 values) stay within 4 GiB, i.e. up to n ~ 370 000; beyond that the
+// Usable while n_t (n_t + 1) x 128 FP32 values stay within 4 GiB, i.e. up to
+// n ~ 370 000 (its row partials are about a quarter of that); beyond that the
 // one-sided kernel evaluates every entry.
 bool kv_tcs_usable(const Ctx& h) {
     const double n_t = (double)((h.n + TM - 1) / TM);

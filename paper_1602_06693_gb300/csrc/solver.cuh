@@ -19,7 +19,7 @@ struct MixedOps {
     std::function<void(const double*, int64_t, int, double*, int64_t)> inner_mv64, inner_pc64;
     // O = K_y V with FP64-class accuracy
     std::function<void(const double*, int64_t, int, double*, int64_t)> outer_mv;
-    // R = B - K_y X and the per-column ||R||^2, ||B||^2; certify: native FP64
+    // R = B - K_y X and the per-column ||R||^2, ||B||^2; certify: FP64 accuracy
     // (the value the stop test is decided on), else FP64-class (steering only)
     std::function<void(const double*, int64_t, int, const double*, int64_t, double*,
                        std::vector<double>&, std::vector<double>&, bool certify)>
