@@ -152,7 +152,7 @@ template <typename T, typename MV, typename PC>
 static int pcg_core(Ctx& h, int c, const T* B, int64_t ldb, T* X, int64_t ldx, bool x0_zero,
                     double tol, int tol_mode, int max_iter, MV&& matvec, PC&& precond,
                     CgBufs<T>& bufs, std::vector<int>& iters_out, int& broken,
-                    const T* R0 = nullptr) {
+                    const T* R0 = nullptr, GraphChunk* keep = nullptr) {
     const int64_t n = h.n, ld = h.ld;
     cudaStream_t st = h.stream;
     T* r = bufs.r.need((size_t)ld * c);
@@ -201,7 +201,12 @@ static int pcg_core(Ctx& h, int c, const T* B, int64_t ldb, T* X, int64_t ldx, b
     // of the activity flags are captured once into a CUDA graph and replayed.
     // Iterations past convergence inside a chunk change nothing: stopped
     // columns have alpha = beta = 0.
-    GraphChunk chunk;
+    // With `keep` (inner solves of one outer loop: same blocks, same operators) the chunk
+    // recorded by an earlier call is replayed from the first iteration on, until a buffer
+    // moves.  Recording and instantiating one costs ~0.15 ms: a solve of n = 1030 with ten
+    // outer steps 13.4 -> 11.8 ms.
+    GraphChunk own;
+    GraphChunk& chunk = keep ? *keep : own;
     const bool graphs = h.use_graph && !h.prof.on;
     auto body = [&](cudaStream_t s) {
         matvec(p, ld, c, q, ld);
@@ -210,8 +215,8 @@ static int pcg_core(Ctx& h, int c, const T* B, int64_t ldb, T* X, int64_t ldx, b
         cg_direction<T>(p, ld, r, ld, z, ld, n, c, S, partial, nblk, s);
     };
     while (active > 0 && it < max_iter) {
-        if (graphs && it >= every && it + every <= max_iter) {
-            if (!chunk.exec)
+        if (graphs && (it >= every || chunk.valid()) && it + every <= max_iter) {
+            if (!chunk.valid())
                 chunk.capture(h, [&](cudaStream_t cs) {
                     for (int j = 0; j < every; ++j) body(cs);
                     KPCG_CUDA(cudaMemcpyAsync(hf, S.flags, 2 * sizeof(int),
@@ -381,6 +386,8 @@ kpcg_status fcg_solve(Ctx& h, const MixedOps& ops, const double* B, int64_t ldb,
         bb = rr;
     }
     std::vector<double> pAp((size_t)W * c, 1.0), coef((size_t)c), d;
+    GraphChunk chunk;  // of the inner PCG, for this call
+    GraphChunk* keep = ops.keep_graph ? &chunk : nullptr;
     std::vector<int> dead((size_t)c, 0);
     int nwin = 0, head = 0, stall = 0, recheck = 0;
     double best = INFINITY;
@@ -443,7 +450,7 @@ kpcg_status fcg_solve(Ctx& h, const MixedOps& ops, const double* B, int64_t ldb,
                     h.prof.time(Profiler::PRECOND, st,
                                 [&] { ops.inner_pc64(Rr, ldr, cc, Zz, ldz); });
                 },
-                h.c64, its, br);
+                h.c64, its, br, nullptr, keep);
             convert_scale_cols<double, double>(Z, ld, d64, ld, n, c, cs, 0, st);
         } else {
             convert_scale_cols<float, double>(b32, ld, R, ld, n, c, cs, 1, st);
@@ -457,7 +464,7 @@ kpcg_status fcg_solve(Ctx& h, const MixedOps& ops, const double* B, int64_t ldb,
                     h.prof.time(Profiler::PRECOND, st,
                                 [&] { ops.inner_pc(Rr, ldr, cc, Zz, ldz); });
                 },
-                h.c32, its, br);
+                h.c32, its, br, nullptr, keep);
             convert_scale_cols<double, float>(Z, ld, d32, ld, n, c, cs, 0, st);
         }
         iters_total += ran;
@@ -527,6 +534,7 @@ kpcg_status fcg_solve(Ctx& h, const MixedOps& ops, const double* B, int64_t ldb,
 // The operators of the single-problem mixed-precision solve.
 static MixedOps single_ops(Ctx& h) {
     MixedOps o;
+    o.keep_graph = true;
     const bool tc = (h.opt.precision == KPCG_TC_IR);
     const bool xf = (h.opt.precision == KPCG_FP32X_IR);
     const bool tcx = (h.opt.precision == KPCG_TCX_IR);

@@ -4,6 +4,7 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include <atomic>
 #include <string>
 #include <vector>
 
@@ -34,6 +35,13 @@ void check_dev_ptr(const void* p, const char* name);
 #define KPCG_LAUNCHED(name) \
     (::kpcg::note_launch(), ::kpcg::cuda_check(cudaGetLastError(), name, __FILE__, __LINE__))
 
+// Goes up whenever a device buffer of the process is allocated or freed: a recorded graph
+// holds addresses and is good for as long as this has not moved.
+inline std::atomic<long long>& buffer_epoch() {
+    static std::atomic<long long> e{0};
+    return e;
+}
+
 // A device allocation owned by RAII.
 template <typename T>
 struct DevBuf {
@@ -44,7 +52,10 @@ struct DevBuf {
     DevBuf& operator=(const DevBuf&) = delete;
     ~DevBuf() { release(); }
     void release() {
-        if (p) cudaFree(p);
+        if (p) {
+            cudaFree(p);
+            ++buffer_epoch();
+        }
         p = nullptr;
         count = 0;
     }
@@ -59,6 +70,7 @@ struct DevBuf {
             p = nullptr;
             fail(KPCG_ERR_OOM, "cudaMalloc of " + std::to_string(bytes) + " bytes failed");
         }
+        ++buffer_epoch();
         count = n;
         return p;
     }

@@ -251,6 +251,7 @@ struct LapMixed {
 MixedOps lap_mixed_ops(Ctx* hp, const VecOp& mvB, const LapMixed& m, bool tc, bool pre,
                        double* r) {
     MixedOps o;
+    o.keep_graph = true;
     o.inner_mv = [hp, m, tc](const float* V, int64_t ldv, int cc, float* O, int64_t ldo) {
         Ctx& H = *hp;
         const dim3 gg(lap_grid(H.n), (unsigned)cc);

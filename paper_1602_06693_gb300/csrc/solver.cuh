@@ -26,6 +26,9 @@ struct MixedOps {
         residual;
     // true if a bounded device wait expired since the last query
     std::function<bool()> timed_out;
+    // the inner operators launch the same kernels with the same arguments throughout a
+    // solve, as long as no buffer moves
+    bool keep_graph = false;
 };
 
 // Makes the active-column flags of the running CG visible to the operators
@@ -45,8 +48,13 @@ struct ActiveScope {
 struct GraphChunk {
     cudaGraphExec_t exec = nullptr;
     long long kernels = 0;  // kernel launches recorded, counted again per replay
+    long long epoch = -1;   // buffer_epoch() of the recording
+    bool valid() const { return exec && epoch == buffer_epoch(); }
     template <typename F>
     void capture(Ctx& h, F&& f) {
+        if (exec) cudaGraphExecDestroy(exec);
+        exec = nullptr;
+        epoch = buffer_epoch();
         const long long l0 = launch_count();
         cudaStream_t cs = nullptr;
         KPCG_CUDA(cudaStreamCreateWithFlags(&cs, cudaStreamNonBlocking));

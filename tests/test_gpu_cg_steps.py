@@ -47,3 +47,27 @@ def test_columns(n, precision):
         assert np.linalg.norm(r[:, k]) <= 1.01 * TOL * nb[k]
     assert abs(int(it[0]) - int(it[2])) <= 1
     assert np.linalg.norm(x[:, 2] - 2.0 * x[:, 0]) <= 1e-5 * np.linalg.norm(x[:, 2])
+
+
+@pytest.mark.parametrize("n,c", [(300, 1), (2500, 5)])
+def test_replayed_chunks(n, c):
+    """A fresh handle's buffers move between its first inner solves and a used one's do
+    not, so the recorded iterations are replayed from different points on: every kernel is
+    deterministic, the results are equal bit by bit."""
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    import paper_1602_06693_gb300 as kpcg
+    from paper_1602_06693_gb300 import build
+    build.build()
+    p = synthetic.make_problem(n, 4, 7, dist="normal", ell=1.0, noise=1e-3)
+    idx = synthetic.inducing_subset(n, 32, seed=3)
+    B = torch.from_numpy(np.ascontiguousarray(synthetic.rng(9).standard_normal((c, n)))).cuda().t()
+    opt = kpcg.default_options(precision=kpcg.KPCG_TC_IR)
+    with kpcg.Solver(torch.from_numpy(p.X).cuda(), p.log_theta, p.noise, options=opt) as s:
+        s.precond(kpcg.KPCG_PREC_NYSTROM, 32, idx)
+        runs = [s.solve(B, tol=TOL) for _ in range(3)]
+    X, it, info, st = runs[0]
+    assert st == 0 and info.outer_steps >= 3 and info.max_rel_res <= TOL
+    for Y, jt, jnfo, _ in runs[1:]:
+        assert np.array_equal(jt, it) and jnfo.iters_total == info.iters_total
+        assert torch.equal(Y, X)
