@@ -847,7 +847,8 @@ void kv_fx(Ctx& h, const double* V, int64_t ldv, int c, const double* B, int64_t
         fx_stage_v_kernel<<<(unsigned)((thr + 127) / 128), 128, 0, st>>>(Vk, ldv, n, n_pad, nc, cpad,
                                                                          mx, Vop);
         KPCG_LAUNCHED("fx_stage_v_kernel");
-        if (nc <= 2)
+        // V is staged at the call's width: a narrow last pass of a wide block keeps that layout
+        if (cpad == 8 && nc <= 2)
             launch_fx_ks<8, 2>(h, Vop, n_pad, nc, nsplit, gps, part);
         else if (cpad == 8)
             launch_fx_ks<8, 8>(h, Vop, n_pad, nc, nsplit, gps, part);
