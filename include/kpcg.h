@@ -119,15 +119,15 @@ typedef struct {
                              in kpcg_info; default 0                           */
     int32_t wait_stall;   /* test hook of the bounded waits: 1 makes the MMA
                              thread of the single-problem tensor-core kernels
-                             first wait on a barrier nothing arrives at, so the
-                             wait expires and the call returns KPCG_ERR_TIMEOUT;
-                             default 0                                          */
+                             (the double-float ones excepted) first wait on a
+                             barrier nothing arrives at, so the wait expires and
+                             the call returns KPCG_ERR_TIMEOUT; default 0       */
     int64_t wait_limit_ns; /* limit of each wait inside the tensor-core kernels
-                             (ns); 0 = the default, 2 s, which the FP64-class
-                             product and the preconditioner set-up always
-                             use; a wait that expires
-                             records an error, lets the kernel's own bulk copies
-                             land, frees its tensor memory and returns          */
+                             (ns); 0 = the default, 2 s, which the product of FP64
+                             accuracy and the preconditioner set-up use unless
+                             wait_stall is set; a wait that expires records an
+                             error, lets the kernel's own bulk copies land,
+                             frees its tensor memory and returns                */
     int32_t inner_f64;    /* KPCG_TCX_IR: 1 runs the inner PCG on FP64 vectors
                              (the sliced tensor-core product takes them as FP32
                              pairs and returns FP64), so the inner solve is

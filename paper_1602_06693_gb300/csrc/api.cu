@@ -304,6 +304,7 @@ static double precond_noise(const Ctx& h) {
 static void build_precond(Ctx& h) {
     h.P.reset();
     ++h.pversion;
+    h.P.stall_ns = setup_stall_ns(h);
     const double nz = precond_noise(h);
     if (h.pkind == KPCG_PREC_NYSTROM)
         nystrom_setup(h.P, h.xs32.p, h.xs64.p, h.n, h.dp, h.c0_32(), h.c0_64(), nz,

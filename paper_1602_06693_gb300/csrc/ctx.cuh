@@ -239,10 +239,16 @@ void kv_tcd(Ctx& h, const double* V, int64_t ldv, int c, const double* B, int64_
 bool kv_tcd_supported(const Ctx& h);
 // FP64-class K.V in fixed point on the tensor cores (kv_fx.cu; arguments of
 // kv_df), for handles where kv_fx_usable holds: d <= 16, scaled inputs within
-// smax, c columns' partial sums within 4 GiB.
+// smax, c columns' partial sums within 4 GiB.  limited: its waits follow the options'
+// wait_limit_ns.
 void kv_fx(Ctx& h, const double* V, int64_t ldv, int c, const double* B, int64_t ldb, double* O,
-           int64_t ldo, double noise);
+           int64_t ldo, double noise, bool limited);
 bool kv_fx_usable(Ctx& h, int c, double smax);
+// PrecondState::stall_ns of a set-up under the handle's options.
+inline int64_t setup_stall_ns(const Ctx& h) {
+    if (!h.opt.wait_stall) return 0;
+    return h.opt.wait_limit_ns > 0 ? h.opt.wait_limit_ns : 2000000000;
+}
 // Double-float inputs of the handle (exp2 table, log2(s^2) pair), kv_df.cu.
 void df_prepare(Ctx& h);
 // Column count from which the inner products of the mixed solvers use

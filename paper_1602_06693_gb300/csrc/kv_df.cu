@@ -970,7 +970,7 @@ void kv_f64_sym(Ctx& h, const double* V, int64_t ldv, int c, const double* B, in
     // (|y| <= 8: the dropped levels stay near 2^-53 of an entry): 12.1 ms against
     // 119.6 ms at n = 65536, d = 8 and 0.07 against 0.18 ms at n = 200, one column
     if (kv_fx_usable(h, c, 8.0)) {
-        kv_fx(h, V, ldv, c, B, ldb, O, ldo, noise);
+        kv_fx(h, V, ldv, c, B, ldb, O, ldo, noise, false);
         return;
     }
     // otherwise on the FP64 pipe: symmetric tile pairs halve the exps but take at
@@ -1028,7 +1028,7 @@ void kv_df(Ctx& h, const double* V, int64_t ldv, int c, const double* B, int64_t
     // (n = 2000, one column: 0.077 against 0.097 ms).  Up to |y| = 64 its dropped levels
     // stay below the 2^-45 of a double-float entry.
     if (h.df_tensor && (c >= 3 || h.d > 10 || h.n <= 2048) && kv_fx_usable(h, c, 64.0)) {
-        kv_fx(h, V, ldv, c, B, ldb, O, ldo, noise);
+        kv_fx(h, V, ldv, c, B, ldb, O, ldo, noise, true);
         return;
     }
     // the squared distances on the tensor cores where the sliced layout fits

@@ -197,7 +197,7 @@ __global__ void __launch_bounds__(QWARPS * 32, 1)
     kv_fx_kernel(const __half* __restrict__ Aop, const __half* __restrict__ Bop,
                  const __half* __restrict__ Vop, int64_t n, int64_t n_pad, int ncols,
                  int groups_per_split, FxScale w, const uint64_t* __restrict__ gtab,
-                 double* __restrict__ part, int* __restrict__ err, uint64_t wait_ns) {
+                 double* __restrict__ part, int* __restrict__ err, uint64_t wait_ns, int stall) {
     using S = FxSmem<SUBT, CPAD>;
     extern __shared__ uint8_t smem_raw[];
     uint8_t* smem = reinterpret_cast<uint8_t*>(
@@ -214,7 +214,8 @@ __global__ void __launch_bounds__(QWARPS * 32, 1)
     uint64_t* bfree = bfull + 1;     // byte MMAs of a unit done
     uint64_t* afull = bfree + 1;
     uint64_t* done = afull + 1;
-    uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(done + 1);
+    uint64_t* never = done + 1;  // test hook: no thread ever arrives here
+    uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(never + 1);
     double* comb = reinterpret_cast<double*>(smem);  // after the loop: [CPAD][128]
     __shared__ int s_fail;
 
@@ -240,6 +241,7 @@ __global__ void __launch_bounds__(QWARPS * 32, 1)
         mbar_init(bfree, 1);
         mbar_init(afull, 1);
         mbar_init(done, 1);
+        mbar_init(never, 1);
         s_fail = 0;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
@@ -290,7 +292,9 @@ __global__ void __launch_bounds__(QWARPS * 32, 1)
         }
     } else if (warp == 1) {
         const uint32_t el = elect_one();
-        if (!mbar_wait_warp(afull, 0, deadline)) fail = 1;
+        // test hook: a wait on a barrier nothing arrives at runs out
+        if (stall && !mbar_wait_warp(never, 0, deadline)) fail = 1;
+        if (!fail && !mbar_wait_warp(afull, 0, deadline)) fail = 1;
         fence_after();
         const uint32_t a0 = su32(sA);
         // the levels of unit t
@@ -672,7 +676,7 @@ __global__ void fx_reduce_kernel(const double* __restrict__ part, int64_t n_pad,
 
 template <int SUBT, int KS, int CPAD, int CU>
 void launch_fx(Ctx& h, const uint8_t* Vop, int64_t n_pad, int ncols, int nsplit, int gps,
-               double* part) {
+               double* part, uint64_t wait_ns) {
     using S = FxSmem<SUBT, CPAD>;
     static const bool attr = [] {
         KPCG_CUDA(cudaFuncSetAttribute(kv_fx_kernel<SUBT, KS, CPAD, CU>,
@@ -686,17 +690,17 @@ void launch_fx(Ctx& h, const uint8_t* Vop, int64_t n_pad, int ncols, int nsplit,
                                    S::kTotal, h.stream>>>(
         reinterpret_cast<const __half*>(h.fxA.p), reinterpret_cast<const __half*>(h.fxB.p),
         reinterpret_cast<const __half*>(Vop), h.n, n_pad, ncols, gps, w, h.fx_tab.p, part,
-        h.tc_err.p, kWaitNs);
+        h.tc_err.p, wait_ns, h.opt.wait_stall ? 1 : 0);
     KPCG_LAUNCHED("kv_fx_kernel");
 }
 
 template <int CPAD, int CU>
 void launch_fx_ks(Ctx& h, const uint8_t* Vop, int64_t n_pad, int ncols, int nsplit, int gps,
-                  double* part) {
+                  double* part, uint64_t wait_ns) {
     if (h.d + 4 <= 16)
-        launch_fx<2, 1, CPAD, CU>(h, Vop, n_pad, ncols, nsplit, gps, part);
+        launch_fx<2, 1, CPAD, CU>(h, Vop, n_pad, ncols, nsplit, gps, part, wait_ns);
     else
-        launch_fx<3, 2, CPAD, CU>(h, Vop, n_pad, ncols, nsplit, gps, part);
+        launch_fx<3, 2, CPAD, CU>(h, Vop, n_pad, ncols, nsplit, gps, part, wait_ns);
 }
 
 // floor(sqrt(v))
@@ -823,10 +827,13 @@ bool kv_fx_usable(Ctx& h, int c, double smax) {
 }
 
 void kv_fx(Ctx& h, const double* V, int64_t ldv, int c, const double* B, int64_t ldb, double* O,
-           int64_t ldo, double noise) {
+           int64_t ldo, double noise, bool limited) {
     if (h.n <= 0 || c <= 0) return;
     cudaStream_t st = h.stream;
     const int64_t n = h.n, n_pad = (n + 127) / 128 * 128;
+    const uint64_t wait_ns = (limited || h.opt.wait_stall) && h.opt.wait_limit_ns > 0
+                                 ? (uint64_t)h.opt.wait_limit_ns
+                                 : kWaitNs;
     fx_prepare(h);
     fx_operands(h, n_pad);
     int nsplit, gps;
@@ -849,13 +856,13 @@ void kv_fx(Ctx& h, const double* V, int64_t ldv, int c, const double* B, int64_t
         KPCG_LAUNCHED("fx_stage_v_kernel");
         // V is staged at the call's width: a narrow last pass of a wide block keeps that layout
         if (cpad == 8 && nc <= 2)
-            launch_fx_ks<8, 2>(h, Vop, n_pad, nc, nsplit, gps, part);
+            launch_fx_ks<8, 2>(h, Vop, n_pad, nc, nsplit, gps, part, wait_ns);
         else if (cpad == 8)
-            launch_fx_ks<8, 8>(h, Vop, n_pad, nc, nsplit, gps, part);
+            launch_fx_ks<8, 8>(h, Vop, n_pad, nc, nsplit, gps, part, wait_ns);
         else if (cpad == 16)
-            launch_fx_ks<16, 16>(h, Vop, n_pad, nc, nsplit, gps, part);
+            launch_fx_ks<16, 16>(h, Vop, n_pad, nc, nsplit, gps, part, wait_ns);
         else
-            launch_fx_ks<24, 24>(h, Vop, n_pad, nc, nsplit, gps, part);
+            launch_fx_ks<24, 24>(h, Vop, n_pad, nc, nsplit, gps, part, wait_ns);
         fx_reduce_kernel<<<dim3((unsigned)((n + 127) / 128), (unsigned)nc), 128, 0, st>>>(
             part, n_pad, nsplit, nc, mx, h.s2, h.xs64.p, h.dp, h.c0_64(), Vk, ldv, noise,
             B ? B + (int64_t)k0 * ldb : nullptr, ldb, O + (int64_t)k0 * ldo, ldo, n);

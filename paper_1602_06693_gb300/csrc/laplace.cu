@@ -422,6 +422,7 @@ kpcg_status kpcg_laplace(kpcg_t h, const double* y, double newton_tol, int32_t m
                 KPCG_CUDA(cudaMemcpyAsync(sWb, sW, sizeof(double) * n, cudaMemcpyDeviceToDevice,
                                           st));
                 const auto s0 = std::chrono::steady_clock::now();
+                c.LP.stall_ns = setup_stall_ns(c);
                 laplace_precond_setup(c.LP, c.lkxu0, builds == 1, c.xs32.p, c.xs64.p, n, c.dp,
                                       c.c0_64(), sW, c.pidx.data(), c.psize, st);
                 KPCG_CUDA(cudaStreamSynchronize(st));
@@ -528,6 +529,7 @@ kpcg_status kpcg_laplace_predict(kpcg_t h, const double* y, const double* f, con
             const bool pre = c.pkind == KPCG_PREC_NYSTROM;
             if (pre) {
                 const auto s0 = std::chrono::steady_clock::now();
+                c.LP.stall_ns = setup_stall_ns(c);
                 laplace_precond_setup(c.LP, c.lkxu0, true, c.xs32.p, c.xs64.p, n, c.dp,
                                       c.c0_64(), sW, c.pidx.data(), c.psize, st);
                 pre_built = 1;

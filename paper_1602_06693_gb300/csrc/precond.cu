@@ -699,7 +699,7 @@ static void nys_syrk_factor(PrecondState& P, int64_t n, int64_t m, cudaStream_t 
     double* part = P.scratch.need((size_t)nsplit * m * m);
     int* late = P.status.need(2) + 1;
     KPCG_CUDA(cudaMemsetAsync(late, 0, sizeof(int), st));
-    syrk_fx(P.KXU.p, n, m, P.digits, part, late, st);
+    syrk_fx(P.KXU.p, n, m, P.digits, part, late, P.stall_ns, st);
     syrk_reduce_kernel<<<(unsigned)((m * m + 255) / 256), 256, 0, st>>>(part, nsplit, m, M0);
     KPCG_LAUNCHED("syrk_reduce_kernel");
     int bad = 0;

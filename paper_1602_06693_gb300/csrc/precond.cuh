@@ -25,6 +25,8 @@ struct PrecondState {
     DevBuf<uint8_t> digits;  // row blocks of K_XU as digits (syrk_fx.cu)
     DevBuf<double> wpart, w, y;
     DevBuf<int> status;
+    // test hook of the set-up's bounded waits: > 0 lets one run out after so many ns
+    int64_t stall_ns = 0;
     double apply_noise = 0.0;  // divisor of the Nystrom apply (1 for FITC's scaled form)
     DevBuf<double> dscale;     // FITC: D^{-1/2}, D = diag(K - Q) + sigma^2
     DevBuf<double> tmp64;      // FITC: scaled right-hand sides
@@ -103,10 +105,10 @@ void pitc_setup(PrecondState& P, const float* xs32, const double* xs64, int64_t 
 
 // part[s] (s < syrk_fx_splits(n, m), each m x m row-major) = parts of the lower triangle
 // of KXU^T KXU (KXU n x m FP32 pairs) in fixed point on the tensor cores (syrk_fx.cu).
-// err is set if a bounded wait expires.
+// err is set if a bounded wait expires; stall_ns > 0 makes one expire (test hook).
 int syrk_fx_splits(int64_t n, int64_t m);
 void syrk_fx(const float2* KXU, int64_t n, int64_t m, DevBuf<uint8_t>& work, double* part,
-             int* err, cudaStream_t st);
+             int* err, int64_t stall_ns, cudaStream_t st);
 
 // ------------------------------------------- batched Nystrom apply
 // Problems laid out column by column (problem p owns columns p*c .. p*c+c-1

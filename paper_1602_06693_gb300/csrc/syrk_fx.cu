@@ -136,7 +136,7 @@ __host__ __device__ inline void syrk_tile(int x, int& T, int& u) {
 __global__ void __launch_bounds__(YWARPS * 32, 1)
     syrk_fx_kernel(const uint8_t* __restrict__ dig, int64_t m, int ct, int ngroups,
                    int groups_per_split, const unsigned* __restrict__ mx, int first,
-                   double* __restrict__ part, int* __restrict__ err) {
+                   double* __restrict__ part, int* __restrict__ err, uint64_t wait_ns, int stall) {
     extern __shared__ uint8_t smem_raw[];
     uint8_t* smem = reinterpret_cast<uint8_t*>(
         (reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
@@ -146,7 +146,8 @@ __global__ void __launch_bounds__(YWARPS * 32, 1)
     uint64_t* lfull = empty + YNST;  // levels of YG stages ready
     uint64_t* lfree = lfull + 1;     // levels read
     uint64_t* done = lfree + 1;
-    uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(done + 1);
+    uint64_t* never = done + 1;  // test hook: no thread ever arrives here
+    uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(never + 1);
     __shared__ int s_fail;
 
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -164,6 +165,7 @@ __global__ void __launch_bounds__(YWARPS * 32, 1)
         mbar_init(lfull, 1);
         mbar_init(lfree, YEPI);
         mbar_init(done, 1);
+        mbar_init(never, 1);
         s_fail = 0;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
@@ -178,7 +180,7 @@ __global__ void __launch_bounds__(YWARPS * 32, 1)
     __syncthreads();
     fence_after();
     const uint32_t tmem = *tmem_slot;
-    const uint64_t deadline = gtimer() + kWaitNs;
+    const uint64_t deadline = gtimer() + wait_ns;
     int fail = 0;
 
     if (warp == 0) {
@@ -207,6 +209,8 @@ __global__ void __launch_bounds__(YWARPS * 32, 1)
         }
     } else if (warp == 1) {
         const uint32_t el = elect_one();
+        // test hook: a wait on a barrier nothing arrives at runs out
+        if (stall && !mbar_wait_warp(never, 0, deadline)) fail = 1;
         for (int t = 0; t < nst && !fail; ++t) {
             const int s = t % YNST, g = t / YG;
             if (!mbar_wait_warp(&full[s], (uint32_t)(t / YNST) & 1u, deadline) ||
@@ -334,7 +338,7 @@ int syrk_fx_splits(int64_t n, int64_t m) {
 }
 
 void syrk_fx(const float2* KXU, int64_t n, int64_t m, DevBuf<uint8_t>& work, double* part,
-             int* err, cudaStream_t st) {
+             int* err, int64_t stall_ns, cudaStream_t st) {
     const int64_t ct = (m + 127) / 128, group = YR * YG;
     int64_t rows;
     int nsplit;
@@ -364,7 +368,8 @@ void syrk_fx(const float2* KXU, int64_t n, int64_t m, DevBuf<uint8_t>& work, dou
         const int ngroups = (int)(here / group);
         // every split writes (the first block) or adds to its part, also when it has no rows
         syrk_fx_kernel<<<dim3((unsigned)tiles, (unsigned)nsplit), YWARPS * 32, kSmemY, st>>>(
-            dig, m, (int)ct, ngroups, (ngroups + nsplit - 1) / nsplit, mx, i0 == 0, part, err);
+            dig, m, (int)ct, ngroups, (ngroups + nsplit - 1) / nsplit, mx, i0 == 0, part, err,
+            stall_ns > 0 ? (uint64_t)stall_ns : kWaitNs, stall_ns > 0 ? 1 : 0);
         KPCG_LAUNCHED("syrk_fx_kernel");
     }
 }
