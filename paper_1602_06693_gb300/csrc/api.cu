@@ -737,11 +737,12 @@ kpcg_status solve_impl(Ctx& h, const double* B, int64_t ldb, int c, double tol,
                            steps, rr, bb);
         rr_current = (status == KPCG_OK);  // converged exits certify on a recomputed residual
     }
-    if (kv_tc_error(h)) fail(KPCG_ERR_TIMEOUT, "a bounded wait in the tensor-core K.V expired");
     // FP64 residual of what is returned (the single-precision FP32 solver
     // checked its own operator only)
     double maxrel = 0.0;
     if (!rr_current || prec == KPCG_FP32) residual_f64(h, B, ldb, c, Xout, ldx, R, rr, bb);
+    // after the last product: an expired wait is not a large residual
+    if (kv_tc_error(h)) fail(KPCG_ERR_TIMEOUT, "a bounded wait in the tensor-core K.V expired");
     bool all = true;
     for (int k = 0; k < c; ++k) {
         if (bb[k] > 0) maxrel = std::max(maxrel, std::sqrt(rr[k] / bb[k]));

@@ -67,3 +67,19 @@ def test_setup(kpcg):
         s.set_options(kpcg.default_options(**opt))
         s.precond(kpcg.KPCG_PREC_NYSTROM, 200, idx)
         assert torch.equal(s.precond_apply(R), want)
+
+
+@pytest.mark.parametrize("precision,max_iter", [("KPCG_FP32", 100000), ("KPCG_FP64", 0)])
+def test_last_residual_of_a_solve(kpcg, precision, max_iter):
+    """The residual of what a solve returns is its last product, and the only one of these
+    two: FP32 iterations take the FP32 kernel, and without a budget nothing iterates."""
+    p = synthetic.make_problem(1500, 8, 5, dist="normal", ell=3.0, noise=1e-1)
+    y = torch.from_numpy(p.y).cuda()
+    opt = dict(precision=getattr(kpcg, precision), max_iter=max_iter)
+    with kpcg.Solver(torch.from_numpy(p.X).cuda(), p.log_theta, p.noise) as s:
+        s.set_options(kpcg.default_options(**opt, **STALL))
+        _timeout(kpcg, lambda: s.solve(y, tol=1e-4))
+        s.set_options(kpcg.default_options())
+        s.matvec_f64(y, impl=0)  # the flag is cleared
+        x, _, info, st = s.solve(y, tol=1e-8)
+        assert st == 0 and info.max_rel_res <= 1e-8
