@@ -234,8 +234,10 @@ kpcg_status kpcg_precond_pitc(kpcg_t h, int64_t m, const int64_t* idx, int64_t b
  * matrix-free product of Sec. 2.1.  impl 0: FP64 accuracy, the product of KPCG_FP64
  * and of the certified residuals: for d <= 16 and scaled inputs |x'| within ~8 in
  * fixed point on the tensor cores (exact level sums of 10-bit slices of x',
- * 56-bit entries and digits of V, sums without rounding; errors at or below
- * those of FP64 sums), else entries and sums in native FP64;
+ * entries good to 2^-54 of their size and to 2^-63 s^2, digits of V to 2^-63 of
+ * its column's largest value, sums without rounding: an error against the
+ * largest entry and value, where FP64 errs against each entry's), else entries
+ * and sums in native FP64;
  * impl 1: the double-float product of KPCG_DF64 and of the outer loop of the
  * mixed modes (FP32-pair arithmetic, about 44 bits per entry, sums carried as
  * FP32 pairs and added in FP64), or the fixed-point product where that is the

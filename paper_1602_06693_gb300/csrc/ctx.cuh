@@ -164,6 +164,7 @@ struct Ctx {
     DevBuf<uint8_t> fxA, fxB, fxV;
     DevBuf<uint64_t> fx_tab;
     DevBuf<unsigned long long> fx_max;
+    DevBuf<int> fxVsum;
     DevBuf<double> fxPart;
     // per-point-exact tensor-core operands (kv_tcx_apply), rebuilt when theta changes
     int tcx_version = -1, tcx_kch = 0, tcx_nmma = 0;

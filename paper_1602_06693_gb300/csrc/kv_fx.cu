@@ -25,24 +25,34 @@
 //    numbers; T = 2^(-(n mod 4096)/4096) is a 57-bit integer of the table, the
 //    product T (2^r - 1) two FP32 numbers whose integer parts are read off the
 //    mantissas of sums with 1.5 2^k and added to T as 64-bit integers; the
-//    result is shifted right by n >> 12 and rounded.  K/s^2 = M 2^-55, M a 56-bit
-//    integer, to about 2^-54 relative.
-// 3. Contraction.  The seven bytes of M are FP16 subnormals as they stand
-//    (byte 2^-24), written to tensor memory as the A operand of a second chain of
+//    result is shifted right by n >> 12 and rounded.  K/s^2 = M 2^-62, M an integer,
+//    to about 2^-54 relative and 2^-63 absolute.
+// 3. Contraction.  M is written in eight balanced digits of base 256: 128 is added to
+//    all of its bytes but the top one, and what the 128s put into a sum, which depends on
+//    V alone, is taken out of the integer sums again.  The bytes are FP16 subnormals as
+//    they stand (byte 2^-24), written to tensor memory as the A operand of a second chain of
 //    MMAs against V cut into eight balanced bytes per column (scaled by a
 //    power of two per column).  Products of byte levels l = a + b add in FP32
 //    accumulators that hold integers below 2^24 over 64 columns; they are then
 //    added to 32-bit integers, which go to FP64 once per work item.  Levels
-//    >= 8 are dropped (2^-63 of max|K| max|V|).  The sum itself has no rounding.
+//    >= 8 are dropped: 2^-62 of max|K| max|V| per product or less, of either sign.  The
+//    sum itself has no rounding.
+//
+// Entries and columns of V are thus cut at an absolute place, 2^-63 of the largest.  On n
+// entries that are small against one (a narrow kernel, V of one sign) such errors add up
+// unless they are of either sign: with seven unsigned bytes (unit 2^-55) a row of n = 65536
+// was off by 2e-14, with eight unsigned ones, for a constant V with digits, by 1.4e-14
+// (products of its constant digits with unsigned bytes in the dropped levels), with these by
+// 7e-16; FP64 sums by 1e-15 to 3e-15.
 //
 // What bounds it: issue of the epilogue, 82 instructions per entry with one
 // column (ncu at n = 16384: issue 74%, the FP32 and ALU pipes 42% each, DRAM the operands once),
 // nearly independent of the number of columns, where the FP64 kernel needs 28 + 2 c FP64
 // operations per pair of points (two per clock and SM) and the double-float one 67 + 25 c
-// FP32 instructions.  n = 65536, d = 8: 12.1 ms with one column (FP64: 119.6 ms), 14.8 ms
-// with nine (double-float: 40.8 ms); n = 45730, d = 9, 17 columns: 8.2 ms (36.1 ms).
+// FP32 instructions.  n = 65536, d = 8: 13.0 ms with one column (FP64: 119.6 ms; 12.1 ms with
+// seven unsigned bytes); n = 45730, d = 9, 17 columns: 8.8 ms (double-float: 36.1 ms).
 // Errors against extended precision on random, constant and smooth vectors: 1e-16 to
-// 5e-16 of the result, at or below those of the FP64 kernel.
+// 5e-16 of the result.
 //
 // Layout.  A work item is 128 rows x a run of 64-column groups of two 32-column
 // units.  18 warps: warp 0 bulk-copies a group's B operand and V bytes into a
@@ -57,7 +67,7 @@
 // accumulators overlap without being the same is not defined.  (Units of 16 columns with
 // two sets of warps on alternate units took a third longer: twice the distance MMAs, and an
 // MMA takes the same time whatever N is below 64.)
-// TMEM: 6 x 32 columns of levels, 7 x 16 of bytes, 8 x cpad (<= 192) of sums.
+// TMEM: 6 x 32 columns of levels, 8 x 16 of bytes, 8 x cpad (<= 192) of sums: all of it.
 // Every mbarrier wait is bounded.
 #include <cuda_fp16.h>
 #include <cuda_runtime.h>
@@ -77,7 +87,7 @@ constexpr int QNS = 6;       // slices of y, levels of the distance
 constexpr int QU = 32;       // columns per unit (N of the distance MMAs)
 constexpr int QG = 64;       // columns per group (one ring stage, one drain)
 constexpr int QUG = QG / QU;  // units per group
-constexpr int QNK = 7;       // bytes of K
+constexpr int QNK = 8;       // bytes of K
 constexpr int QNV = 8;       // bytes of V
 constexpr int QEPI = 16;     // epilogue warps
 constexpr int QWARPS = 2 + QEPI;
@@ -93,6 +103,8 @@ constexpr int kMaxGroups = 120;
 // M1 = 1.5 2^-12 (unit 2^-35) and M3 = 1.5 2^-33 (unit 2^-56), taken off the table's
 // entries so that the mantissas can be added as they are.
 constexpr uint64_t kTabOff = ((uint64_t)0x39C00000u << 21) + 0x2F400000u;
+// 128 in every byte of an entry but the top one
+constexpr uint64_t kDigitOff = 0x0080808080808080ull;
 
 struct FxScale {
     float w0, w1, w2, w3, w4;  // S^2 2^(-17 - 10 k)
@@ -106,8 +118,9 @@ struct FxSmem {
     static constexpr uint32_t kZ = (QNK - 1) * CPAD * 128; // rows of zeros in front of them
     static constexpr uint32_t kStage = QUG * kB + kZ + kV;
     static constexpr uint32_t kTab = QTAB * 8;
-    static constexpr uint32_t kBars = 1024;
+    static constexpr uint32_t kBars = 1024;  // and the V sums behind them
     static constexpr uint32_t kTotal = 1024 + kA + QNST * kStage + kTab + kBars;
+    static_assert(256 + QNV * CPAD * 4 <= kBars, "barriers and V sums");
     static_assert(CPAD * 128 * 8 <= kA + QNST * kStage, "combination buffer");
 };
 
@@ -138,7 +151,7 @@ __device__ __forceinline__ uint32_t prmt(uint32_t a, uint32_t b, uint32_t sel) {
     return __byte_perm(a, b, sel);
 }
 
-// M with K/s^2 = M 2^-55 from the six level accumulators of an entry (step 2
+// kDigitOff + M with K/s^2 = M 2^-62 from the six level accumulators of an entry (step 2
 // of the file's comment); tab holds round(2^(56 - j/4096)) - kTabOff.
 __device__ __forceinline__ uint64_t fx_entry(float L0, float L1, float L2, float L3, float L4,
                                              float L5, const FxScale& w,
@@ -183,20 +196,19 @@ __device__ __forceinline__ uint64_t fx_entry(float L0, float L1, float L2, float
     const float g3 = __fadd_rn(y, 0x1.8p-33f);
     uint64_t M = T + ((uint64_t)__float_as_uint(g1) << 21);
     M += (uint64_t)__float_as_uint(g3);
-    // rounded to nearest: cut off instead, the 2^-56 lost on average by each of n
-    // small entries would add up on a vector of one sign
+    // rounded to nearest: cut off instead, the 2^-63 lost on average by each of n
+    // entries would add up on a vector of one sign
     uint64_t r;
-    asm("shr.u64 %0, %1, %2;" : "=l"(r) : "l"(M), "r"(nb >> 12));  // 0 from 64 on
-    r = (r + 1) >> 1;
-    return r;
+    asm("shr.u64 %0, %1, %2;" : "=l"(r) : "l"(M << 7), "r"(nb >> 12));  // 0 from 64 on
+    return (r + (2 * kDigitOff + 1)) >> 1;
 }
 
 // CU: columns of V whose sums are kept (<= CPAD)
 template <int SUBT, int KS, int CPAD, int CU>
 __global__ void __launch_bounds__(QWARPS * 32, 1)
     kv_fx_kernel(const __half* __restrict__ Aop, const __half* __restrict__ Bop,
-                 const __half* __restrict__ Vop, int64_t n, int64_t n_pad, int ncols,
-                 int groups_per_split, FxScale w, const uint64_t* __restrict__ gtab,
+                 const __half* __restrict__ Vop, const int* __restrict__ vsum, int64_t n,
+                 int64_t n_pad, int ncols, int groups_per_split, FxScale w, const uint64_t* __restrict__ gtab,
                  double* __restrict__ part, int* __restrict__ err, uint64_t wait_ns, int stall) {
     using S = FxSmem<SUBT, CPAD>;
     extern __shared__ uint8_t smem_raw[];
@@ -216,6 +228,8 @@ __global__ void __launch_bounds__(QWARPS * 32, 1)
     uint64_t* done = afull + 1;
     uint64_t* never = done + 1;  // test hook: no thread ever arrives here
     uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(never + 1);
+    // 128 (V bytes above level l) over the item's columns: [l][column of V]
+    int* off = reinterpret_cast<int*>(sStage + QNST * S::kStage + S::kTab + 256);
     double* comb = reinterpret_cast<double*>(smem);  // after the loop: [CPAD][128]
     __shared__ int s_fail;
 
@@ -290,6 +304,17 @@ __global__ void __launch_bounds__(QWARPS * 32, 1)
                 (void)mbar_wait(&full[q % QNST], (uint32_t)(q / QNST) & 1u, dl2);
             (void)mbar_wait(afull, 0, dl2);
         }
+        __syncwarp();
+        int t[QNV * CPAD / 32];
+#pragma unroll
+        for (int e = 0; e < QNV * CPAD / 32; ++e) t[e] = 0;
+        const int* vs = vsum + (size_t)g0 * (QNV * CPAD) + lane;
+#pragma unroll 8
+        for (int g = 0; g < ngroups; ++g)
+#pragma unroll
+            for (int e = 0; e < QNV * CPAD / 32; ++e) t[e] += __ldg(vs + (size_t)g * (QNV * CPAD) + e * 32);
+#pragma unroll
+        for (int e = 0; e < QNV * CPAD / 32; ++e) off[lane + e * 32] = t[e];
     } else if (warp == 1) {
         const uint32_t el = elect_one();
         // test hook: a wait on a barrier nothing arrives at runs out
@@ -412,12 +437,12 @@ __global__ void __launch_bounds__(QWARPS * 32, 1)
                         hi[q] = (uint32_t)(M >> 32);
                         lo[q] = (uint32_t)M;
                     }
-                    if (t == tdiag) {  // the entries of points with themselves: 2^55
+                    if (t == tdiag) {  // the entries of points with themselves: 2^62
 #pragma unroll
                         for (int q = 0; q < 4; ++q)
                             if (cg * 8 + c0 + q0 + q == lane) {
-                                hi[q] = 1u << 23;
-                                lo[q] = 0u;
+                                hi[q] = (1u << 30) + (uint32_t)(kDigitOff >> 32);
+                                lo[q] = (uint32_t)kDigitOff;
                             }
                     }
                     if (c0 + q0 == 0 && t > 0) {
@@ -433,16 +458,18 @@ __global__ void __launch_bounds__(QWARPS * 32, 1)
                     }
                     const uint32_t tb = lane_base + kByteT + (uint32_t)(cg * 4 + (c0 + q0) / 2);
                     // 16-bit lanes (byte, 0): columns 2 v and 2 v + 1 of the chunk
+                    const uint32_t t0 = prmt(hi[0], hi[1], 0x7632), t1 = prmt(hi[2], hi[3], 0x7632);
                     const uint32_t h0 = prmt(hi[0], hi[1], 0x5410), h1 = prmt(hi[2], hi[3], 0x5410);
-                    const uint32_t l0 = prmt(lo[0], lo[1], 0x5410), l1 = prmt(lo[2], lo[3], 0x5410);
                     const uint32_t m0 = prmt(lo[0], lo[1], 0x7632), m1 = prmt(lo[2], lo[3], 0x7632);
-                    tmem_st2(tb + 0 * 16, prmt(hi[0], hi[1], 0x7632), prmt(hi[2], hi[3], 0x7632));
-                    tmem_st2(tb + 1 * 16, prmt(h0, 0u, 0x4341), prmt(h1, 0u, 0x4341));
-                    tmem_st2(tb + 2 * 16, h0 & 0x00ff00ffu, h1 & 0x00ff00ffu);
-                    tmem_st2(tb + 3 * 16, prmt(m0, 0u, 0x4341), prmt(m1, 0u, 0x4341));
-                    tmem_st2(tb + 4 * 16, m0 & 0x00ff00ffu, m1 & 0x00ff00ffu);
-                    tmem_st2(tb + 5 * 16, prmt(l0, 0u, 0x4341), prmt(l1, 0u, 0x4341));
-                    tmem_st2(tb + 6 * 16, l0 & 0x00ff00ffu, l1 & 0x00ff00ffu);
+                    const uint32_t l0 = prmt(lo[0], lo[1], 0x5410), l1 = prmt(lo[2], lo[3], 0x5410);
+                    tmem_st2(tb + 0 * 16, prmt(t0, 0u, 0x4341), prmt(t1, 0u, 0x4341));
+                    tmem_st2(tb + 1 * 16, t0 & 0x00ff00ffu, t1 & 0x00ff00ffu);
+                    tmem_st2(tb + 2 * 16, prmt(h0, 0u, 0x4341), prmt(h1, 0u, 0x4341));
+                    tmem_st2(tb + 3 * 16, h0 & 0x00ff00ffu, h1 & 0x00ff00ffu);
+                    tmem_st2(tb + 4 * 16, prmt(m0, 0u, 0x4341), prmt(m1, 0u, 0x4341));
+                    tmem_st2(tb + 5 * 16, m0 & 0x00ff00ffu, m1 & 0x00ff00ffu);
+                    tmem_st2(tb + 6 * 16, prmt(l0, 0u, 0x4341), prmt(l1, 0u, 0x4341));
+                    tmem_st2(tb + 7 * 16, l0 & 0x00ff00ffu, l1 & 0x00ff00ffu);
                 }
                 if (fail) break;
             }
@@ -466,14 +493,17 @@ __global__ void __launch_bounds__(QWARPS * 32, 1)
     fence_before();
     __syncthreads();
     fence_after();
-    // sums of levels 2 cg, 2 cg + 1 (weight 2^(-14 - 8 l)), smallest first, in FP64
+    // sums of levels 2 cg, 2 cg + 1 (weight 2^(-13 - 8 l)), less what the bytes' 128s have
+    // put into them, smallest first, in FP64
 #pragma unroll 1
     for (int g = 3; g >= 0; --g) {
         if (warp >= 2 && cg == g) {
-            const double sc = ldexp(1.0, -14 - 16 * g);
+            const double sc = ldexp(1.0, -13 - 16 * g);
 #pragma unroll
             for (int k = 0; k < CU; ++k) {
-                const double v = fma((double)acc[1][k], 0x1p-8, (double)acc[0][k]) * sc;
+                const int d0 = acc[0][k] - off[2 * g * CPAD + k];
+                const int d1 = acc[1][k] - off[(2 * g + 1) * CPAD + k];
+                const double v = fma((double)d1, 0x1p-8, (double)d0) * sc;
                 comb[k * 128 + row] = (g == 3) ? v : comb[k * 128 + row] + v;
             }
         }
@@ -601,12 +631,13 @@ __global__ void fx_prep_kernel(const double* __restrict__ xs64, int64_t n, int64
 
 // V's columns as eight balanced bytes each, v = 2^e sum_b v_b 2^(-7 - 8b), 2^e > max|v|:
 // per group of 64 rows of V, operand rows (b, column) of 64 FP16, swizzled.  One
-// thread per (group, column, 8 rows).  Columns with a value that is not
-// finite are left zero (the reduction computes them entry by entry).
+// thread per (group, column, 8 rows).  vsum[group][l][column] = 128 sum of the bytes b < l over
+// the group.  Columns with a value that is not finite are left zero (the reduction
+// computes them entry by entry).
 __global__ void fx_stage_v_kernel(const double* __restrict__ V, int64_t ldv, int64_t n,
                                   int64_t n_pad, int ncols, int cpad,
                                   const unsigned long long* __restrict__ mx,
-                                  uint8_t* __restrict__ Vop) {
+                                  uint8_t* __restrict__ Vop, int* __restrict__ vsum) {
     const int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (e >= (n_pad / 8) * cpad) return;
     // consecutive threads: the 8-row chunks of a column (coalesced reads)
@@ -615,10 +646,13 @@ __global__ void fx_stage_v_kernel(const double* __restrict__ V, int64_t ldv, int
     const int64_t g = chunk >> 3;
     const int c8 = (int)(chunk & 7);
     uint32_t out[QNV][4];
+    int sum[QNV];
 #pragma unroll
-    for (int b = 0; b < QNV; ++b)
+    for (int b = 0; b < QNV; ++b) {
+        sum[b] = 0;
 #pragma unroll
         for (int w = 0; w < 4; ++w) out[b][w] = 0u;
+    }
     if (k < ncols && mx[k] != 0 && mx[k] < 0x7ff0000000000000ull) {
         int ex;
         (void)frexp(__longlong_as_double((long long)mx[k]), &ex);
@@ -630,6 +664,7 @@ __global__ void fx_stage_v_kernel(const double* __restrict__ V, int64_t ldv, int
             for (int b = 0; b < QNV; ++b) {
                 const double v = rint(h);
                 h = (h - v) * 256.0;
+                sum[b] += (int)v;
                 const uint32_t bits = __half_as_ushort(__float2half_rn((float)v));
                 out[b][r >> 1] |= bits << (16 * (r & 1));
             }
@@ -640,6 +675,15 @@ __global__ void fx_stage_v_kernel(const double* __restrict__ V, int64_t ldv, int
         const int rr = b * cpad + k;
         *reinterpret_cast<uint4*>(Vop + ((size_t)g * QNV * cpad + rr) * 128 + ((c8 ^ (rr & 7)) * 16)) =
             make_uint4(out[b][0], out[b][1], out[b][2], out[b][3]);
+    }
+    // over the group's eight threads, neighbours of a warp (n_pad / 8 is a multiple of 16)
+    int above = 0;
+#pragma unroll
+    for (int b = 0; b < QNV; ++b) {
+#pragma unroll
+        for (int o = 4; o > 0; o >>= 1) sum[b] += __shfl_xor_sync(0xffffffffu, sum[b], o);
+        if (c8 == 0) vsum[((size_t)g * QNV + b) * cpad + k] = 128 * above;
+        above += sum[b];
     }
 }
 
@@ -675,7 +719,7 @@ __global__ void fx_reduce_kernel(const double* __restrict__ part, int64_t n_pad,
 }
 
 template <int SUBT, int KS, int CPAD, int CU>
-void launch_fx(Ctx& h, const uint8_t* Vop, int64_t n_pad, int ncols, int nsplit, int gps,
+void launch_fx(Ctx& h, const uint8_t* Vop, const int* vsum, int64_t n_pad, int ncols, int nsplit, int gps,
                double* part, uint64_t wait_ns) {
     using S = FxSmem<SUBT, CPAD>;
     static const bool attr = [] {
@@ -689,18 +733,18 @@ void launch_fx(Ctx& h, const uint8_t* Vop, int64_t n_pad, int ncols, int nsplit,
     kv_fx_kernel<SUBT, KS, CPAD, CU><<<dim3((unsigned)(n_pad / 128), (unsigned)nsplit), QWARPS * 32,
                                    S::kTotal, h.stream>>>(
         reinterpret_cast<const __half*>(h.fxA.p), reinterpret_cast<const __half*>(h.fxB.p),
-        reinterpret_cast<const __half*>(Vop), h.n, n_pad, ncols, gps, w, h.fx_tab.p, part,
+        reinterpret_cast<const __half*>(Vop), vsum, h.n, n_pad, ncols, gps, w, h.fx_tab.p, part,
         h.tc_err.p, wait_ns, h.opt.wait_stall ? 1 : 0);
     KPCG_LAUNCHED("kv_fx_kernel");
 }
 
 template <int CPAD, int CU>
-void launch_fx_ks(Ctx& h, const uint8_t* Vop, int64_t n_pad, int ncols, int nsplit, int gps,
+void launch_fx_ks(Ctx& h, const uint8_t* Vop, const int* vsum, int64_t n_pad, int ncols, int nsplit, int gps,
                   double* part, uint64_t wait_ns) {
     if (h.d + 4 <= 16)
-        launch_fx<2, 1, CPAD, CU>(h, Vop, n_pad, ncols, nsplit, gps, part, wait_ns);
+        launch_fx<2, 1, CPAD, CU>(h, Vop, vsum, n_pad, ncols, nsplit, gps, part, wait_ns);
     else
-        launch_fx<3, 2, CPAD, CU>(h, Vop, n_pad, ncols, nsplit, gps, part, wait_ns);
+        launch_fx<3, 2, CPAD, CU>(h, Vop, vsum, n_pad, ncols, nsplit, gps, part, wait_ns);
 }
 
 // floor(sqrt(v))
@@ -841,6 +885,7 @@ void kv_fx(Ctx& h, const double* V, int64_t ldv, int c, const double* B, int64_t
     const int step = fx_pass(c);
     const int cpad = step <= 8 ? 8 : step <= 16 ? 16 : 24;
     uint8_t* Vop = h.fxV.need((size_t)(n_pad / QG) * QNV * cpad * 128);
+    int* vsum = h.fxVsum.need((size_t)(n_pad / QG) * QNV * cpad);
     double* part = h.fxPart.need((size_t)nsplit * step * n_pad);
     unsigned long long* mx = h.fx_max.need(32);
     for (int k0 = 0; k0 < c; k0 += step) {
@@ -852,17 +897,17 @@ void kv_fx(Ctx& h, const double* V, int64_t ldv, int c, const double* B, int64_t
         KPCG_LAUNCHED("fx_absmax_kernel");
         const int64_t thr = (n_pad / 8) * cpad;
         fx_stage_v_kernel<<<(unsigned)((thr + 127) / 128), 128, 0, st>>>(Vk, ldv, n, n_pad, nc, cpad,
-                                                                         mx, Vop);
+                                                                         mx, Vop, vsum);
         KPCG_LAUNCHED("fx_stage_v_kernel");
         // V is staged at the call's width: a narrow last pass of a wide block keeps that layout
         if (cpad == 8 && nc <= 2)
-            launch_fx_ks<8, 2>(h, Vop, n_pad, nc, nsplit, gps, part, wait_ns);
+            launch_fx_ks<8, 2>(h, Vop, vsum, n_pad, nc, nsplit, gps, part, wait_ns);
         else if (cpad == 8)
-            launch_fx_ks<8, 8>(h, Vop, n_pad, nc, nsplit, gps, part, wait_ns);
+            launch_fx_ks<8, 8>(h, Vop, vsum, n_pad, nc, nsplit, gps, part, wait_ns);
         else if (cpad == 16)
-            launch_fx_ks<16, 16>(h, Vop, n_pad, nc, nsplit, gps, part, wait_ns);
+            launch_fx_ks<16, 16>(h, Vop, vsum, n_pad, nc, nsplit, gps, part, wait_ns);
         else
-            launch_fx_ks<24, 24>(h, Vop, n_pad, nc, nsplit, gps, part, wait_ns);
+            launch_fx_ks<24, 24>(h, Vop, vsum, n_pad, nc, nsplit, gps, part, wait_ns);
         fx_reduce_kernel<<<dim3((unsigned)((n + 127) / 128), (unsigned)nc), 128, 0, st>>>(
             part, n_pad, nsplit, nc, mx, h.s2, h.xs64.p, h.dp, h.c0_64(), Vk, ldv, noise,
             B ? B + (int64_t)k0 * ldb : nullptr, ldb, O + (int64_t)k0 * ldo, ldo, n);
