@@ -236,7 +236,8 @@ kpcg_status kpcg_precond_pitc(kpcg_t h, int64_t m, const int64_t* idx, int64_t b
  * fixed point on the tensor cores (exact level sums of 10-bit slices of x',
  * entries good to 2^-54 of their size and to 2^-63 s^2, digits of V to 2^-63 of
  * its column's largest value, sums without rounding: an error against the
- * largest entry and value, where FP64 errs against each entry's), else entries
+ * largest entry and value, where FP64 errs against each entry's; columns of at
+ * most 32 values, as unit vectors, are summed from FP64 entries), else entries
  * and sums in native FP64;
  * impl 1: the double-float product of KPCG_DF64 and of the outer loop of the
  * mixed modes (FP32-pair arithmetic, about 44 bits per entry, sums carried as

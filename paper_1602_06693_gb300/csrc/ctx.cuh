@@ -163,7 +163,7 @@ struct Ctx {
     double fx_S = 0.0;
     DevBuf<uint8_t> fxA, fxB, fxV;
     DevBuf<uint64_t> fx_tab;
-    DevBuf<unsigned long long> fx_max;
+    DevBuf<uint8_t> fxCols;
     DevBuf<int> fxVsum;
     DevBuf<double> fxPart;
     // per-point-exact tensor-core operands (kv_tcx_apply), rebuilt when theta changes

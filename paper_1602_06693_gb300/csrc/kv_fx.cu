@@ -74,6 +74,7 @@
 
 #include <algorithm>
 #include <cmath>
+#include <cstddef>
 #include <cstring>
 #include <vector>
 
@@ -98,6 +99,16 @@ constexpr int QMAXC = 24;    // columns of V per pass
 constexpr uint32_t kLevT = 0, kByteT = QNS * QU, kSumT = kByteT + QNK * QU / 2;
 // 64-column groups per work item at most: the 32-bit sums take 2^24 per group
 constexpr int kMaxGroups = 120;
+// Columns of V with at most so many values that are not zero go entry by entry
+constexpr int kFew = 32;
+// What is known of a pass's columns of V; all but the lists is cleared before.
+struct FxCols {
+    unsigned long long mx[QMAXC];   // bits of max |v|
+    unsigned long long nnz[QMAXC];  // values that are not zero
+    unsigned got[QMAXC];            // entries of the lists
+    int row[QMAXC][kFew];           // where nnz <= kFew: the values, in any order
+    double val[QMAXC][kFew];
+};
 
 // Integer parts of the table correction: bits(M1) 2^21 + bits(M3) with
 // M1 = 1.5 2^-12 (unit 2^-35) and M3 = 1.5 2^-33 (unit 2^-56), taken off the table's
@@ -519,23 +530,31 @@ __global__ void __launch_bounds__(QWARPS * 32, 1)
 }
 
 // max |x| of an array (as the bits of a non-negative double, which order as
-// unsigned integers; NaN orders above infinity), per column k of the grid.
+// unsigned integers; NaN orders above infinity) and the number of its values that are
+// not zero, per column k of the grid.
 __global__ void fx_absmax_kernel(const double* __restrict__ x, int64_t ldx, int64_t cnt,
-                                 unsigned long long* __restrict__ out) {
+                                 unsigned long long* __restrict__ out,
+                                 unsigned long long* __restrict__ nnz) {
     const int k = blockIdx.y;
     unsigned long long m = 0;
+    unsigned c = 0;
     for (int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; e < cnt;
          e += (int64_t)gridDim.x * blockDim.x) {
         const unsigned long long b =
             (unsigned long long)__double_as_longlong(x[e + (int64_t)k * ldx]) & 0x7fffffffffffffffull;
         m = b > m ? b : m;
+        c += b != 0;
     }
+    c = __reduce_add_sync(0xffffffffu, c);
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) {
         const unsigned long long q = __shfl_xor_sync(0xffffffffu, m, o);
         m = q > m ? q : m;
     }
-    if ((threadIdx.x & 31) == 0 && m) atomicMax(&out[k], m);
+    if ((threadIdx.x & 31) == 0 && m) {
+        atomicMax(&out[k], m);
+        atomicAdd(&nnz[k], (unsigned long long)c);
+    }
 }
 
 // Byte offset of element (r, k) inside a rows x 64 swizzled K-major sub-tile.
@@ -632,12 +651,12 @@ __global__ void fx_prep_kernel(const double* __restrict__ xs64, int64_t n, int64
 // V's columns as eight balanced bytes each, v = 2^e sum_b v_b 2^(-7 - 8b), 2^e > max|v|:
 // per group of 64 rows of V, operand rows (b, column) of 64 FP16, swizzled.  One
 // thread per (group, column, 8 rows).  vsum[group][l][column] = 128 sum of the bytes b < l over
-// the group.  Columns with a value that is not finite are left zero (the reduction
-// computes them entry by entry).
+// the group.  Columns with few values or one that is not finite are left zero (the
+// reduction computes them entry by entry); the few values go to their list.
 __global__ void fx_stage_v_kernel(const double* __restrict__ V, int64_t ldv, int64_t n,
                                   int64_t n_pad, int ncols, int cpad,
-                                  const unsigned long long* __restrict__ mx,
-                                  uint8_t* __restrict__ Vop, int* __restrict__ vsum) {
+                                  FxCols* __restrict__ cols, uint8_t* __restrict__ Vop,
+                                  int* __restrict__ vsum) {
     const int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (e >= (n_pad / 8) * cpad) return;
     // consecutive threads: the 8-row chunks of a column (coalesced reads)
@@ -653,9 +672,22 @@ __global__ void fx_stage_v_kernel(const double* __restrict__ V, int64_t ldv, int
 #pragma unroll
         for (int w = 0; w < 4; ++w) out[b][w] = 0u;
     }
-    if (k < ncols && mx[k] != 0 && mx[k] < 0x7ff0000000000000ull) {
+    const bool few = k < ncols && cols->nnz[k] <= kFew;
+    if (few) {
+#pragma unroll 1
+        for (int64_t j = chunk * 8; j < min(n, chunk * 8 + 8); ++j) {
+            const double v = V[j + (int64_t)k * ldv];
+            if (v != 0.0) {
+                const unsigned at = atomicAdd(&cols->got[k], 1u);
+                if (at < kFew) {
+                    cols->row[k][at] = (int)j;
+                    cols->val[k][at] = v;
+                }
+            }
+        }
+    } else if (k < ncols && cols->mx[k] < 0x7ff0000000000000ull) {
         int ex;
-        (void)frexp(__longlong_as_double((long long)mx[k]), &ex);
+        (void)frexp(__longlong_as_double((long long)cols->mx[k]), &ex);
 #pragma unroll
         for (int r = 0; r < 8; ++r) {
             const int64_t j = chunk * 8 + r;
@@ -687,32 +719,56 @@ __global__ void fx_stage_v_kernel(const double* __restrict__ V, int64_t ldv, int
     }
 }
 
-// O = s^2 2^e (sum of the split partials) + noise V, or B minus that, in FP64.
+// K_ij in FP64
+__device__ __forceinline__ double fx_entry64(const double* __restrict__ xs64, int dp, double c0,
+                                             int64_t i, int64_t j) {
+    double a = c0;
+    for (int r = 0; r < dp; ++r) {
+        const double t = xs64[i * dp + r] - xs64[j * dp + r];
+        a = fma(-t, t, a);
+    }
+    return exp(fmax(a, -708.0));
+}
+
+// O = s^2 2^e (sum of the split partials) + noise V, or B minus that, in FP64.  A column of at
+// most kFew values (a unit vector asks for a column of K, whose entries a cut at an absolute
+// place would not give) is a sum of FP64 entries in the order of the rows: 0.1 ms of FP64 at
+// n = 65536 with all 32.
 __global__ void fx_reduce_kernel(const double* __restrict__ part, int64_t n_pad, int nsplit,
-                                 int ncols, const unsigned long long* __restrict__ mx, double s2,
+                                 int ncols, const FxCols* __restrict__ cols, double s2,
                                  const double* __restrict__ xs64, int dp, double c0,
                                  const double* __restrict__ V, int64_t ldv, double noise,
                                  const double* __restrict__ B, int64_t ldb, double* __restrict__ O,
                                  int64_t ldo, int64_t n) {
+    __shared__ int rows[kFew];
+    __shared__ double vals[kFew];
     const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     const int k = blockIdx.y;
+    const unsigned long long mx = cols->mx[k], nnz = cols->nnz[k];
+    const int nf = nnz <= kFew ? (int)nnz : -1;
+    if (nf >= 0) {  // its values in the order of the rows
+        if ((int)threadIdx.x < nf) {
+            const int row = cols->row[k][threadIdx.x];
+            int rank = 0;
+            for (int u = 0; u < nf; ++u) rank += cols->row[k][u] < row;
+            rows[rank] = row;
+            vals[rank] = cols->val[k][threadIdx.x];
+        }
+        __syncthreads();
+    }
     if (i >= n) return;
     double s = 0.0;
-    if (mx[k] < 0x7ff0000000000000ull) {
+    if (nf >= 0) {
+        for (int u = 0; u < nf; ++u) s = fma(fx_entry64(xs64, dp, c0, i, rows[u]), vals[u], s);
+    } else if (mx < 0x7ff0000000000000ull) {
         for (int sp = 0; sp < nsplit; ++sp) s += part[((size_t)sp * ncols + k) * n_pad + i];
         int ex = 0;
-        if (mx[k]) (void)frexp(__longlong_as_double((long long)mx[k]), &ex);
+        (void)frexp(__longlong_as_double((long long)mx), &ex);
         s = s2 * ldexp(s, ex);
     } else {
         // an infinity or a NaN in the column: every entry in FP64, as IEEE has it
-        for (int64_t j = 0; j < n; ++j) {
-            double a = c0;
-            for (int r = 0; r < dp; ++r) {
-                const double t = xs64[i * dp + r] - xs64[j * dp + r];
-                a = fma(-t, t, a);
-            }
-            s = fma(exp(fmax(a, -708.0)), V[j + (int64_t)k * ldv], s);
-        }
+        for (int64_t j = 0; j < n; ++j)
+            s = fma(fx_entry64(xs64, dp, c0, i, j), V[j + (int64_t)k * ldv], s);
     }
     s = fma(noise, V[i + (int64_t)k * ldv], s);
     O[i + (int64_t)k * ldo] = B ? (B[i + (int64_t)k * ldb] - s) : s;
@@ -778,11 +834,12 @@ void fx_prepare(Ctx& h) {
     if (h.fx_version == h.theta_version) return;
     cudaStream_t st = h.stream;
     const int64_t n = h.n;
-    unsigned long long* mx = h.fx_max.need(32);
+    FxCols* cols = reinterpret_cast<FxCols*>(h.fxCols.need(sizeof(FxCols)));
+    unsigned long long* mx = cols->mx;
     KPCG_CUDA(cudaMemsetAsync(mx, 0, sizeof(unsigned long long), st));
     const int64_t cnt = n * h.dp;
     fx_absmax_kernel<<<(unsigned)std::min<int64_t>((cnt + 1023) / 1024, 608), 256, 0, st>>>(
-        h.xs64.p, 0, cnt, mx);
+        h.xs64.p, 0, cnt, mx, cols->nnz);
     KPCG_LAUNCHED("fx_absmax_kernel");
     unsigned long long bits = 0;
     KPCG_CUDA(cudaMemcpyAsync(&bits, mx, sizeof(bits), cudaMemcpyDeviceToHost, st));
@@ -887,17 +944,17 @@ void kv_fx(Ctx& h, const double* V, int64_t ldv, int c, const double* B, int64_t
     uint8_t* Vop = h.fxV.need((size_t)(n_pad / QG) * QNV * cpad * 128);
     int* vsum = h.fxVsum.need((size_t)(n_pad / QG) * QNV * cpad);
     double* part = h.fxPart.need((size_t)nsplit * step * n_pad);
-    unsigned long long* mx = h.fx_max.need(32);
+    FxCols* cols = reinterpret_cast<FxCols*>(h.fxCols.need(sizeof(FxCols)));
     for (int k0 = 0; k0 < c; k0 += step) {
         const int nc = std::min(step, c - k0);
         const double* Vk = V + (int64_t)k0 * ldv;
-        KPCG_CUDA(cudaMemsetAsync(mx, 0, sizeof(unsigned long long) * nc, st));
+        KPCG_CUDA(cudaMemsetAsync(cols, 0, offsetof(FxCols, row), st));
         fx_absmax_kernel<<<dim3((unsigned)std::min<int64_t>((n + 1023) / 1024, 152), (unsigned)nc),
-                           256, 0, st>>>(Vk, ldv, n, mx);
+                           256, 0, st>>>(Vk, ldv, n, cols->mx, cols->nnz);
         KPCG_LAUNCHED("fx_absmax_kernel");
         const int64_t thr = (n_pad / 8) * cpad;
         fx_stage_v_kernel<<<(unsigned)((thr + 127) / 128), 128, 0, st>>>(Vk, ldv, n, n_pad, nc, cpad,
-                                                                         mx, Vop, vsum);
+                                                                         cols, Vop, vsum);
         KPCG_LAUNCHED("fx_stage_v_kernel");
         // V is staged at the call's width: a narrow last pass of a wide block keeps that layout
         if (cpad == 8 && nc <= 2)
@@ -909,7 +966,7 @@ void kv_fx(Ctx& h, const double* V, int64_t ldv, int c, const double* B, int64_t
         else
             launch_fx_ks<24, 24>(h, Vop, vsum, n_pad, nc, nsplit, gps, part, wait_ns);
         fx_reduce_kernel<<<dim3((unsigned)((n + 127) / 128), (unsigned)nc), 128, 0, st>>>(
-            part, n_pad, nsplit, nc, mx, h.s2, h.xs64.p, h.dp, h.c0_64(), Vk, ldv, noise,
+            part, n_pad, nsplit, nc, cols, h.s2, h.xs64.p, h.dp, h.c0_64(), Vk, ldv, noise,
             B ? B + (int64_t)k0 * ldb : nullptr, ldb, O + (int64_t)k0 * ldo, ldo, n);
         KPCG_LAUNCHED("fx_reduce_kernel");
     }
