@@ -330,34 +330,42 @@ __global__ void __launch_bounds__(SWARPS_TCS * 32, 1)
 // fixed order, rounded to FP32.  A CTA takes the 128 rows of one tile, eight groups
 // of threads every eighth partial each, with TwoSum on FP32 pairs (2^-47; two FP64
 // additions per clock and SM made the FP64 sum of all partials 0.25 of the product's
-// 0.82 ms at n = 65536; this takes 0.02 ms), the groups' sums in FP64.
+// 0.82 ms at n = 65536; this takes 0.02 ms), the groups' sums in FP64.  Where an infinity or
+// an overflow on the way has spoilt a pair, the group's partials are added in FP64.
 __global__ void __launch_bounds__(1024)
     tcs_reduce_kernel(const float* __restrict__ prow, const float* __restrict__ pcol,
                       const int* __restrict__ col_start, const int* __restrict__ col_items,
                       int64_t n_t, const float* __restrict__ V, float noise,
                       float* __restrict__ O, int64_t n) {
-    __shared__ float2 red[8][TM];
+    __shared__ double red[8][TM];
     const int64_t a = blockIdx.x;
     const int r = threadIdx.x & (TM - 1), g = threadIdx.x / TM;
     float s = 0.f, c = 0.f;
-    auto add = [&](float x) {
+    auto each = [&](auto&& add) {
+#pragma unroll 4
+        for (int64_t J = a / 2 + g; J < (n_t + 1) / 2; J += 8) add(prow[tcs_pair(J, a) * TM + r]);
+#pragma unroll 4
+        for (int e = col_start[a / 2] + g; e < col_start[a / 2 + 1]; e += 8)
+            add(pcol[(size_t)col_items[e] * SN + (a & 1) * TN + r]);
+    };
+    each([&](float x) {
         const float t = s + x;
         const float z = t - s;
         c += (s - (t - z)) + (x - z);
         s = t;
-    };
-#pragma unroll 4
-    for (int64_t J = a / 2 + g; J < (n_t + 1) / 2; J += 8) add(prow[tcs_pair(J, a) * TM + r]);
-#pragma unroll 4
-    for (int e = col_start[a / 2] + g; e < col_start[a / 2 + 1]; e += 8)
-        add(pcol[(size_t)col_items[e] * SN + (a & 1) * TN + r]);
-    red[g][r] = make_float2(s, c);
+    });
+    double sum = (double)s + (double)c;
+    if (!isfinite(sum)) {
+        sum = 0.0;
+        each([&](float x) { sum += (double)x; });
+    }
+    red[g][r] = sum;
     __syncthreads();
     const int64_t i = a * TM + r;
     if (g != 0 || i >= n) return;
     double o = (double)noise * (double)V[i];
 #pragma unroll
-    for (int q = 0; q < 8; ++q) o += (double)red[q][r].x + (double)red[q][r].y;
+    for (int q = 0; q < 8; ++q) o += red[q][r];
     O[i] = (float)o;
 }
 
