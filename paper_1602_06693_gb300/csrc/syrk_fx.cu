@@ -88,7 +88,9 @@ __global__ void syrk_digits_kernel(const float2* __restrict__ KXU, int64_t n, in
     const int64_t cols = ct * 128;
     if (e >= nrows / 8 * cols) return;
     const int64_t a = e % cols, r8 = e / cols;  // consecutive threads: consecutive columns
-    const float sc = exp2f((float)(7 - pair_exponent(*mx)));
+    // 2^(7 - exponent) from its bits: the products below and the epilogue's way back
+    // rely on an exact power of two, exp2f promises two ulps.  The exponent is -100 .. 130.
+    const float sc = __int_as_float((127 + 7 - pair_exponent(*mx)) << 23);
     float h[8], l[8];
 #pragma unroll
     for (int r = 0; r < 8; ++r) {
