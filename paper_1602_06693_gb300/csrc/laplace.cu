@@ -384,6 +384,15 @@ kpcg_status kpcg_laplace(kpcg_t h, const double* y, double newton_tol, int32_t m
         KPCG_CUDA(cudaMemsetAsync(a, 0, sizeof(double) * ld, st));
         const unsigned g = lap_grid(n);
         const bool pre = c.pkind == KPCG_PREC_NYSTROM;
+        // P_B is built two or three times: its scratch lives for the fit
+        struct KeepDigits {
+            PrecondState& P;
+            explicit KeepDigits(PrecondState& p) : P(p) { P.keep_digits = true; }
+            ~KeepDigits() {
+                P.keep_digits = false;
+                P.digits.release();
+            }
+        } keep_digits(c.LP);
         const VecOp mvB = make_bop(&c, sW, u, w);
         const VecOp pcB = make_bpc(&c, pre);
         // mixed precision (KPCG_TC_IR / KPCG_FP32_IR): FP32 W^1/2 and scratch

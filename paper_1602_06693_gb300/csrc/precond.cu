@@ -705,6 +705,7 @@ static void nys_syrk_factor(PrecondState& P, int64_t n, int64_t m, cudaStream_t 
     int bad = 0;
     KPCG_CUDA(cudaMemcpyAsync(&bad, late, sizeof(int), cudaMemcpyDeviceToHost, st));
     KPCG_CUDA(cudaStreamSynchronize(st));
+    if (!P.keep_digits) P.digits.release();
     if (bad) fail(KPCG_ERR_TIMEOUT, "a bounded wait in the Nystrom set-up expired");
     P.jitter = factor_with_rule(P, M0, m, st, what);
 }

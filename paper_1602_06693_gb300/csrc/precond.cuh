@@ -22,7 +22,10 @@ struct PrecondState {
     DevBuf<double> M;        // Cholesky factor(s) L
     DevBuf<double> U;        // L^{-T}, row-major (per block for block-Jacobi)
     DevBuf<double> scratch;  // split partials of the set-up products
-    DevBuf<uint8_t> digits;  // row blocks of K_XU as digits (syrk_fx.cu)
+    // row blocks of K_XU as digits (syrk_fx.cu), up to 96 MB, given back after a set-up (a
+    // batch keeps many preconditioners) unless further set-ups follow at once
+    DevBuf<uint8_t> digits;
+    bool keep_digits = false;
     DevBuf<double> wpart, w, y;
     DevBuf<int> status;
     // test hook of the set-up's bounded waits: > 0 lets one run out after so many ns
