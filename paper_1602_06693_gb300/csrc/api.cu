@@ -14,6 +14,7 @@
 #include "kpcg_internal.cuh"
 #include "ctx.cuh"
 #include "precond.cuh"
+#include "smem_limits.h"
 #include "solver.cuh"
 
 namespace kpcg {
@@ -29,6 +30,15 @@ void cuda_check(cudaError_t e, const char* what, const char* file, int line) {
 }
 
 static thread_local long long g_launches = 0;
+void allow_smem_of(const void* kern, size_t bytes) {
+    static SmemLimits limits;
+    int dev = 0;
+    KPCG_CUDA(cudaGetDevice(&dev));
+    limits.allow(dev, kern, bytes, [&] {
+        KPCG_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                       (int)bytes));
+    });
+}
 void note_launch() { ++g_launches; }
 void note_launches(long long k) { g_launches += k; }
 bool trace_on() {

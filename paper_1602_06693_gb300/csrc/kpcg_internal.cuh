@@ -42,6 +42,13 @@ inline std::atomic<long long>& buffer_epoch() {
     return e;
 }
 
+// Allows a kernel `bytes` of dynamic shared memory on the current device.
+void allow_smem_of(const void* kern, size_t bytes);
+template <typename... A>
+void allow_smem(void (*kern)(A...), size_t bytes) {
+    allow_smem_of(reinterpret_cast<const void*>(kern), bytes);
+}
+
 // A device allocation owned by RAII.
 template <typename T>
 struct DevBuf {

@@ -850,12 +850,7 @@ static void df_sym_launch1(const float4* xs, int64_t n, int nt, float c0h, float
                            const int4* work, int nwork, int G, int nchunk, double* prow,
                            double* pcol, cudaStream_t st) {
     const size_t smem = df_sym_smem<DP, CB>();
-    static bool attr = false;
-    if (!attr) {
-        KPCG_CUDA(cudaFuncSetAttribute(kv_df_sym_kernel<DP, CB>,
-                                       cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-        attr = true;
-    }
+    allow_smem(kv_df_sym_kernel<DP, CB>, smem);
     kv_df_sym_kernel<DP, CB><<<nwork, ST, smem, st>>>(xs, n, nt, c0h, c0l, V, ldv, ncols, tab,
                                                       work, G, nchunk, prow, pcol);
     KPCG_LAUNCHED("kv_df_sym_kernel");
@@ -942,12 +937,7 @@ static void f64_sym_launch1(const double* xs, int64_t n, int nt, double c0, cons
                             double* prow, double* pcol, const double* tab64, cudaStream_t st) {
     const size_t smem =
         sizeof(double) * (ST * DP + ST * CB + CB * ST * (SCW + 1) + CB * 4 * SCW + NTAB64);
-    static bool attr = false;
-    if (!attr) {
-        KPCG_CUDA(cudaFuncSetAttribute(kv_f64_sym_kernel<DP, CB>,
-                                       cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-        attr = true;
-    }
+    allow_smem(kv_f64_sym_kernel<DP, CB>, smem);
     kv_f64_sym_kernel<DP, CB><<<nwork, ST, smem, st>>>(xs, n, nt, c0, V, ldv, ncols, work, G,
                                                        nchunk, prow, pcol, tab64);
     KPCG_LAUNCHED("kv_f64_sym_kernel");
@@ -1077,12 +1067,7 @@ static void xf_sym_launch1(const float2* xs, int64_t n, int nt, float c0, const 
                            double* prow, double* pcol, cudaStream_t st) {
     const size_t smem = sizeof(float2) * ST * DP + sizeof(float) * ST * CB +
                         sizeof(float) * CB * ST * (SCW + 1) + sizeof(float2) * CB * 4 * SCW;
-    static bool attr = false;
-    if (!attr) {
-        KPCG_CUDA(cudaFuncSetAttribute(kv_xf_sym_kernel<DP, CB, EXPP>,
-                                       cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-        attr = true;
-    }
+    allow_smem(kv_xf_sym_kernel<DP, CB, EXPP>, smem);
     kv_xf_sym_kernel<DP, CB, EXPP><<<nwork, ST, smem, st>>>(xs, n, nt, c0, V, ldv, ncols, work, G,
                                                             nchunk, prow, pcol);
     KPCG_LAUNCHED("kv_xf_sym_kernel");

@@ -778,12 +778,7 @@ template <int SUBT, int KS, int CPAD, int CU>
 void launch_fx(Ctx& h, const uint8_t* Vop, const int* vsum, int64_t n_pad, int ncols, int nsplit, int gps,
                double* part, uint64_t wait_ns) {
     using S = FxSmem<SUBT, CPAD>;
-    static const bool attr = [] {
-        KPCG_CUDA(cudaFuncSetAttribute(kv_fx_kernel<SUBT, KS, CPAD, CU>,
-                                       cudaFuncAttributeMaxDynamicSharedMemorySize, S::kTotal));
-        return true;
-    }();
-    (void)attr;
+    allow_smem(kv_fx_kernel<SUBT, KS, CPAD, CU>, S::kTotal);
     const float w0 = (float)std::ldexp(h.fx_S * h.fx_S, -17);
     const FxScale w{w0, w0 * 0x1p-10f, w0 * 0x1p-20f, w0 * 0x1p-30f, w0 * 0x1p-40f};
     kv_fx_kernel<SUBT, KS, CPAD, CU><<<dim3((unsigned)(n_pad / 128), (unsigned)nsplit), QWARPS * 32,

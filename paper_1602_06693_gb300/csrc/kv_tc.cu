@@ -567,12 +567,7 @@ void launch_tc(const Ctx& h, const __nv_bfloat16* A, const __nv_bfloat16* B, con
     const uint64_t wait_ns =
         h.opt.wait_limit_ns > 0 ? (uint64_t)h.opt.wait_limit_ns : kWaitNs;
     using S = TcSmem<KCH, CB, EXACT == 2 ? 2 : 1>;
-    static bool attr = false;
-    if (!attr) {
-        KPCG_CUDA(cudaFuncSetAttribute(kv_tc_kernel<KCH, CB, EXACT>,
-                                       cudaFuncAttributeMaxDynamicSharedMemorySize, S::kTotal));
-        attr = true;
-    }
+    allow_smem(kv_tc_kernel<KCH, CB, EXACT>, S::kTotal);
     dim3 grid((unsigned)(n_pad / TM), (unsigned)nsplit);
     kv_tc_kernel<KCH, CB, EXACT><<<grid, NWARPS * 32, S::kTotal, st>>>(
         A, B, Vs, h.n, n_pad, ncols, tps, part, err, nmma, escale, part64, wait_ns,
@@ -1166,12 +1161,7 @@ __global__ void tc_batch_reduce_kernel(const TcBatchProb* __restrict__ probs,
 template <int CB>
 void launch_tc_batch(TcBatch& b, int ncols, const int* active, int cpp, cudaStream_t st) {
     using S = TcBSmem<CB>;
-    static bool attr = false;
-    if (!attr) {
-        KPCG_CUDA(cudaFuncSetAttribute(kv_tc_batch_kernel<CB>,
-                                       cudaFuncAttributeMaxDynamicSharedMemorySize, S::kTotal));
-        attr = true;
-    }
+    allow_smem(kv_tc_batch_kernel<CB>, S::kTotal);
     const int grid = std::max(1, std::min(b.grid, b.nitems));
     kv_tc_batch_kernel<CB><<<grid, NWARPS * 32, S::kTotal, st>>>(
         b.probs.p, b.items.p, b.nitems, b.Vs.p, b.nv, ncols, active, cpp, b.part.p, b.err.p);

@@ -869,12 +869,7 @@ template <int KCH, int CB>
 void launch_tcd(const Ctx& h, const TcdLayout& L, const float2* Vs, int64_t na_pad,
                 int64_t nb_pad, int ncols, double* part, int nsplit, int tps, cudaStream_t st) {
     using S = TcdSmem<KCH, CB>;
-    static bool attr = false;
-    if (!attr) {
-        KPCG_CUDA(cudaFuncSetAttribute(kv_tcd_kernel<KCH, CB>,
-                                       cudaFuncAttributeMaxDynamicSharedMemorySize, S::kTotal));
-        attr = true;
-    }
+    allow_smem(kv_tcd_kernel<KCH, CB>, S::kTotal);
     const uint64_t wait_ns = h.opt.wait_limit_ns > 0 ? (uint64_t)h.opt.wait_limit_ns : kWaitNs;
     dim3 grid((unsigned)(na_pad / 128), (unsigned)nsplit);
     kv_tcd_kernel<KCH, CB><<<grid, DWARPS * 32, S::kTotal, st>>>(
@@ -905,12 +900,7 @@ template <int KCH, int CB>
 void launch_tcds(const Ctx& h, const TcdLayout& L, const float2* Vs, int64_t n_pad, int ncols,
                  double* prow, double* pcol, cudaStream_t st) {
     using S = TcdsSmem<KCH, CB>;
-    static bool attr = false;
-    if (!attr) {
-        KPCG_CUDA(cudaFuncSetAttribute(kv_tcds_kernel<KCH, CB>,
-                                       cudaFuncAttributeMaxDynamicSharedMemorySize, S::kTotal));
-        attr = true;
-    }
+    allow_smem(kv_tcds_kernel<KCH, CB>, S::kTotal);
     const uint64_t wait_ns = h.opt.wait_limit_ns > 0 ? (uint64_t)h.opt.wait_limit_ns : kWaitNs;
     kv_tcds_kernel<KCH, CB><<<(unsigned)h.tcds_nitems, SWARPS * 32, S::kTotal, st>>>(
         reinterpret_cast<const __nv_bfloat16*>(h.tcdA.p),

@@ -380,12 +380,7 @@ __global__ void tcs_stage_v_kernel(const float* __restrict__ V, int64_t n, int64
 template <int KCH>
 void launch_tcs(const Ctx& h, const float* Vs, float* prow, float* pcol, cudaStream_t st) {
     using S = TcsSmem<KCH>;
-    static bool attr = false;
-    if (!attr) {
-        KPCG_CUDA(cudaFuncSetAttribute(kv_tcs_kernel<KCH>,
-                                       cudaFuncAttributeMaxDynamicSharedMemorySize, S::kTotal));
-        attr = true;
-    }
+    allow_smem(kv_tcs_kernel<KCH>, S::kTotal);
     const uint64_t wait_ns = h.opt.wait_limit_ns > 0 ? (uint64_t)h.opt.wait_limit_ns : kWaitNs;
     kv_tcs_kernel<KCH><<<(unsigned)h.tcs_nitems, SWARPS_TCS * 32, S::kTotal, st>>>(
         reinterpret_cast<const __nv_bfloat16*>(h.tcA.p),

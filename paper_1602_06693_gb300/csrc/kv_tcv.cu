@@ -438,12 +438,7 @@ void launch_tcv(const Ctx& h, const __nv_bfloat16* A, const __nv_bfloat16* B, co
                 int64_t n_pad, int ncols, float* part, int nsplit, int tps, cudaStream_t st) {
     const uint64_t wait_ns = h.opt.wait_limit_ns > 0 ? (uint64_t)h.opt.wait_limit_ns : kWaitNs;
     using S = TcvSmem<KCH, NB>;
-    static bool attr = false;
-    if (!attr) {
-        KPCG_CUDA(cudaFuncSetAttribute(kv_tcv_kernel<KCH, NB>,
-                                       cudaFuncAttributeMaxDynamicSharedMemorySize, S::kTotal));
-        attr = true;
-    }
+    allow_smem(kv_tcv_kernel<KCH, NB>, S::kTotal);
     dim3 grid((unsigned)(n_pad / TM), (unsigned)nsplit);
     kv_tcv_kernel<KCH, NB><<<grid, VWARPS * 32, S::kTotal, st>>>(
         A, B, Vop, h.n, n_pad, ncols, tps, part, h.tc_err.p, wait_ns, h.opt.wait_stall ? 1 : 0,
@@ -918,12 +913,7 @@ __global__ void tcv_batch_reduce_kernel(const TcBatchProb* __restrict__ probs,
 template <int NB>
 void launch_tcv_batch(TcBatch& b, int ncols, const int* active, int cpp, cudaStream_t st) {
     using S = TcvSmem<2, NB>;
-    static bool attr = false;
-    if (!attr) {
-        KPCG_CUDA(cudaFuncSetAttribute(kv_tcv_batch_kernel<NB>,
-                                       cudaFuncAttributeMaxDynamicSharedMemorySize, S::kTotal));
-        attr = true;
-    }
+    allow_smem(kv_tcv_batch_kernel<NB>, S::kTotal);
     const int grid = std::max(1, std::min(b.grid, b.nitems));
     kv_tcv_batch_kernel<NB><<<grid, VWARPS * 32, S::kTotal, st>>>(
         b.probs.p, b.items.p, b.nitems, reinterpret_cast<const __half*>(b.Vh.p), ncols, active,

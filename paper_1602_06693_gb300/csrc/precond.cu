@@ -22,7 +22,6 @@
 #include <cuda_runtime.h>
 
 #include <algorithm>
-#include <map>
 #include <utility>
 #include <vector>
 
@@ -31,16 +30,6 @@
 #include "precond.cuh"
 
 namespace kpcg {
-
-// Raise a kernel's dynamic shared-memory limit once per size (the first
-// call runs outside any graph capture; later ones find it raised).
-static void raise_smem_limit(const void* kern, size_t smem) {
-    static std::map<const void*, size_t> done;
-    size_t& have = done[kern];
-    if (smem <= have) return;
-    KPCG_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-    have = smem;
-}
 
 namespace {
 
@@ -993,7 +982,7 @@ void pitc_setup(PrecondState& P, const float* xs32, const double* xs64, int64_t 
     (void)factor_with_rule(P, Kuu, m, st, "K_UU");
     double* V = P.tmp64.need((size_t)n * m);
     const size_t smem = sizeof(double) * (size_t)m;
-    if (smem > 48 * 1024) raise_smem_limit((const void*)pitc_v_kernel, smem);
+    allow_smem(pitc_v_kernel, smem);
     pitc_v_kernel<<<(unsigned)n, 256, smem, st>>>(P.KXU.p, n, m, P.U.p, V);
     KPCG_LAUNCHED("pitc_v_kernel");
     // D = bldiag(K - Q) + noise I and its block factors L_D, U_D = L_D^{-T}
@@ -1097,7 +1086,7 @@ static void nystrom_apply(const PrecondState& P, const T* R, int64_t ldr, int c,
     auto go = [&](auto kern, int rows_per_warp) {
         const int blocks =
             (int)std::min<int64_t>((n + 8 * rows_per_warp - 1) / (8 * rows_per_warp), 152 * 16);
-        if (smem > 48 * 1024) raise_smem_limit((const void*)kern, smem);
+        allow_smem(kern, smem);
         kern<<<blocks, 256, smem, st>>>(P.KXU.p, n, m, w, c, R, ldr, Z, ldz, 1.0 / P.apply_noise);
     };
     if (c == 1)
@@ -1152,7 +1141,7 @@ static void bj_apply(const PrecondState& P, const T* R, int64_t ldr, int c, T* Z
                      cudaStream_t st) {
     const int64_t nb = (P.n + P.b - 1) / P.b;
     const size_t smem = sizeof(double) * 2 * (size_t)P.b;
-    if (smem > 48 * 1024) raise_smem_limit((const void*)bj_apply_kernel<T>, smem);
+    allow_smem(bj_apply_kernel<T>, smem);
     bj_apply_kernel<T><<<dim3((unsigned)nb, c), 256, smem, st>>>(P.U.p, P.n, P.b, R, ldr, Z, ldz);
     KPCG_LAUNCHED("bj_apply_kernel");
 }
@@ -1609,7 +1598,7 @@ void nys_batch_apply(NysBatch& nb, const float* R, int64_t ldr, float* Z, int64_
         const size_t smem = sizeof(float2) * (size_t)nc * (size_t)nb.mmax;
         const bool stage = smem <= 200 * 1024;
         auto go = [&](auto kern) {
-            if (stage && smem > 48 * 1024) raise_smem_limit((const void*)kern, smem);
+            if (stage) allow_smem(kern, smem);
             kern<<<g, 256, stage ? smem : 0, st>>>(nb.probs.p, c, k0, nc, active, nb.u2.p, R, ldr,
                                                    Z, ldz, nrows);
         };

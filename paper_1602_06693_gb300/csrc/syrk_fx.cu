@@ -355,12 +355,7 @@ void syrk_fx(const float2* KXU, int64_t n, int64_t m, DevBuf<uint8_t>& work, dou
     pair_absmax_kernel<<<(unsigned)std::min<int64_t>((n * m + 1023) / 1024, 152 * 8), 256, 0, st>>>(
         KXU, n * m, mx);
     KPCG_LAUNCHED("pair_absmax_kernel");
-    static const bool attr = [] {
-        KPCG_CUDA(cudaFuncSetAttribute(syrk_fx_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                       (int)kSmemY));
-        return true;
-    }();
-    (void)attr;
+    allow_smem(syrk_fx_kernel, kSmemY);
     for (int64_t i0 = 0; i0 < n; i0 += rows) {
         const int64_t here = std::min(rows, (n - i0 + group - 1) / group * group);
         const int64_t thr = here / 8 * ct * 128;
