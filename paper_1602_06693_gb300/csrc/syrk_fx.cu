@@ -13,9 +13,12 @@
 // the others <= 128, so over 128 rows |L_l| < 7.1 x 128 x 2^14 < 2^24.  After every 128
 // rows the levels go into two 64-bit integers per entry (l = 0..3 and 4..7), at the end of
 // a work item to FP64.  What is lost: an entry's digits below 2^-63 S and the levels >= 8
-// (about 2^-64 S^2 per row, of either sign); the sum itself has no rounding.  With seven
-// digits it would be 2^-56 S^2 per row, which for n = 65536 and a narrow kernel is more
-// than the rounding of an FP64 sum.
+// (about 2^-64 S^2 per row, of either sign); the sum itself has no rounding.  On the
+// diagonal the squares d_4(i,a)^2 of level 8 are of one sign, 2^-66 S^2 per row, and made a
+// narrow kernel's entries at n = 65536 up to 1.3e-14 too small (FP64 sums: 2e-16 .. 2e-15):
+// the digits' kernel adds them up beside its work and they go into the sum (6e-17).  With
+// seven digits the levels lost would be 2^-56 S^2 per row, more than the rounding of an
+// FP64 sum.
 //
 // Layout.  syrk_digits_kernel lays the digits of a block of rows out as swizzled K-major
 // operands: per 32 rows and 128 columns of K_XU four sub-tiles of 128 x 128 bytes, two
@@ -79,11 +82,11 @@ __device__ __forceinline__ int pair_exponent(unsigned mx) {
     return max((int)(mx >> 23) - 125, -100);
 }
 
-// Digits of rows i0 .. i0 + nrows - 1 (zero past n and past column m).  One thread per
-// column and 8 rows.
+// Digits of rows i0 .. i0 + nrows - 1 (zero past n and past column m), and the squares of
+// the fifth added to sq, per column.  One thread per column and 8 rows.
 __global__ void syrk_digits_kernel(const float2* __restrict__ KXU, int64_t n, int64_t m, int64_t i0,
                                    int64_t nrows, int64_t ct, const unsigned* __restrict__ mx,
-                                   uint8_t* __restrict__ dig) {
+                                   uint8_t* __restrict__ dig, unsigned long long* __restrict__ sq) {
     const int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     const int64_t cols = ct * 128;
     if (e >= nrows / 8 * cols) return;
@@ -103,6 +106,7 @@ __global__ void syrk_digits_kernel(const float2* __restrict__ KXU, int64_t n, in
     const int c8 = (int)(r8 & 3);      // 16-byte chunk of the 64 bytes of a digit
     const int row = (int)(a & 127);
     uint8_t* base = dig + ((size_t)chunk * ct + (size_t)(a >> 7)) * kTileA + row * 128;
+    float sum4 = 0.f;  // at most 8 x 2^14
 #pragma unroll
     for (int d = 0; d < YND; ++d) {
         uint32_t w[4];
@@ -116,6 +120,7 @@ __global__ void syrk_digits_kernel(const float2* __restrict__ KXU, int64_t n, in
                 const float bb = s - h[r + z];
                 const float e = (h[r + z] - (s - bb)) + (l[r + z] - bb);
                 v[z] = rintf(s);
+                if (d == YND / 2) sum4 = fmaf(v[z], v[z], sum4);
                 h[r + z] = (s - v[z]) * 256.f;
                 l[r + z] = e * 256.f;
             }
@@ -126,6 +131,7 @@ __global__ void syrk_digits_kernel(const float2* __restrict__ KXU, int64_t n, in
         *reinterpret_cast<uint4*>(base + (size_t)(d >> 1) * kSubA + ((c ^ (row & 7)) * 16)) =
             make_uint4(w[0], w[1], w[2], w[3]);
     }
+    if (sum4 > 0.f) atomicAdd(&sq[a], (unsigned long long)sum4);
 }
 
 // Tile x of the lower triangle: rows 128 T .. + 127, columns 64 u .. + 63, u < 2 T + 2.
@@ -137,8 +143,8 @@ __host__ __device__ inline void syrk_tile(int x, int& T, int& u) {
 
 __global__ void __launch_bounds__(YWARPS * 32, 1)
     syrk_fx_kernel(const uint8_t* __restrict__ dig, int64_t m, int ct, int ngroups,
-                   int groups_per_split, const unsigned* __restrict__ mx, int first,
-                   double* __restrict__ part, int* __restrict__ err, uint64_t wait_ns, int stall) {
+                   int groups_per_split, const unsigned* __restrict__ mx,
+                   const unsigned long long* __restrict__ sq, int first, double* __restrict__ part, int* __restrict__ err, uint64_t wait_ns, int stall) {
     extern __shared__ uint8_t smem_raw[];
     uint8_t* smem = reinterpret_cast<uint8_t*>(
         (reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
@@ -291,7 +297,8 @@ __global__ void __launch_bounds__(YWARPS * 32, 1)
 #pragma unroll
             for (int b = 0; b < YN / 2; ++b) {
                 if (b0 + b > a) continue;
-                const double v = fma((double)hi[b], 0x1p-38, (double)lo[b] * 0x1p-70) * sc;
+                double v = fma((double)hi[b], 0x1p-38, (double)lo[b] * 0x1p-70) * sc;
+                if (b0 + b == a && sq && blockIdx.y == 0) v = fma((double)sq[a], 0x1p-78 * sc, v);
                 P[a * m + b0 + b] = first ? v : P[a * m + b0 + b] + v;
             }
     }
@@ -348,10 +355,12 @@ void syrk_fx(const float2* KXU, int64_t n, int64_t m, DevBuf<uint8_t>& work, dou
     const int64_t ub = (m + YN - 1) / YN;
     int tiles = 0;
     for (int64_t T = 0; T < ct; ++T) tiles += (int)std::min(2 * T + 2, ub);
-    uint8_t* w = work.need(256 + (size_t)(rows / YR) * ct * kTileA);
+    const size_t head = 256 + sizeof(unsigned long long) * (size_t)ct * 128;
+    uint8_t* w = work.need(head + (size_t)(rows / YR) * ct * kTileA);
     unsigned* mx = reinterpret_cast<unsigned*>(w);
-    uint8_t* dig = w + 256;
-    KPCG_CUDA(cudaMemsetAsync(mx, 0, sizeof(unsigned), st));
+    unsigned long long* sq = reinterpret_cast<unsigned long long*>(w + 256);
+    uint8_t* dig = w + head;
+    KPCG_CUDA(cudaMemsetAsync(w, 0, head, st));
     pair_absmax_kernel<<<(unsigned)std::min<int64_t>((n * m + 1023) / 1024, 152 * 8), 256, 0, st>>>(
         KXU, n * m, mx);
     KPCG_LAUNCHED("pair_absmax_kernel");
@@ -360,12 +369,13 @@ void syrk_fx(const float2* KXU, int64_t n, int64_t m, DevBuf<uint8_t>& work, dou
         const int64_t here = std::min(rows, (n - i0 + group - 1) / group * group);
         const int64_t thr = here / 8 * ct * 128;
         syrk_digits_kernel<<<(unsigned)((thr + 255) / 256), 256, 0, st>>>(KXU, n, m, i0, here, ct, mx,
-                                                                          dig);
+                                                                          dig, sq);
         KPCG_LAUNCHED("syrk_digits_kernel");
         const int ngroups = (int)(here / group);
         // every split writes (the first block) or adds to its part, also when it has no rows
         syrk_fx_kernel<<<dim3((unsigned)tiles, (unsigned)nsplit), YWARPS * 32, kSmemY, st>>>(
-            dig, m, (int)ct, ngroups, (ngroups + nsplit - 1) / nsplit, mx, i0 == 0, part, err,
+            dig, m, (int)ct, ngroups, (ngroups + nsplit - 1) / nsplit, mx,
+            i0 + rows >= n ? sq : nullptr, i0 == 0, part, err,
             stall_ns > 0 ? (uint64_t)stall_ns : kWaitNs, stall_ns > 0 ? 1 : 0);
         KPCG_LAUNCHED("syrk_fx_kernel");
     }

@@ -79,3 +79,47 @@ def test_inner_matrix(n, d, m, ell, noise, s2):
         return (e / np.linalg.norm(ref.astype(np.float64), axis=0)).max()
 
     assert err(Z) <= 8.0 * err(yard), (err(Z), err(yard))
+
+
+@pytest.mark.parametrize("n,d,m,ell,noise", [(65536, 8, 16, 0.6, 1e-3), (65536, 8, 12, 0.6, 1e-2),
+                                             (65536, 12, 16, 1.0, 1e-3)])
+def test_narrow_kernel(n, d, m, ell, noise):
+    """Many entries far below the one of size 1: what is cut off each of them must not add up
+    over the n rows.  Six to fifteen units of 1e-15 missing on M's diagonal (the squares
+    of the digits below 2^-32) show as 13 to 27 times the yardstick, which works on K_XU
+    as the library keeps it, in FP32 pairs."""
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    import paper_1602_06693_gb300 as kpcg
+    from paper_1602_06693_gb300 import build
+    build.build()
+    p = synthetic.make_problem(n, d, 11, dist="normal", ell=ell, s2=1.0, noise=noise)
+    idx = synthetic.inducing_subset(n, m, seed=3)
+    Y = p.X.astype(LD) * np.exp(-LD(p.log_theta[0]))
+
+    def K(A, B):
+        return np.exp(-sum((A[:, r][:, None] - B[:, r][None]) ** 2 for r in range(d)) / 2)
+
+    kxu, kuu = K(Y, Y[idx]), K(Y[idx], Y[idx])
+    at = np.array([0, 1, 7, n // 3, n - 1, idx[0], idx[m // 2], idx[-1]])
+    R = np.zeros((n, len(at)))
+    R[at, np.arange(len(at))] = 1.0
+    ref = (R.astype(LD) - kxu @ _solve(_factor(LD(noise) * kuu + kxu.T @ kxu), kxu[at].T)) / LD(noise)
+    k64 = kxu.astype(np.float64)
+    hi = k64.astype(np.float32)
+    k64 = hi.astype(np.float64) + (k64 - hi).astype(np.float32)
+    S = np.zeros((m, m))
+    for i in range(0, n, 512):
+        S += k64[i:i + 512].T @ k64[i:i + 512]
+    u = _solve(np.linalg.cholesky(noise * kuu.astype(np.float64) + S), k64[at].T.copy())
+    yard = (R.astype(LD) - k64.astype(LD) @ u.astype(LD)) / LD(noise)
+    opt = kpcg.default_options(precision=kpcg.KPCG_FP64)
+    with kpcg.Solver(torch.from_numpy(p.X).cuda(), p.log_theta, p.noise, options=opt) as s:
+        s.precond(kpcg.KPCG_PREC_NYSTROM, m, idx)
+        Z = s.precond_apply(torch.from_numpy(np.ascontiguousarray(R.T)).cuda().t()).cpu().numpy()
+
+    def err(z):
+        e = np.linalg.norm((z - ref).astype(np.float64), axis=0)
+        return (e / np.linalg.norm(ref.astype(np.float64), axis=0)).max()
+
+    assert err(Z) <= 8.0 * err(yard), (err(Z), err(yard))
