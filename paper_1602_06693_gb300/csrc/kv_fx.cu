@@ -665,10 +665,10 @@ __global__ void fx_stage_v_kernel(const double* __restrict__ V, int64_t ldv, int
     const int64_t g = chunk >> 3;
     const int c8 = (int)(chunk & 7);
     uint32_t out[QNV][4];
-    int sum[QNV];
+    float sum[QNV];  // at most 64 x 128 over a group
 #pragma unroll
     for (int b = 0; b < QNV; ++b) {
-        sum[b] = 0;
+        sum[b] = 0.f;
 #pragma unroll
         for (int w = 0; w < 4; ++w) out[b][w] = 0u;
     }
@@ -696,8 +696,9 @@ __global__ void fx_stage_v_kernel(const double* __restrict__ V, int64_t ldv, int
             for (int b = 0; b < QNV; ++b) {
                 const double v = rint(h);
                 h = (h - v) * 256.0;
-                sum[b] += (int)v;
-                const uint32_t bits = __half_as_ushort(__float2half_rn((float)v));
+                const float vf = (float)v;
+                sum[b] += vf;
+                const uint32_t bits = __half_as_ushort(__float2half_rn(vf));
                 out[b][r >> 1] |= bits << (16 * (r & 1));
             }
         }
@@ -715,7 +716,7 @@ __global__ void fx_stage_v_kernel(const double* __restrict__ V, int64_t ldv, int
 #pragma unroll
         for (int o = 4; o > 0; o >>= 1) sum[b] += __shfl_xor_sync(0xffffffffu, sum[b], o);
         if (c8 == 0) vsum[((size_t)g * QNV + b) * cpad + k] = 128 * above;
-        above += sum[b];
+        above += (int)sum[b];
     }
 }
 
