@@ -957,8 +957,10 @@ void kv_f64_sym(Ctx& h, const double* V, int64_t ldv, int c, const double* B, in
                 double* O, int64_t ldo, double noise) {
     if (h.n <= 0 || c <= 0) return;
     // the fixed-point tensor-core product wherever its operands keep FP64 accuracy
-    // (|y| <= 8: the dropped levels stay near 2^-53 of an entry): 12.1 ms against
-    // 119.6 ms at n = 65536, d = 8 and 0.07 against 0.18 ms at n = 200, one column
+    // (|y| <= 8, inputs within 9.4 lengthscales of their mean: the dropped levels stay near
+    // 2^-53 of an entry): 12.9 ms against 119.6 ms at n = 65536, d = 8 and 0.07 against
+    // 0.18 ms at n = 200, one column.  Beyond that range the step back to the FP64 pipe is
+    // a factor of nine; wider slices would need a seventh level of the distance
     if (kv_fx_usable(h, c, 8.0)) {
         kv_fx(h, V, ldv, c, B, ldb, O, ldo, noise, false);
         return;
@@ -1011,13 +1013,15 @@ void kv_df(Ctx& h, const double* V, int64_t ldv, int c, const double* B, int64_t
            int64_t ldo, double noise) {
     if (h.n <= 0 || c <= 0) return;
     // the fixed-point product (kv_fx.cu; one time for any number of columns) where it is
-    // the faster one: from three columns on (n = 65536, d = 8: 13.0 against
-    // 20.9 ms at three, 14.8 against 40.8 ms at nine; 12.2 against 11.2 ms at two),
+    // the faster one: from three columns on (n = 65536, d = 8: 13.9 against
+    // 20.9 ms at three, 15.2 against 40.8 ms at nine; 12.9 against 10.1 ms at two),
     // for d > 10, whose distances the kernels below take from the FP32 pipe (d = 14,
-    // one column, n = 16384: 0.92 against 1.63 ms), and for few row tiles
-    // (n = 2000, one column: 0.077 against 0.097 ms).  Up to |y| = 64 its dropped levels
-    // stay below the 2^-45 of a double-float entry.
-    if (h.df_tensor && (c >= 3 || h.d > 10 || h.n <= 2048) && kv_fx_usable(h, c, 64.0)) {
+    // one column, n = 16384: 0.94 against 1.63 ms), and for few row tiles, as calls
+    // (n = 500 .. 2000, d = 8, one column: 67 .. 82 against 88 .. 92 us; 2100: 88 against
+    // 93) but not for one or two (n = 50: 66 against 51, n = 200: 67 against 64).  Up to
+    // |y| = 64 its dropped levels stay below the 2^-45 of a double-float entry.
+    const bool few_tiles = h.n > 256 && h.n <= 2048;
+    if (h.df_tensor && (c >= 3 || h.d > 10 || few_tiles) && kv_fx_usable(h, c, 64.0)) {
         kv_fx(h, V, ldv, c, B, ldb, O, ldo, noise, true);
         return;
     }

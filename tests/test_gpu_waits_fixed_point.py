@@ -83,3 +83,18 @@ def test_last_residual_of_a_solve(kpcg, precision, max_iter):
         s.matvec_f64(y, impl=0)  # the flag is cleared
         x, _, info, st = s.solve(y, tol=1e-8)
         assert st == 0 and info.max_rel_res <= 1e-8
+
+
+@pytest.mark.parametrize("n,fixed", [(50, False), (256, False), (257, True), (2048, True),
+                                     (2049, False)])
+def test_where_the_double_float_product_takes_it(kpcg, n, fixed):
+    """One column, d <= 10: only a few row tiles go to the fixed-point kernel, which the test
+    hook of the waits tells from the double-float ones; fewer or more are slower there."""
+    p = synthetic.make_problem(n, 8, 5, dist="normal", ell=3.0, noise=1e-2)
+    V = torch.from_numpy(synthetic.rng(3).standard_normal(n)).cuda()
+    with kpcg.Solver(torch.from_numpy(p.X).cuda(), p.log_theta, p.noise, ard=p.ard) as s:
+        s.set_options(kpcg.default_options(**STALL))
+        if fixed:
+            _timeout(kpcg, lambda: s.matvec_f64(V, impl=1))
+        else:
+            s.matvec_f64(V, impl=1)
