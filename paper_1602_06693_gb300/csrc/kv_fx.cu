@@ -763,9 +763,10 @@ __global__ void fx_reduce_kernel(const double* __restrict__ part, int64_t n_pad,
         for (int u = 0; u < nf; ++u) s = fma(fx_entry64(xs64, dp, c0, i, rows[u]), vals[u], s);
     } else if (mx < 0x7ff0000000000000ull) {
         for (int sp = 0; sp < nsplit; ++sp) s += part[((size_t)sp * ncols + k) * n_pad + i];
-        int ex = 0;
+        // one power of two for V and s^2: neither alone may leave the range that O keeps
+        int ex = 0, e2 = 0;
         (void)frexp(__longlong_as_double((long long)mx), &ex);
-        s = s2 * ldexp(s, ex);
+        s = ldexp(frexp(s2, &e2) * s, ex + e2);
     } else {
         // an infinity or a NaN in the column: every entry in FP64, as IEEE has it
         for (int64_t j = 0; j < n; ++j)
