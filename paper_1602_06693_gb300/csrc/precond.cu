@@ -375,10 +375,12 @@ __device__ __forceinline__ void nys_proj_body(const float2* __restrict__ KXU, in
 __host__ __device__ inline int proj_aw(int64_t m) { return m <= 32 ? 32 : m <= 64 ? 64 : m <= 128 ? 128 : 256; }
 
 // Rows per CTA of the projection: eight CTAs per SM over the whole call (`work` =
-// sum over problems of column blocks x rows), between 32 and 512 rows.
-int64_t nys_rows_per_split(int64_t work) {
+// sum over problems of column blocks x rows), between 32 and 512 rows, and more where
+// the longest problem (nmax rows) would otherwise have over 65535 ranges, a grid's limit.
+int64_t nys_rows_per_split(int64_t work, int64_t nmax) {
     const int64_t r = (work / (152 * 8) + 31) / 32 * 32;
-    return std::max<int64_t>(32, std::min<int64_t>(512, r));
+    const int64_t least = (nmax + 65535 * 32 - 1) / (65535 * 32) * 32;
+    return std::max<int64_t>(least, std::max<int64_t>(32, std::min<int64_t>(512, r)));
 }
 
 // w_part[s][k][a] = sum_{i in split s} KXU[i][a] R[i][k] for one problem.
@@ -1043,7 +1045,7 @@ static double* nystrom_project(const PrecondState& P, const T* R, int64_t ldr, i
     const int64_t n = P.n, m = P.m;
     const int aw = proj_aw(m);
     const int64_t ablk = (m + aw - 1) / aw;
-    const int64_t rps = nys_rows_per_split(ablk * n);
+    const int64_t rps = nys_rows_per_split(ablk * n, n);
     const int nsplit = (int)((n + rps - 1) / rps);
     double* part = const_cast<PrecondState&>(P).wpart.need((size_t)nsplit * c * m);
     double* w = const_cast<PrecondState&>(P).w.need((size_t)c * m);
@@ -1499,10 +1501,12 @@ void nys_batch_plan(NysBatch& nb, const std::vector<const PrecondState*>& Ps, in
     auto uses = [](const PrecondState& P) {
         return P.ready && (P.kind == KPCG_PREC_NYSTROM || P.kind == KPCG_PREC_SPECTRAL);
     };
-    int64_t work = 0;
-    for (const PrecondState* P : Ps)
+    int64_t work = 0, nmax = 0;
+    for (const PrecondState* P : Ps) {
+        nmax = std::max(nmax, P->n);
         if (uses(*P)) work += (P->m + proj_aw(P->m) - 1) / proj_aw(P->m) * P->n;
-    const int64_t rps = nys_rows_per_split(work);
+    }
+    const int64_t rps = nys_rows_per_split(work, nmax);
     for (int p = 0; p < nb.P; ++p) {
         const PrecondState& P = *Ps[(size_t)p];
         NysBatchProb& q = nb.hprobs[(size_t)p];
