@@ -72,9 +72,9 @@ __global__ void __launch_bounds__(128)
     if (j0 >= bq || status[q]) return;
     const int nb = (int)min((int64_t)NB, bq - j0);
     double* M = A + q * stride + j0 * bq + j0;
-    for (int e = threadIdx.x; e < NB * NB; e += 128) {
-        const int r = e / NB, c = e % NB;  // the identity past nb
-        S[r][c] = (r < nb && c < nb) ? M[r * bq + c] : (r == c ? 1.0 : 0.0);
+    for (int e = threadIdx.x; e < nb * nb; e += 128) {
+        const int r = e / nb, c = e % nb;  // what lies past nb reaches nothing before it
+        S[r][c] = M[r * bq + c];
     }
     __syncthreads();
     const int row = threadIdx.x >> 2, part = threadIdx.x & 3;
@@ -83,9 +83,10 @@ __global__ void __launch_bounds__(128)
     for (int v = 0; v < NB / 4; ++v) x[v] = S[row][4 * v + part];
 #pragma unroll
     for (int j = 0; j < NB; ++j) {
+        if (j >= nb) break;
         // column j of rows >= j is final in S
         const double piv = S[j][j];
-        if (j < nb && (!(piv > thr) || !isfinite(piv))) {
+        if (!(piv > thr) || !isfinite(piv)) {
             if (threadIdx.x == 0) status[q] = (int)(j0 + j + 1);
             return;
         }
@@ -131,13 +132,10 @@ __global__ void __launch_bounds__(128)
     if (i0 >= i1) return;
     double* G = (U ? U : A) + q * stride + i0 * bq + j0;
     const int nr = (int)min((int64_t)32, i1 - i0);
-    for (int e = threadIdx.x; e < NB * NB; e += 128) {
-        const int r = e / NB, c = e % NB;
-        L[r][c] = (r < nb && c < nb) ? M[r * bq + c] : (r == c ? 1.0 : 0.0);
-        X[r][c] = (r < nr && c < nb) ? G[r * bq + c] : 0.0;
-    }
+    for (int e = threadIdx.x; e < nb * nb; e += 128) L[e / nb][e % nb] = M[e / nb * bq + e % nb];
+    for (int e = threadIdx.x; e < nr * nb; e += 128) X[e / nb][e % nb] = G[e / nb * bq + e % nb];
     __syncthreads();
-    if (threadIdx.x < NB) inv[threadIdx.x] = 1.0 / L[threadIdx.x][threadIdx.x];
+    if (threadIdx.x < nb) inv[threadIdx.x] = 1.0 / L[threadIdx.x][threadIdx.x];
     __syncthreads();
     const int row = threadIdx.x >> 2, part = threadIdx.x & 3;
     double x[NB / 4];
@@ -145,6 +143,7 @@ __global__ void __launch_bounds__(128)
     for (int v = 0; v < NB / 4; ++v) x[v] = X[row][4 * v + part];
 #pragma unroll
     for (int t = 0; t < NB; ++t) {
+        if (t >= nb) break;
         const double xt = div_by(__shfl_sync(0xffffffffu, x[t / 4], t % 4, 4), L[t][t], inv[t]);
         if (part == t % 4) x[t / 4] = xt;
 #pragma unroll
@@ -154,10 +153,7 @@ __global__ void __launch_bounds__(128)
 #pragma unroll
     for (int v = 0; v < NB / 4; ++v) X[row][4 * v + part] = x[v];
     __syncthreads();
-    for (int e = threadIdx.x; e < NB * NB; e += 128) {
-        const int r = e / NB, c = e % NB;
-        if (r < nr && c < nb) G[r * bq + c] = X[r][c];
-    }
+    for (int e = threadIdx.x; e < nr * nb; e += 128) G[e / nb * bq + e % nb] = X[e / nb][e % nb];
 }
 
 // Trailing update A22 -= L21 L21^T on the lower triangle, or (U given) U2 -= U1 L21^T for the
