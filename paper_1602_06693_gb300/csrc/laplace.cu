@@ -385,14 +385,14 @@ kpcg_status kpcg_laplace(kpcg_t h, const double* y, double newton_tol, int32_t m
         const unsigned g = lap_grid(n);
         const bool pre = c.pkind == KPCG_PREC_NYSTROM;
         // P_B is built two or three times: its scratch lives for the fit
-        struct KeepDigits {
+        struct KeepScratch {
             PrecondState& P;
-            explicit KeepDigits(PrecondState& p) : P(p) { P.keep_digits = true; }
-            ~KeepDigits() {
-                P.keep_digits = false;
-                P.digits.release();
+            explicit KeepScratch(PrecondState& p) : P(p) { P.keep_scratch = true; }
+            ~KeepScratch() {
+                P.keep_scratch = false;
+                P.scratch.release();
             }
-        } keep_digits(c.LP);
+        } keep_scratch(c.LP);
         const VecOp mvB = make_bop(&c, sW, u, w);
         const VecOp pcB = make_bpc(&c, pre);
         // mixed precision (KPCG_TC_IR / KPCG_FP32_IR): FP32 W^1/2 and scratch

@@ -647,12 +647,16 @@ static void nys_gather_kxu(PrecondState& P, const float* xs32, const double* xs6
 // 3e-12 * max diag(A0), else the jitter 1e-12 tr(A0)/m 10^k, k = 0..6, is added;
 // a nearly singular matrix otherwise "factors" or not depending on rounding,
 // and pivots near zero make a useless preconditioner.  Returns the jitter.
+// late (device, may be null): the flag of a wait that expired on the way to A0.
 static double factor_with_rule(PrecondState& P, const double* A0, int64_t m, cudaStream_t st,
-                               const char* what) {
+                               const char* what, const int* late = nullptr) {
     std::vector<double> diag((size_t)m);
     KPCG_CUDA(cudaMemcpy2DAsync(diag.data(), sizeof(double), A0, sizeof(double) * (m + 1),
                                 sizeof(double), (size_t)m, cudaMemcpyDeviceToHost, st));
+    int bad = 0;
+    if (late) KPCG_CUDA(cudaMemcpyAsync(&bad, late, sizeof(int), cudaMemcpyDeviceToHost, st));
     KPCG_CUDA(cudaStreamSynchronize(st));
+    if (bad) fail(KPCG_ERR_TIMEOUT, "a bounded wait in the Nystrom set-up expired");
     double tr = 0.0, dmax = 0.0;
     for (double v : diag) {
         tr += v;
@@ -661,7 +665,7 @@ static double factor_with_rule(PrecondState& P, const double* A0, int64_t m, cud
     const double kPivotTol = 3e-12;
     double* M = P.M.need((size_t)m * m);
     double* U = P.U.need((size_t)m * m);
-    int* status = P.status.need(2);
+    int* status = P.status.need(1);
     int rc = 1;
     double jitter = 0.0;
     for (int k = -1; k <= 6 && rc; ++k) {
@@ -683,18 +687,15 @@ static void nys_syrk_factor(PrecondState& P, int64_t n, int64_t m, cudaStream_t 
                             const char* what) {
     double* M0 = P.M0.p;
     const int nsplit = syrk_fx_splits(n, m);
-    double* part = P.scratch.need((size_t)nsplit * m * m);
-    int* late = P.status.need(2) + 1;
-    KPCG_CUDA(cudaMemsetAsync(late, 0, sizeof(int), st));
-    syrk_fx(P.KXU.p, n, m, P.digits, part, late, P.stall_ns, st);
+    const size_t parts = sizeof(double) * (size_t)nsplit * (size_t)m * (size_t)m;
+    const size_t at = (parts + 255) / 256 * 256;
+    uint8_t* work = P.scratch.need(at + syrk_fx_bytes(n, m));
+    double* part = reinterpret_cast<double*>(work);
+    const int* late = syrk_fx(P.KXU.p, n, m, work + at, part, P.stall_ns, st);
     syrk_reduce_kernel<<<(unsigned)((m * m + 255) / 256), 256, 0, st>>>(part, nsplit, m, M0);
     KPCG_LAUNCHED("syrk_reduce_kernel");
-    int bad = 0;
-    KPCG_CUDA(cudaMemcpyAsync(&bad, late, sizeof(int), cudaMemcpyDeviceToHost, st));
-    KPCG_CUDA(cudaStreamSynchronize(st));
-    if (!P.keep_digits) P.digits.release();
-    if (bad) fail(KPCG_ERR_TIMEOUT, "a bounded wait in the Nystrom set-up expired");
-    P.jitter = factor_with_rule(P, M0, m, st, what);
+    P.jitter = factor_with_rule(P, M0, m, st, what, late);
+    if (!P.keep_scratch) P.scratch.release();
 }
 
 // M0 = noise K_UU + K_UX K_XU, factored by the rule.

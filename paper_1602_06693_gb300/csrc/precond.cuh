@@ -21,11 +21,11 @@ struct PrecondState {
     DevBuf<double> M0;       // sigma^2 K_UU + K_UX K_XU before jitter
     DevBuf<double> M;        // Cholesky factor(s) L
     DevBuf<double> U;        // L^{-T}, row-major (per block for block-Jacobi)
-    DevBuf<double> scratch;  // split partials of the set-up products
-    // row blocks of K_XU as digits (syrk_fx.cu), up to 96 MB, given back after a set-up (a
-    // batch keeps many preconditioners) unless further set-ups follow at once
-    DevBuf<uint8_t> digits;
-    bool keep_digits = false;
+    // split partials of the set-up's sum and row blocks of K_XU as digits (syrk_fx.cu), up to
+    // 96 MB of them, given back after a set-up (a batch keeps many preconditioners)
+    // unless further set-ups follow at once
+    DevBuf<uint8_t> scratch;
+    bool keep_scratch = false;
     DevBuf<double> wpart, w, y;
     DevBuf<int> status;
     // test hook of the set-up's bounded waits: > 0 lets one run out after so many ns
@@ -47,7 +47,6 @@ struct PrecondState {
         M.release();
         U.release();
         scratch.release();
-        digits.release();
         wpart.release();
         w.release();
         y.release();
@@ -108,10 +107,12 @@ void pitc_setup(PrecondState& P, const float* xs32, const double* xs64, int64_t 
 
 // part[s] (s < syrk_fx_splits(n, m), each m x m row-major) = parts of the lower triangle
 // of KXU^T KXU (KXU n x m FP32 pairs) in fixed point on the tensor cores (syrk_fx.cu).
-// err is set if a bounded wait expires; stall_ns > 0 makes one expire (test hook).
+// work: syrk_fx_bytes(n, m), aligned to 256.  Returns the device flag that a bounded wait
+// sets if it expires (in work); stall_ns > 0 makes one expire (test hook).
 int syrk_fx_splits(int64_t n, int64_t m);
-void syrk_fx(const float2* KXU, int64_t n, int64_t m, DevBuf<uint8_t>& work, double* part,
-             int* err, int64_t stall_ns, cudaStream_t st);
+size_t syrk_fx_bytes(int64_t n, int64_t m);
+const int* syrk_fx(const float2* KXU, int64_t n, int64_t m, uint8_t* work, double* part,
+                   int64_t stall_ns, cudaStream_t st);
 
 // ------------------------------------------- batched Nystrom apply
 // Problems laid out column by column (problem p owns columns p*c .. p*c+c-1

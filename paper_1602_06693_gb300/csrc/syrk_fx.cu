@@ -85,10 +85,10 @@ __device__ __forceinline__ int pair_exponent(unsigned mx) {
 // Digits of rows i0 .. i0 + nrows - 1 (zero past n and past column m), and the squares of
 // the fifth added to sq, per column.  One thread per column and 8 rows.
 __global__ void syrk_digits_kernel(const float2* __restrict__ KXU, int64_t n, int64_t m, int64_t i0,
-                                   int64_t nrows, int64_t ct, const unsigned* __restrict__ mx,
+                                   int64_t nrows, int64_t ct, int cw, const unsigned* __restrict__ mx,
                                    uint8_t* __restrict__ dig, unsigned long long* __restrict__ sq) {
     const int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    const int64_t cols = ct * 128;
+    const int64_t cols = ct * cw;
     if (e >= nrows / 8 * cols) return;
     const int64_t a = e % cols, r8 = e / cols;  // consecutive threads: consecutive columns
     // 2^(7 - exponent) from its bits: the products below and the epilogue's way back
@@ -105,7 +105,8 @@ __global__ void syrk_digits_kernel(const float2* __restrict__ KXU, int64_t n, in
     const int64_t chunk = r8 / 4;      // 32 rows
     const int c8 = (int)(r8 & 3);      // 16-byte chunk of the 64 bytes of a digit
     const int row = (int)(a & 127);
-    uint8_t* base = dig + ((size_t)chunk * ct + (size_t)(a >> 7)) * kTileA + row * 128;
+    const uint32_t sub = (uint32_t)cw * 128;
+    uint8_t* base = dig + ((size_t)chunk * ct + (size_t)(a >> 7)) * 4 * sub + row * 128;
     float sum4 = 0.f;  // at most 8 x 2^14
 #pragma unroll
     for (int d = 0; d < YND; ++d) {
@@ -128,7 +129,7 @@ __global__ void syrk_digits_kernel(const float2* __restrict__ KXU, int64_t n, in
             w[r >> 1] = *reinterpret_cast<const uint32_t*>(&p);
         }
         const int c = (d & 1) * 4 + c8;
-        *reinterpret_cast<uint4*>(base + (size_t)(d >> 1) * kSubA + ((c ^ (row & 7)) * 16)) =
+        *reinterpret_cast<uint4*>(base + (size_t)(d >> 1) * sub + ((c ^ (row & 7)) * 16)) =
             make_uint4(w[0], w[1], w[2], w[3]);
     }
     if (sum4 > 0.f) atomicAdd(&sq[a], (unsigned long long)sum4);
@@ -142,7 +143,7 @@ __host__ __device__ inline void syrk_tile(int x, int& T, int& u) {
 }
 
 __global__ void __launch_bounds__(YWARPS * 32, 1)
-    syrk_fx_kernel(const uint8_t* __restrict__ dig, int64_t m, int ct, int ngroups,
+    syrk_fx_kernel(const uint8_t* __restrict__ dig, int64_t m, int ct, int cw, int ngroups,
                    int groups_per_split, const unsigned* __restrict__ mx,
                    const unsigned long long* __restrict__ sq, int first, double* __restrict__ part, int* __restrict__ err, uint64_t wait_ns, int stall) {
     extern __shared__ uint8_t smem_raw[];
@@ -201,14 +202,17 @@ __global__ void __launch_bounds__(YWARPS * 32, 1)
                     break;
                 }
                 uint8_t* st = smem + (size_t)s * kStageY;
-                const uint8_t* row = dig + (size_t)(g0 * YG + t) * ct * kTileA;
-                mbar_expect_tx(&full[s], kStageY);
-                bulk_g2s(st, row + (size_t)T * kTileA, kTileA, &full[s]);
+                const uint32_t sub = (uint32_t)cw * 128;
+                const uint8_t* row = dig + (size_t)(g0 * YG + t) * ct * 4 * sub;
                 // columns 64 u .. + 63: half of every sub-tile of column tile u / 2
-                for (int q = 0; q < 4; ++q)
-                    bulk_g2s(st + kTileA + q * (kSubA / 2),
-                             row + (size_t)(u >> 1) * kTileA + q * kSubA + (u & 1) * (kSubA / 2),
-                             kSubA / 2, &full[s]);
+                const uint32_t half = (uint32_t)(u & 1) * (kSubA / 2);
+                const uint32_t nb = min(kSubA / 2, sub - half);
+                mbar_expect_tx(&full[s], 4 * (sub + nb));
+                for (int q = 0; q < 4; ++q) {
+                    bulk_g2s(st + q * kSubA, row + ((size_t)T * 4 + q) * sub, sub, &full[s]);
+                    bulk_g2s(st + kTileA + q * (kSubA / 2), row + ((size_t)(u >> 1) * 4 + q) * sub + half,
+                             nb, &full[s]);
+                }
             }
             // the CTA exits only once the copies it issued have landed
             const uint64_t dl2 = gtimer() + 200000000ull;
@@ -346,39 +350,61 @@ int syrk_fx_splits(int64_t n, int64_t m) {
     return nsplit;
 }
 
-void syrk_fx(const float2* KXU, int64_t n, int64_t m, DevBuf<uint8_t>& work, double* part,
-             int* err, int64_t stall_ns, cudaStream_t st) {
+// What the work area holds before the digits: the largest entry, the flag of an expired wait,
+// the squares of the fifth digits.
+static size_t syrk_fx_head(int64_t m) {
+    return 256 + sizeof(unsigned long long) * (size_t)((m + 127) / 128 * 128);
+}
+
+// Columns a column tile has in memory: up to 128 the eights that hold m.  What the tiles
+// in shared memory keep past them reaches only rows and columns of the sum past m, which are
+// not stored.  (With 128 of them a set-up of n = 1030, m = 8 worked on 2.4 MB instead of
+// 0.15, and the driver's calls for more than 2 MB are slow: 314 -> 167 us.)
+static int syrk_fx_cols(int64_t m) { return m > 120 ? 128 : (int)((m + 7) / 8 * 8); }
+
+size_t syrk_fx_bytes(int64_t n, int64_t m) {
+    int64_t rows;
+    int nsplit;
+    syrk_fx_plan(n, m, rows, nsplit);
+    return syrk_fx_head(m) +
+           (size_t)(rows / YR) * (size_t)((m + 127) / 128) * (size_t)syrk_fx_cols(m) * 512;
+}
+
+const int* syrk_fx(const float2* KXU, int64_t n, int64_t m, uint8_t* work, double* part,
+                   int64_t stall_ns, cudaStream_t st) {
     const int64_t ct = (m + 127) / 128, group = YR * YG;
+    const int cw = syrk_fx_cols(m);
     int64_t rows;
     int nsplit;
     syrk_fx_plan(n, m, rows, nsplit);
     const int64_t ub = (m + YN - 1) / YN;
     int tiles = 0;
     for (int64_t T = 0; T < ct; ++T) tiles += (int)std::min(2 * T + 2, ub);
-    const size_t head = 256 + sizeof(unsigned long long) * (size_t)ct * 128;
-    uint8_t* w = work.need(head + (size_t)(rows / YR) * ct * kTileA);
-    unsigned* mx = reinterpret_cast<unsigned*>(w);
-    unsigned long long* sq = reinterpret_cast<unsigned long long*>(w + 256);
-    uint8_t* dig = w + head;
-    KPCG_CUDA(cudaMemsetAsync(w, 0, head, st));
+    const size_t head = syrk_fx_head(m);
+    unsigned* mx = reinterpret_cast<unsigned*>(work);
+    int* err = reinterpret_cast<int*>(work + 128);
+    unsigned long long* sq = reinterpret_cast<unsigned long long*>(work + 256);
+    uint8_t* dig = work + head;
+    KPCG_CUDA(cudaMemsetAsync(work, 0, head, st));
     pair_absmax_kernel<<<(unsigned)std::min<int64_t>((n * m + 1023) / 1024, 152 * 8), 256, 0, st>>>(
         KXU, n * m, mx);
     KPCG_LAUNCHED("pair_absmax_kernel");
     allow_smem(syrk_fx_kernel, kSmemY);
     for (int64_t i0 = 0; i0 < n; i0 += rows) {
         const int64_t here = std::min(rows, (n - i0 + group - 1) / group * group);
-        const int64_t thr = here / 8 * ct * 128;
-        syrk_digits_kernel<<<(unsigned)((thr + 255) / 256), 256, 0, st>>>(KXU, n, m, i0, here, ct, mx,
+        const int64_t thr = here / 8 * ct * cw;
+        syrk_digits_kernel<<<(unsigned)((thr + 255) / 256), 256, 0, st>>>(KXU, n, m, i0, here, ct, cw, mx,
                                                                           dig, sq);
         KPCG_LAUNCHED("syrk_digits_kernel");
         const int ngroups = (int)(here / group);
         // every split writes (the first block) or adds to its part, also when it has no rows
         syrk_fx_kernel<<<dim3((unsigned)tiles, (unsigned)nsplit), YWARPS * 32, kSmemY, st>>>(
-            dig, m, (int)ct, ngroups, (ngroups + nsplit - 1) / nsplit, mx,
+            dig, m, (int)ct, cw, ngroups, (ngroups + nsplit - 1) / nsplit, mx,
             i0 + rows >= n ? sq : nullptr, i0 == 0, part, err,
             stall_ns > 0 ? (uint64_t)stall_ns : kWaitNs, stall_ns > 0 ? 1 : 0);
         KPCG_LAUNCHED("syrk_fx_kernel");
     }
+    return err;
 }
 
 }  // namespace kpcg
