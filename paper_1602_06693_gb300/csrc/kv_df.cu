@@ -965,10 +965,14 @@ void kv_f64_sym(Ctx& h, const double* V, int64_t ldv, int c, const double* B, in
         kv_fx(h, V, ldv, c, B, ldb, O, ldo, noise, false);
         return;
     }
-    // otherwise on the FP64 pipe: symmetric tile pairs halve the exps but take at
-    // most two columns per pass; from three columns on, one pass over up to 16
-    // columns of the plain kernel computes each entry's exp fewer times
-    if (!(h.dp <= 16 && h.n >= 4 * ST) || (c >= 3 && h.dp <= 16)) {
+    // otherwise on the FP64 pipe: symmetric tile pairs halve the exps but take at most two
+    // columns per pass, the plain kernel takes up to 16 in one.  Two passes against one:
+    // n = 4000, d = 8, three and four columns 1.20 and 1.25 against 1.25 ms, n = 16000 15.8 and
+    // 16.3 against 18.4 ms, but n = 1500 0.36 and 0.38 against 0.20 ms; five columns lose at
+    // every size (n = 16000 23.9 against 20.2 ms).  Beyond 180 000 rows the symmetric one's
+    // column partials pass 4 GiB
+    const bool two_passes = c > 2 && c <= 4 && h.n > 1900 && h.n <= 180000;
+    if (!(h.dp <= 16 && h.n >= 4 * ST) || (h.dp <= 16 && c > 2 && !two_passes)) {
         kv_f64(h.xs64.p, h.n, h.dp, h.c0_64(), noise, V, ldv, c, B, ldb, O, ldo, h.kvws, h.stream);
         return;
     }

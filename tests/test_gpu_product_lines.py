@@ -1,0 +1,40 @@
+"""The FP64 products on both sides of the sizes where another kernel takes them.
+
+Few rows go to the plain or double-float kernels, more to the fixed-point one; beyond its
+range three and four columns go to the symmetric FP64 kernel from 2000 rows on, the plain
+one takes 5 to 7 columns as eight.  Bounds norm-wise against |K_y| |V|: FP64 products
+2^-46 as in the other sizes, double-float entries are good to 2^-44 of the largest: 2^-43.
+"""
+import numpy as np
+import pytest
+
+import oracle
+import synthetic
+
+pytestmark = pytest.mark.gpu
+
+torch = pytest.importorskip("torch")
+
+
+def _check(n, d, c, impl, ell, tol):
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    import paper_1602_06693_gb300 as kpcg
+    from paper_1602_06693_gb300 import build
+    build.build()
+    p = synthetic.make_problem(n, d, 7, dist="normal", ell=ell, s2=1.7, noise=1e-3)
+    V = synthetic.rng(8).standard_normal((n, c))
+    l, s2 = oracle.split_theta(p.log_theta, p.d, p.ard)
+    ref = oracle.kyv(p.X, l, s2, p.noise, V)
+    big = oracle.kyv(p.X, l, s2, p.noise, np.abs(V))
+    with kpcg.Solver(torch.from_numpy(p.X).cuda(), p.log_theta, p.noise, ard=p.ard) as s:
+        Vd = torch.from_numpy(np.ascontiguousarray(V.T)).cuda().t()
+        O = s.matvec_f64(Vd, impl=impl).cpu().numpy()
+    assert (np.linalg.norm(O - ref, axis=0) <= tol * np.linalg.norm(big, axis=0)).all()
+
+
+@pytest.mark.parametrize("n,d,c", [
+    (300, 4, 3), (300, 4, 5), (2000, 8, 3), (2001, 8, 3), (2001, 8, 4), (2001, 8, 5), (700, 16, 6),
+    (700, 16, 7), (700, 3, 9), (700, 3, 19), (300, 20, 3), (300, 20, 7), (300, 20, 9)])
+def test_beyond_the_fixed_point_range(n, d, c):
+    _check(n, d, c, 0, 0.1, 2.0 ** -46)
