@@ -1137,12 +1137,13 @@ kpcg_status kpcg_matvec_f64(kpcg_t h, const double* V, int64_t ldv, int32_t c, d
         kpcg::check_dev_ptr(V, "V");
         kpcg::check_dev_ptr(O, "O");
         if (impl == 0) {
-            kpcg::kv_f64_sym(*h, V, ldv, c, nullptr, 0, O, ldo, h->noise);
-            if (kpcg::kv_tc_error(*h))
+            // (reading the flag takes 10 us, a third of a call on a few rows)
+            if (kpcg::kv_f64_sym(*h, V, ldv, c, nullptr, 0, O, ldo, h->noise) &&
+                kpcg::kv_tc_error(*h))
                 fail(KPCG_ERR_TIMEOUT, "a bounded wait in the tensor-core K.V expired");
         } else if (impl == 1) {
-            kpcg::kv_df(*h, V, ldv, c, nullptr, 0, O, ldo, h->noise);
-            if (kpcg::kv_tc_error(*h))
+            if (kpcg::kv_df(*h, V, ldv, c, nullptr, 0, O, ldo, h->noise) &&
+                kpcg::kv_tc_error(*h))
                 fail(KPCG_ERR_TIMEOUT, "a bounded wait in the tensor-core K.V expired");
         } else if (impl == 3) {
             // the double-float kernel on the FP32 pipe alone (no tensor-core distances)

@@ -193,14 +193,15 @@ struct Ctx {
 // Tensor-core K.V on the handle's inputs (kv_tc.cu).
 void kv_tc_apply(Ctx& h, const float* V, int64_t ldv, int c, float* O, int64_t ldo, float noise);
 // O = K V + noise V (or B - that when B != nullptr) with the double-float
-// kernel (kv_df.cu); FP64 in and out.
-void kv_df(Ctx& h, const double* V, int64_t ldv, int c, const double* B, int64_t ldb, double* O,
+// kernel (kv_df.cu) or the fixed-point one where that is faster; FP64 in and out.  True
+// if a kernel with bounded waits took it.
+bool kv_df(Ctx& h, const double* V, int64_t ldv, int c, const double* B, int64_t ldb, double* O,
            int64_t ldo, double noise);
 // FP64 product (certified residuals, KPCG_FP64): in fixed point on the tensor cores
 // (kv_fx.cu) where that is FP64-accurate, else native FP64 on symmetric tile
 // pairs (kv_df.cu) or, for small n, d > 16 or three and more columns, the row-split
-// kernel.  Same arguments as kv_df.
-void kv_f64_sym(Ctx& h, const double* V, int64_t ldv, int c, const double* B, int64_t ldb,
+// kernel.  Arguments and result of kv_df.
+bool kv_f64_sym(Ctx& h, const double* V, int64_t ldv, int c, const double* B, int64_t ldb,
                 double* O, int64_t ldo, double noise);
 // O = (K + noise I) V in FP32 with exact pairwise differences of the split
 // inputs and compensated sums (kv_df.cu; d <= 16).  expp 0: MUFU exp2,

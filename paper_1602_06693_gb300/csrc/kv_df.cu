@@ -953,17 +953,22 @@ static void f64_sym_launch(int cb, const double* xs, int64_t n, int nt, double c
         f64_sym_launch1<DP, 2>(xs, n, nt, c0, V, ldv, ncols, work, nwork, G, nchunk, prow, pcol, tab64, st);
 }
 
-void kv_f64_sym(Ctx& h, const double* V, int64_t ldv, int c, const double* B, int64_t ldb,
+bool kv_f64_sym(Ctx& h, const double* V, int64_t ldv, int c, const double* B, int64_t ldb,
                 double* O, int64_t ldo, double noise) {
-    if (h.n <= 0 || c <= 0) return;
+    if (h.n <= 0 || c <= 0) return false;
     // the fixed-point tensor-core product wherever its operands keep FP64 accuracy
     // (|y| <= 8, inputs within 9.4 lengthscales of their mean: the dropped levels stay near
     // 2^-53 of an entry): 12.9 ms against 119.6 ms at n = 65536, d = 8 and 0.07 against
     // 0.18 ms at n = 200, one column.  Beyond that range the step back to the FP64 pipe is
-    // a factor of nine; wider slices would need a seventh level of the distance
-    if (kv_fx_usable(h, c, 8.0)) {
+    // a factor of nine; wider slices would need a seventh level of the distance.
+    // Its five launches lose to the plain kernel's two on very few rows, as calls with
+    // d = 8: n = 1 28 against 53 us, n = 16 one column 60 against 76, sixteen 76 against
+    // 87 (n = 24 102 against 99); half the rows where it needs more passes (17 columns,
+    // n = 8 78 against 86, n = 12 99 against 90)
+    const bool tiny = h.n <= ((c + 15) / 16 <= (c + 23) / 24 ? 16 : 8);
+    if (!tiny && kv_fx_usable(h, c, 8.0)) {
         kv_fx(h, V, ldv, c, B, ldb, O, ldo, noise, false);
-        return;
+        return true;
     }
     // otherwise on the FP64 pipe: symmetric tile pairs halve the exps but take at most two
     // columns per pass, the plain kernel takes up to 16 in one.  Two passes against one:
@@ -974,7 +979,7 @@ void kv_f64_sym(Ctx& h, const double* V, int64_t ldv, int c, const double* B, in
     const bool two_passes = c > 2 && c <= 4 && h.n > 1900 && h.n <= 180000;
     if (!(h.dp <= 16 && h.n >= 4 * ST) || (h.dp <= 16 && c > 2 && !two_passes)) {
         kv_f64(h.xs64.p, h.n, h.dp, h.c0_64(), noise, V, ldv, c, B, ldb, O, ldo, h.kvws, h.stream);
-        return;
+        return false;
     }
     cudaStream_t st = h.stream;
     const int64_t n = h.n;
@@ -1011,35 +1016,52 @@ void kv_f64_sym(Ctx& h, const double* V, int64_t ldv, int c, const double* B, in
         KPCG_LAUNCHED("kv_df_sym_reduce_kernel");
         k0 += cb;
     }
+    return false;
 }
 
-void kv_df(Ctx& h, const double* V, int64_t ldv, int c, const double* B, int64_t ldb, double* O,
+// Whether the fixed-point product beats the double-float kernels, as calls in us
+// (double-float against fixed point):
+//  d <= 10, one or two columns: few row tiles (n = 500 .. 2000, d = 8: 88 .. 92 against 67 .. 82;
+//      2100: 93 against 88) but not one or two (n = 50: 51 against 66, n = 200: 64 against
+//      67); n = 65536, two columns 10.1 against 12.9 ms;
+//  three columns (two passes) from 96 rows on (96: 62 against 66, 128: 74 against 66), four (one
+//      pass) from 256 on (160: 67 against 73, 512: 104 against 70), more from 16 on (n = 8,
+//      five: 60 against 72); n = 65536, d = 8: three 20.9 against 13.9 ms, nine 40.8 against
+//      15.2 ms;
+//  d > 10, whose distances the double-float kernels take from the FP32 pipe: up to four
+//      columns from 512 rows on (n = 500, d = 12, one: 51 against 58, 512: 73 against 62;
+//      n = 16384, d = 14, one 1.63 against 0.94 ms); up to sixteen with d <= 12 from 1536
+//      on (n = 1000, five: 62 against 73, 2000: 90 against 86); others from 32 or 48 on
+//      (d = 14, n = 32, nine: 68 against 126, 48: 84 against 75; five: 55 against 71).
+static bool fx_beats_df(int64_t n, int d, int c) {
+    if (d <= 10) {
+        if (c <= 2) return n > 256 && n <= 2048;
+        return n > (c == 3 ? 96 : c == 4 ? 256 : c <= 8 ? 16 : 0);
+    }
+    return n > (c <= 4 ? 511 : c <= 16 && d <= 12 ? 1536 : c <= 8 ? 48 : 32);
+}
+
+bool kv_df(Ctx& h, const double* V, int64_t ldv, int c, const double* B, int64_t ldb, double* O,
            int64_t ldo, double noise) {
-    if (h.n <= 0 || c <= 0) return;
-    // the fixed-point product (kv_fx.cu; one time for any number of columns) where it is
-    // the faster one: from three columns on (n = 65536, d = 8: 13.9 against
-    // 20.9 ms at three, 15.2 against 40.8 ms at nine; 12.9 against 10.1 ms at two),
-    // for d > 10, whose distances the kernels below take from the FP32 pipe (d = 14,
-    // one column, n = 16384: 0.94 against 1.63 ms), and for few row tiles, as calls
-    // (n = 500 .. 2000, d = 8, one column: 67 .. 82 against 88 .. 92 us; 2100: 88 against
-    // 93) but not for one or two (n = 50: 66 against 51, n = 200: 67 against 64).  Up to
-    // |y| = 64 its dropped levels stay below the 2^-45 of a double-float entry.
-    const bool few_tiles = h.n > 256 && h.n <= 2048;
-    if (h.df_tensor && (c >= 3 || h.d > 10 || few_tiles) && kv_fx_usable(h, c, 64.0)) {
+    if (h.n <= 0 || c <= 0) return false;
+    // the fixed-point product (kv_fx.cu; one time for any number of columns) where it is the
+    // faster one.  Up to |y| = 64 its dropped levels stay below the 2^-45 of a double-float
+    // entry
+    if (h.df_tensor && fx_beats_df(h.n, h.d, c) && kv_fx_usable(h, c, 64.0)) {
         kv_fx(h, V, ldv, c, B, ldb, O, ldo, noise, true);
-        return;
+        return true;
     }
     // the squared distances on the tensor cores where the sliced layout fits
     if (h.df_tensor && kv_tcd_supported(h)) {
         kv_tcd(h, V, ldv, c, B, ldb, O, ldo, noise);
-        return;
+        return true;
     }
     df_prepare(h);
     // The symmetric kernel pays off once there are several tile pairs per SM,
     // and while few columns are in the product.
     if (h.dp <= 16 && h.n >= 4 * ST && h.df_symmetric && !df_prefer_plain(h.n, h.dp, c)) {
         kv_df_sym(h, V, ldv, c, B, ldb, O, ldo, noise);
-        return;
+        return false;
     }
     cudaStream_t st = h.stream;
     const int64_t n = h.n;
@@ -1067,6 +1089,7 @@ void kv_df(Ctx& h, const double* V, int64_t ldv, int c, const double* B, int64_t
         KPCG_LAUNCHED("kv_df_reduce_kernel");
         k0 += ncols;
     }
+    return false;
 }
 
 template <int DP, int CB, int EXPP>

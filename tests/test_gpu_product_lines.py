@@ -33,6 +33,20 @@ def _check(n, d, c, impl, ell, tol):
     assert (np.linalg.norm(O - ref, axis=0) <= tol * np.linalg.norm(big, axis=0)).all()
 
 
+@pytest.mark.parametrize("n", [8, 9, 16, 17])
+@pytest.mark.parametrize("d,c", [(8, 1), (3, 7), (16, 16), (8, 17), (12, 25)])
+def test_fp64_few_rows(n, d, c):
+    _check(n, d, c, 0, 2.0, 2.0 ** -46)
+
+
+@pytest.mark.parametrize("n,d,c", [
+    (96, 8, 3), (97, 8, 3), (256, 8, 4), (257, 8, 4), (16, 8, 5), (17, 8, 8), (511, 12, 1),
+    (512, 14, 4), (1536, 12, 5), (1537, 11, 16), (32, 14, 9), (33, 14, 17), (48, 13, 8),
+    (49, 13, 5)])
+def test_double_float_lines(n, d, c):
+    _check(n, d, c, 1, 2.0, 2.0 ** -43)
+
+
 @pytest.mark.parametrize("n,d,c", [
     (300, 4, 3), (300, 4, 5), (2000, 8, 3), (2001, 8, 3), (2001, 8, 4), (2001, 8, 5), (700, 16, 6),
     (700, 16, 7), (700, 3, 9), (700, 3, 19), (300, 20, 3), (300, 20, 7), (300, 20, 9)])
