@@ -1029,8 +1029,9 @@ bool kv_f64_sym(Ctx& h, const double* V, int64_t ldv, int c, const double* B, in
 //      five: 60 against 72); n = 65536, d = 8: three 20.9 against 13.9 ms, nine 40.8 against
 //      15.2 ms;
 //  d > 10, whose distances the double-float kernels take from the FP32 pipe: up to four
-//      columns from 512 rows on (n = 500, d = 12, one: 51 against 58, 512: 73 against 62;
-//      n = 16384, d = 14, one 1.63 against 0.94 ms); up to sixteen with d <= 12 from 1536
+//      columns from 512 rows on (n = 500, d = 12, one: 51 against 58, 512: 73 against 62),
+//      one and two with d > 12 from 2048 on (1000: 65 against 65, 2000: 67 against 77, 2100: 86
+//      against 82; n = 16384, d = 14, one 1.63 against 0.94 ms); up to sixteen with d <= 12 from 1536
 //      on (n = 1000, five: 62 against 73, 2000: 90 against 86); others from 32 or 48 on
 //      (d = 14, n = 32, nine: 68 against 126, 48: 84 against 75; five: 55 against 71).
 static bool fx_beats_df(int64_t n, int d, int c) {
@@ -1038,6 +1039,7 @@ static bool fx_beats_df(int64_t n, int d, int c) {
         if (c <= 2) return n > 256 && n <= 2048;
         return n > (c == 3 ? 96 : c == 4 ? 256 : c <= 8 ? 16 : 0);
     }
+    if (c <= 2 && d > 12) return n > 2048;
     return n > (c <= 4 ? 511 : c <= 16 && d <= 12 ? 1536 : c <= 8 ? 48 : 32);
 }
 

@@ -42,7 +42,7 @@ def test_fp64_few_rows(n, d, c):
 @pytest.mark.parametrize("n,d,c", [
     (96, 8, 3), (97, 8, 3), (256, 8, 4), (257, 8, 4), (16, 8, 5), (17, 8, 8), (511, 12, 1),
     (512, 14, 4), (1536, 12, 5), (1537, 11, 16), (32, 14, 9), (33, 14, 17), (48, 13, 8),
-    (49, 13, 5)])
+    (49, 13, 5), (2048, 16, 2), (2049, 13, 1)])
 def test_double_float_lines(n, d, c):
     _check(n, d, c, 1, 2.0, 2.0 ** -43)
 
