@@ -1251,7 +1251,7 @@ def run_kv(args):
     ms /= args.steps
     rates = probed_rates(kpcg)
     rates["bf16_tflops"] = float(measured_peaks().get("bf16_tflops", 1934.6))
-    if args.kv_impl == "df" and (c > 2 or p.n <= 2048):
+    if args.kv_impl == "df" and (c > 2 or 256 < p.n <= 2048):
         kname = FX_NAME  # the double-float entry takes it there
     roof = alu_roofline(kname, p.n, p.d, c, ms, rates)
     roof.update({"peak_source": PEAK_SOURCE, "traffic": known_traffic(kname, p.n),

@@ -237,12 +237,14 @@ kpcg_status kpcg_precond_pitc(kpcg_t h, int64_t m, const int64_t* idx, int64_t b
  * entries good to 2^-54 of their size and to 2^-63 s^2, digits of V to 2^-63 of
  * its column's largest value, sums without rounding: an error against the
  * largest entry and value, where FP64 errs against each entry's; columns of at
- * most 32 values, as unit vectors, are summed from FP64 entries), else entries
- * and sums in native FP64;
+ * most 32 values, as unit vectors, are summed from FP64 entries), else, and for
+ * the fewest rows, entries and sums in native FP64 (beyond |x'| ~ 8 that takes about
+ * nine times as long for one column, n = 65536: 119.7 against 12.9 ms);
  * impl 1: the double-float product of KPCG_DF64 and of the outer loop of the
  * mixed modes (FP32-pair arithmetic, about 44 bits per entry, sums carried as
  * FP32 pairs and added in FP64), or the fixed-point product where that is the
- * faster one (three and more columns, d > 10, few rows); in double-float for
+ * faster one (one or two columns of 257 to 2048 rows; three and more columns, or d > 10,
+ * from a few tens to 2049 rows on); in double-float for
  * d <= 10 the squared distances come from exact integer level sums of 8-bit
  * slices of x' on the tensor cores, each pair of points evaluated once for
  * both triangles of K (n > 128), for larger d from exact grid differences on

@@ -45,12 +45,12 @@
 // (products of its constant digits with unsigned bytes in the dropped levels), with these by
 // 7e-16; FP64 sums by 1e-15 to 3e-15.
 //
-// What bounds it: issue of the epilogue, 82 instructions per entry with one
-// column (ncu at n = 16384: issue 74%, the FP32 and ALU pipes 42% each, DRAM the operands once),
+// What bounds it: issue of the epilogue, 84 instructions per entry with one
+// column (ncu at n = 16384: issue 73%, the ALU pipe 43%, FP32 39%, DRAM the operands once),
 // nearly independent of the number of columns, where the FP64 kernel needs 28 + 2 c FP64
 // operations per pair of points (two per clock and SM) and the double-float one 67 + 25 c
-// FP32 instructions.  n = 65536, d = 8: 13.0 ms with one column (FP64: 119.6 ms; 12.1 ms with
-// seven unsigned bytes); n = 45730, d = 9, 17 columns: 8.8 ms (double-float: 36.1 ms).
+// FP32 instructions.  n = 65536, d = 8: 12.9 ms with one column (FP64: 119.6 ms; 12.1 ms with
+// seven unsigned bytes); n = 45730, d = 9, 17 columns: 8.7 ms (double-float: 36.1 ms).
 // Errors against extended precision on random, constant and smooth vectors: 1e-16 to
 // 5e-16 of the result.
 //

@@ -1,4 +1,4 @@
-// Shared pieces of the tcgen05 kernels (kv_tc.cu, kv_tcv.cu): tile shape,
+// Shared pieces of the tcgen05 kernels (the kv_tc*.cu files, kv_fx.cu, syrk_fx.cu): tile shape,
 // mbarrier / bulk-copy / tcgen05 wrappers in inline PTX, the 128-byte swizzle
 // of the K-major operand layout.  Every wait is bounded by %globaltimer.
 #pragma once
